@@ -221,6 +221,8 @@ HELM_API helm_status helm_plan_tiles(const helm_plan* plan, int* policy);
  * launch is a critical path: a plan's own solve, or, in a batch step, the lane with the
  * longest predicted solve when it holds that solve alone; the other lanes keep its own
  * launch.
+ * Solves of n = 31 or 63 run all their outer steps in one launch of a small cluster each,
+ * unless HELM_COARSE_CTA asks for the one-CTA tail and its separate launches (the same bits).
  * The results agree to the inner precision's rounding.  helm_plan_coarse_mode reports the
  * policy and, if cluster_used is not NULL, whether the plan's last built outer step used the
  * cluster (0 before its first solve).  helm_batch_set_coarse_mode applies a policy to every

@@ -163,7 +163,7 @@ struct PlanState {
     size_t mg_cap = 0;
     ResItem* d_res = nullptr;
     size_t res_cap = 0;
-    int nres = 0, max_tail = 1, damp_any = 0;
+    int nres = 0, max_tail = 1, damp_any = 0, small_cs = 0, l0_off = 0, l0_cnt = 0;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     cudaGraphConditionalHandle cond = 0;
@@ -201,12 +201,14 @@ struct Engine {
     // forms level 1's ascent inside the fused finest kernel (as HELM_COARSE_CLUSTER does),
     // trading throughput it does not need for latency.
     bool latency = false;
+    // solves of other classes or sizes run beside this engine's in the batch's steps
+    bool mixed_sizes = false;
     cudaStream_t cap_stream = nullptr;
     int cap = 0;                               // descriptor slots
     std::vector<Instance*> slots;              // nullptr = free
     InstDesc* d_desc = nullptr;
     InstState* d_state = nullptr;
-    int* d_ctrl = nullptr;                     // [0] steps done, [1] step budget, [2] go, [3] arrivals
+    int* d_ctrl = nullptr;                     // [0] steps done, [1] step budget, [2] go, [3] arrivals, [4] launch's steps
     int* h_ctrl = nullptr;                     // pinned mirror
     InstState* h_state = nullptr;              // pinned mirror (cap entries)
     // page-locked staging of a starting instance's descriptor and state (a copy from
@@ -233,6 +235,9 @@ struct Engine {
     std::vector<LaunchRec> vcyc_plain;         // one V-cycle from the current iterate
     int max_tail = 1;
     int damp_any = 0;                          // some slot's instance has p != 0
+    // 2D complex64 solves of one small size run all their steps in one launch of a cluster
+    // of small_cs CTAs each (small2d.cu; 0: launch by launch), from their level-0 items
+    int small_cs = 0, l0_off = 0, l0_cnt = 0;
     bool dirty = true;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
@@ -257,6 +262,9 @@ struct Engine {
         std::swap(nres, p.nres);
         std::swap(max_tail, p.max_tail);
         std::swap(damp_any, p.damp_any);
+        std::swap(small_cs, p.small_cs);
+        std::swap(l0_off, p.l0_off);
+        std::swap(l0_cnt, p.l0_cnt);
         std::swap(graph, p.graph);
         std::swap(exec, p.exec);
         std::swap(cond, p.cond);
@@ -297,11 +305,15 @@ struct Engine {
         D = D_;
         prec = prec_;
         HELM_CK(cudaStreamCreateWithFlags(&cap_stream, cudaStreamNonBlocking));
-        HELM_CK(cudaMalloc(&d_ctrl, 4 * sizeof(int)));
+        HELM_CK(cudaMalloc(&d_ctrl, 8 * sizeof(int)));
+        HELM_CK(cudaMemset(d_ctrl, 0, 8 * sizeof(int)));
         HELM_CK(cudaMallocHost(&h_ctrl, 4 * sizeof(int)));
         HELM_CK(setup_tail(D, prec == HELM_PREC_FP64 ? 0 : 1));
         if (D == 2) HELM_CK(setup_2d(prec == HELM_PREC_FP64 ? 0 : 1));
-        if (D == 2 && prec != HELM_PREC_FP64) ctail_setup();
+        if (D == 2 && prec != HELM_PREC_FP64) {
+            ctail_setup();
+            HELM_CK(setup_small2d());
+        }
         HELM_CK(setup_generic(D, prec == HELM_PREC_FP64 ? 0 : 1));
         HELM_CK(setup_outer());
         return grow(4);
@@ -425,15 +437,19 @@ struct Engine {
                 b_res += pts(d.n) * (16.0 + eb + 16.0 + 16.0 + eb);
             }
         // level-0 items (zeroing when nu1 == 0)
-        const int l0_off = (int)items.size();
-        int nl0 = 0, w_l0 = 0;
+        l0_off = (int)items.size();
+        int nl0 = 0, w_l0 = 0, n_l0 = -1;
         for (int i = 0; i < cap; ++i)
             if (slots[i]) {
                 items.push_back(MgItem{i, 0});
                 ++nl0;
+                n_l0 = (n_l0 == -1 || n_l0 == slots[i]->d.n) ? slots[i]->d.n : -2;   // -2: several sizes
                 const LevelDesc& L = slots[i]->d.lev[0];
                 w_l0 = std::max(w_l0, L.pitch * L.rows * ((D == 3) ? L.rows : 1));
             }
+        l0_cnt = nl0;
+        small_cs = (D == 2 && prec != HELM_PREC_FP64 && n_l0 > 0 && coarse != HELM_COARSE_CTA)
+                       ? small2d_fits(n_l0, nl0, mixed_sizes) : 0;
         for (int i = 0; i < cap; ++i) {
             if (!slots[i]) continue;
             const InstDesc& d = slots[i]->d;
@@ -696,6 +712,21 @@ struct Engine {
         return HELM_OK;
     }
 
+    // One outer step of every instance; of small solves, all their remaining steps up to the
+    // budget.
+    helm_status enqueue_step(cudaStream_t s)
+    {
+        if (!small_cs) return enqueue(step, s, false);
+        int n = 0;
+        for (auto* p : slots)
+            if (p) n = p->d.n;
+        HELM_CK(launch_small2d(d_desc, d_state, d_mg + l0_off, l0_cnt, n, small_cs, nu1, nu2, cycles, damp_any,
+                               d_ctrl, s));
+        return HELM_OK;
+    }
+    // kernels launched by a run that made `steps` steps
+    uint64_t step_launches(int steps) const { return small_cs ? (steps > 0) : (uint64_t)steps * step.size(); }
+
     // (Re)build the graph: a single WHILE node whose body is one outer step.
     helm_status build_graph()
     {
@@ -725,7 +756,7 @@ struct Engine {
     // whether any instance has a damping term (it selects the residual kernels' variant).
     std::vector<long> current_signature() const
     {
-        std::vector<long> sig{cap, nu1, nu2, cycles, tiles, coarse, latency ? 1L : 0L};
+        std::vector<long> sig{cap, nu1, nu2, cycles, tiles, coarse, (latency ? 1L : 0L) + (mixed_sizes ? 2L : 0L)};
         long damp = 0;
         for (int i = 0; i < cap; ++i) {
             sig.push_back(slots[i] ? (long)slots[i]->d.n * 4 + (long)slots[i]->d.D : -1L);
@@ -777,7 +808,7 @@ struct Engine {
     {
         helm_status st = prepare_plan();
         if (st != HELM_OK) return st;
-        if (graph_current()) return HELM_OK;
+        if (small_cs || graph_current()) return HELM_OK;     // small solves: one plain launch
         st = build_graph();
         if (st != HELM_OK) return st;
         graph_sig = plan_sig;
@@ -921,12 +952,17 @@ struct Engine {
         h_ctrl[2] = 1;
         h_ctrl[3] = 0;
         HELM_CK(cudaMemcpyAsync(d_ctrl, h_ctrl, 4 * sizeof(int), cudaMemcpyHostToDevice, s));
-        HELM_CK(cudaGraphLaunch(exec, s));
+        if (small_cs) {
+            st = enqueue_step(s);
+            if (st != HELM_OK) return st;
+        } else {
+            HELM_CK(cudaGraphLaunch(exec, s));
+        }
         HELM_CK(cudaMemcpyAsync(h_ctrl, d_ctrl, 3 * sizeof(int), cudaMemcpyDeviceToHost, s));
         HELM_CK(cudaMemcpyAsync(h_state, d_state, sizeof(InstState) * cap, cudaMemcpyDeviceToHost, s));
         HELM_CK(cudaStreamSynchronize(s));
         if (steps_done) *steps_done = h_ctrl[0];
-        g_launches += (uint64_t)h_ctrl[0] * step.size();
+        g_launches += step_launches(h_ctrl[0]);
         return HELM_OK;
     }
 };
@@ -2021,9 +2057,12 @@ static std::vector<int> rank_engines(helm_batch* b)
     std::stable_sort(order.begin(), order.end(),
                      [](const std::pair<double, int>& x, const std::pair<double, int>& y) { return x.first > y.first; });
     std::vector<int> keys;
+    bool mixed = false;                          // engines of several classes or sizes
+    for (const auto& o : order) mixed = mixed || o.second / HELM_MAX_LANES != order[0].second / HELM_MAX_LANES;
     for (size_t r = 0; r < order.size(); ++r) {
         Engine* E = b->engines[order[r].second].get();
         E->latency = r == 0 && E->active_count() == 1;
+        E->mixed_sizes = mixed;
         keys.push_back(order[r].second);
     }
     return keys;
@@ -2058,7 +2097,7 @@ helm_status helm_batch_step(helm_batch* b, int max_steps)
         // A bounded chunk after a membership change runs as direct launches (finished
         // instances' kernels exit at once); the graph is (re)captured only for runs to
         // completion, so a serving loop that admits between chunks never waits on a capture.
-        const bool direct = max_steps > 0 && max_steps <= 64 && !E->graph_current();
+        const bool direct = E->small_cs || (max_steps > 0 && max_steps <= 64 && !E->graph_current());
         if (!direct) {
             st = E->prepare();
             if (st != HELM_OK) return st;
@@ -2069,8 +2108,8 @@ helm_status helm_batch_step(helm_batch* b, int max_steps)
         E->h_ctrl[3] = 0;
         HELM_CK(cudaMemcpyAsync(E->d_ctrl, E->h_ctrl, 4 * sizeof(int), cudaMemcpyHostToDevice, es));
         if (direct) {
-            for (int k = 0; k < max_steps; ++k) {
-                st = E->enqueue(E->step, es, false);
+            for (int k = 0; k < (E->small_cs ? 1 : max_steps); ++k) {
+                st = E->enqueue_step(es);
                 if (st != HELM_OK) return st;
             }
         } else {
@@ -2101,7 +2140,7 @@ helm_status helm_batch_step(helm_batch* b, int max_steps)
     HELM_CK(cudaStreamSynchronize(b->stream));
     for (int key : launched) {
         Engine* E = b->engines[key].get();
-        g_launches += (uint64_t)E->h_ctrl[0] * E->step.size();
+        g_launches += E->step_launches(E->h_ctrl[0]);
     }
     return retire_finished(b);
 }

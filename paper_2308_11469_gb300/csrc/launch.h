@@ -57,6 +57,8 @@ cudaError_t launch_tail(int D, int prec, int n0, const InstDesc* insts, const In
 size_t tail_smem_bytes(int D, int prec, int n);
 // size of the level the tail solves exactly instead of cycling (0: none); prec 0 = FP64
 int tail_exact_n(int D, int prec);
+// device address of the 2D complex64 exact level's table (after setup_tail)
+const float* tail_table_2d();
 // raise the tail kernel's dynamic shared-memory limit (once, before any capture)
 cudaError_t setup_tail(int D, int prec);
 // cluster tail (2D complex64, cycles without pre-smoothing, level 255 below the top): one
@@ -66,6 +68,16 @@ cudaError_t setup_tail(int D, int prec);
 int ctail_setup();
 cudaError_t launch_ctail(const InstDesc* insts, const InstState* st, const MgItem* items, int nitems,
                          int nu2, cudaStream_t s);
+// whole solves of small 2D complex64 grids (small2d.cu): every remaining outer step of the
+// items (level-0 items of instances of size n), up to the budget ctrl[1] - ctrl[0], in one
+// launch of a cluster of cs CTAs per item.  Adds the steps made to ctrl[0]; ctrl holds 5
+// ints, [3] and [4] zero between launches.  small2d_fits: the cluster size for ninst
+// instances of size n (0: no such kernel, or too many for it); mixed: solves of other sizes
+// run beside them.
+int small2d_fits(int n, int ninst, bool mixed);
+cudaError_t setup_small2d();
+cudaError_t launch_small2d(const InstDesc* insts, InstState* st, const MgItem* items, int nitems, int n, int cs,
+                           int nu1, int nu2, int cycles, int damp, int* ctrl, cudaStream_t s);
 // shared-memory carve-out preferences of the generic and outer kernels
 cudaError_t setup_generic(int D, int prec);
 cudaError_t setup_outer();
