@@ -40,8 +40,6 @@ constexpr int AN_NT = 256;
 constexpr int AN_NC = 8;            // coarsest level (solved exactly)
 constexpr int AN_BAND = 4;          // band half-width around the hole, in nodes of the level
 constexpr int AN_BAND_SWEEPS = 4;
-constexpr bool AN_BAND_SMEM = true;  // band sweeps in shared memory where the ring fits
-constexpr bool AN_TILES = true;      // each side's sweeps of a level in one tile launch
 constexpr bool AN_GRAPHS = true;     // an outer step replayed as one graph launch
 constexpr size_t AN_SMEM_MAX = 227 * 1024;
 enum : unsigned char { AN_PDE = 0, AN_EDGE = 1, AN_HOLE = 2 };
@@ -71,660 +69,441 @@ __device__ __forceinline__ T inward_mean(const T* e, int i, int j, int n)
     return s;
 }
 
-// sum of the non-hole neighbours of a PDE node (hole entries of an iterate are zero)
-template <typename T>
-__device__ __forceinline__ T nbr_sum(const T* e, int q, int S)
-{
-    T a = e[q - S], b = e[q + S], c = e[q - 1], d = e[q + 1];
-    T s;
-    s.x = (a.x + b.x) + (c.x + d.x);
-    s.y = (a.y + b.y) + (c.y + d.y);
-    return s;
-}
+// FP64 <-> inner precision; complex64's format changes run on the integer pipes
+__device__ __forceinline__ double an_widen(float x) { return f2d_bits(x); }
+__device__ __forceinline__ double an_widen(double x) { return x; }
+__device__ __forceinline__ float an_narrow(double x, float) { return d2f_bits(x); }
+__device__ __forceinline__ double an_narrow(double x, double) { return x; }
 
-// Red-black Gauss-Seidel over the box [i0, i1] x [j0, j1] for nodes of colour (i + j) & 1;
-// PDE rows e = (sum of neighbours - h^2 rhs) / (4 + sigma h^2), EDGE rows e = mean of the
-// inward neighbours + h rhs.  pde_only: the band sweeps near the hole.
-template <typename R>
-__global__ void __launch_bounds__(AN_NT)
-k_an_rbgs(typename CX<R>::T* __restrict__ e, const typename CX<R>::T* __restrict__ rhs,
-          const unsigned char* __restrict__ typ, int n, R h, R dinv, int color, int i0, int i1, int j0,
-          int j1)
-{
-    typedef typename CX<R>::T c2;
-    const int S = n + 1;
-    const int half = (j1 - j0 + 2) / 2;
-    const long total = (long)(i1 - i0 + 1) * half;
-    const R h2 = h * h;
-    for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < total; t += (long)gridDim.x * blockDim.x) {
-        const int i = i0 + (int)(t / half);
-        const int j = j0 + (((i + j0) & 1) ^ color) + 2 * (int)(t % half);
-        if (j > j1) continue;
-        const int q = i * S + j;
-        const unsigned char ty = typ[q];
-        if (ty == AN_PDE) {
-            const c2 s = nbr_sum(e, q, S);
-            const c2 r = rhs[q];
-            c2 v;
-            v.x = (s.x - h2 * r.x) * dinv;
-            v.y = (s.y - h2 * r.y) * dinv;
-            e[q] = v;
-        } else if (ty == AN_EDGE) {
-            const c2 m = inward_mean(e, i, j, n);
-            const c2 r = rhs[q];
-            c2 v;
-            v.x = m.x + h * r.x;
-            v.y = m.y + h * r.y;
-            e[q] = v;
-        }
-    }
-}
+// ---------------------------------------------------------------------------
+// A level's side of the cycle in one launch, on windows in shared memory
+// ---------------------------------------------------------------------------
+// Windows are held as two colour planes (node (lx, ly) of the window, whose colour is
+// (gx + gy) & 1, at ly * W / 2 + (lx >> 1) of its colour's plane; W even): a half-sweep
+// reads and writes contiguous words.  Their nodes are numbered row by row over all the
+// CTA's threads, and row types follow from the indices (the hole is an index box), so no
+// type array is read.  Half-sweep k updates the nodes that lie k + 1 inside the window, so
+// that every updated node sees the values of a full-grid sweep.
+// A tile is T x T fine nodes (T / 2 coarse ones a side in the descent): 32, or 16 on the
+// levels that 32 would cut into fewer tiles than there are SMs (an_tile).
+constexpr int AN_TT = 512;           // threads of a tile CTA
 
-// One CTA: `sweeps` red-black sweeps over the PDE nodes of the ring [b0, b1]^2 minus the
-// hole's index box [lo, hi]^2, through L2 (loads bypass L1 so that each half-sweep sees the
-// CTA's previous writes).
-template <typename R>
-__global__ void __launch_bounds__(1024)
-k_an_band(typename CX<R>::T* e, const typename CX<R>::T* __restrict__ rhs, const unsigned char* __restrict__ typ,
-          int n, R h, R dinv, int b0, int b1, int lo, int hi, int sweeps)
-{
-    typedef typename CX<R>::T c2;
-    const int S = n + 1;
-    const int w = b1 - b0 + 1, th = lo - b0, bh = b1 - hi, hh = hi - lo + 1;
-    const int nA = th * w, nB = bh * w, nC = hh * th, nD = hh * bh;
-    const int total = nA + nB + nC + nD;
-    const R h2 = h * h;
-    for (int s = 0; s < 2 * sweeps; ++s) {
-        const int color = s & 1;
-        for (int t = threadIdx.x; t < total; t += blockDim.x) {
-            int i, j;
-            if (t < nA) { i = b0 + t / w; j = b0 + t % w; }
-            else if (t < nA + nB) { const int u = t - nA; i = hi + 1 + u / w; j = b0 + u % w; }
-            else if (t < nA + nB + nC) { const int u = t - nA - nB; i = lo + u / th; j = b0 + u % th; }
-            else { const int u = t - nA - nB - nC; i = lo + u / bh; j = hi + 1 + u % bh; }
-            if (((i + j) & 1) != color) continue;
-            const int q = i * S + j;
-            if (typ[q] != AN_PDE) continue;
-            const c2 a = __ldcg(e + q - S), b = __ldcg(e + q + S), c = __ldcg(e + q - 1), d = __ldcg(e + q + 1);
-            const c2 r = rhs[q];
-            c2 v;
-            v.x = (((a.x + b.x) + (c.x + d.x)) - h2 * r.x) * dinv;
-            v.y = (((a.y + b.y) + (c.y + d.y)) - h2 * r.y) * dinv;
-            __stcg(e + q, v);
-        }
-        __syncthreads();
-    }
-}
-
-// The same sweeps with the ring and a 1-node halo around it staged in shared memory: the
-// ring's four strips (rows b0 - 1 .. lo - 1 and hi + 1 .. b1 + 1 across the band's width
-// plus halo; columns b0 - 1 .. lo - 1 and hi + 1 .. b1 + 1 over the hole's rows); nodes
-// of the hole's box read as zero, as they hold in the iterate.  The ring's rhs is staged
-// by ring index.
-struct AnRing {
-    int b0, b1, lo, hi;
-    int w, th, bh, hh, W2, sA, sB, sC, sD, nA, nB, nC, nD;
-    __host__ __device__ AnRing(int b0_, int b1_, int lo_, int hi_) : b0(b0_), b1(b1_), lo(lo_), hi(hi_)
-    {
-        w = b1 - b0 + 1;
-        th = lo - b0;
-        bh = b1 - hi;
-        hh = hi - lo + 1;
-        W2 = w + 2;
-        sA = (th + 1) * W2;
-        sB = (bh + 1) * W2;
-        sC = hh * (th + 1);
-        sD = hh * (bh + 1);
-        nA = th * w;
-        nB = bh * w;
-        nC = hh * th;
-        nD = hh * bh;
-    }
-    __host__ __device__ int stored() const { return sA + sB + sC + sD; }
-    __host__ __device__ int total() const { return nA + nB + nC + nD; }
-    // shared-memory slot of node (i, j) of the window, -1 inside the hole's box
-    __device__ int slot(int i, int j) const
-    {
-        if (i < lo) return (i - (b0 - 1)) * W2 + (j - (b0 - 1));
-        if (i > hi) return sA + (i - (hi + 1)) * W2 + (j - (b0 - 1));
-        if (j < lo) return sA + sB + (i - lo) * (th + 1) + (j - (b0 - 1));
-        if (j > hi) return sA + sB + sC + (i - lo) * (bh + 1) + (j - (hi + 1));
-        return -1;
-    }
-    // node of window slot u
-    __device__ void window_node(int u, int& i, int& j) const
-    {
-        if (u < sA) { i = b0 - 1 + u / W2; j = b0 - 1 + u % W2; return; }
-        u -= sA;
-        if (u < sB) { i = hi + 1 + u / W2; j = b0 - 1 + u % W2; return; }
-        u -= sB;
-        if (u < sC) { i = lo + u / (th + 1); j = b0 - 1 + u % (th + 1); return; }
-        u -= sC;
-        i = lo + u / (bh + 1);
-        j = hi + 1 + u % (bh + 1);
-    }
-    // node of ring index t (the order of k_an_band)
-    __device__ void ring_node(int t, int& i, int& j) const
-    {
-        if (t < nA) { i = b0 + t / w; j = b0 + t % w; return; }
-        t -= nA;
-        if (t < nB) { i = hi + 1 + t / w; j = b0 + t % w; return; }
-        t -= nB;
-        if (t < nC) { i = lo + t / th; j = b0 + t % th; return; }
-        t -= nC;
-        i = lo + t / bh;
-        j = hi + 1 + t % bh;
-    }
+// index boxes of a level: the hole [lo, hi]^2 and the band ring [b0, b1]^2 around it
+struct AnGeo {
+    int n, lo, hi, b0, b1;
+    __device__ bool hole(int i, int j) const { return i >= lo && i <= hi && j >= lo && j <= hi; }
+    __device__ bool edge(int i, int j) const { return i == 0 || i == n || j == 0 || j == n; }
 };
 
-template <typename R>
-size_t an_band_bytes(const AnRing& g)
-{
-    const size_t c = sizeof(typename CX<R>::T);
-    return (size_t)g.stored() * c + (size_t)g.total() * c;
-}
+// q / d for 0 <= q < 65536, 1 <= d <= 4096 by m = ceil(2^32 / d)
+__device__ __forceinline__ unsigned an_magic(int d) { return 0xffffffffu / (unsigned)d + 1u; }
+__device__ __forceinline__ int an_div(int q, int d, unsigned m) { return d == 1 ? q : (int)__umulhi((unsigned)q, m); }
 
-// Each thread owns ring indices threadIdx.x + 1024 k (k < AN_BAND_PT) and keeps, for each,
-// the shared-memory slots of the node and of its four neighbours (-1: the hole's box),
-// found once; a half-sweep is then shared-memory loads and the update alone.
-constexpr int AN_BAND_PT = 5;
-
-template <typename R>
-__global__ void __launch_bounds__(1024)
-k_an_band_s(typename CX<R>::T* __restrict__ e, const typename CX<R>::T* __restrict__ rhs,
-            const unsigned char* __restrict__ typ, int n, R h, R dinv, AnRing g, int sweeps)
-{
+// a window: origin (y0, x0), even row length W, colour planes of the iterate and the rhs
+template <typename R> struct AnWin {
     typedef typename CX<R>::T c2;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int S = n + 1;
-    const int stored = g.stored(), total = g.total();
-    c2* Es = reinterpret_cast<c2*>(smem_raw);
-    c2* Rs = Es + stored;
-    for (int u = threadIdx.x; u < stored; u += blockDim.x) {
-        int i, j;
-        g.window_node(u, i, j);
-        Es[u] = e[i * S + j];
-    }
-    int self[AN_BAND_PT], nb[AN_BAND_PT][4];
-    unsigned colour = 0;                          // bit k: the owned node's colour
-#pragma unroll
-    for (int k = 0; k < AN_BAND_PT; ++k) {
-        const int t = threadIdx.x + 1024 * k;
-        self[k] = -1;
-        nb[k][0] = nb[k][1] = nb[k][2] = nb[k][3] = -1;
-        if (t < total) {
-            int i, j;
-            g.ring_node(t, i, j);
-            Rs[t] = rhs[i * S + j];
-            if (typ[i * S + j] == AN_PDE) {
-                self[k] = g.slot(i, j);
-                nb[k][0] = g.slot(i - 1, j);
-                nb[k][1] = g.slot(i + 1, j);
-                nb[k][2] = g.slot(i, j - 1);
-                nb[k][3] = g.slot(i, j + 1);
-                colour |= (unsigned)((i + j) & 1) << k;
-            }
-        }
-    }
-    __syncthreads();
-    const R h2 = h * h;
-    c2 z;
-    z.x = 0;
-    z.y = 0;
-    for (int s = 0; s < 2 * sweeps; ++s) {
-        const unsigned color = s & 1;
-#pragma unroll
-        for (int k = 0; k < AN_BAND_PT; ++k) {
-            if (self[k] < 0 || ((colour >> k) & 1u) != color) continue;
-            const c2 a = nb[k][0] < 0 ? z : Es[nb[k][0]], b = nb[k][1] < 0 ? z : Es[nb[k][1]];
-            const c2 c = nb[k][2] < 0 ? z : Es[nb[k][2]], d = nb[k][3] < 0 ? z : Es[nb[k][3]];
-            const c2 r = Rs[threadIdx.x + 1024 * k];
-            c2 v;
-            v.x = (((a.x + b.x) + (c.x + d.x)) - h2 * r.x) * dinv;
-            v.y = (((a.y + b.y) + (c.y + d.y)) - h2 * r.y) * dinv;
-            Es[self[k]] = v;
-        }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int k = 0; k < AN_BAND_PT; ++k) {
-        const int t = threadIdx.x + 1024 * k;
-        if (self[k] < 0) continue;
-        int i, j;
-        g.ring_node(t, i, j);
-        e[i * S + j] = Es[self[k]];
-    }
-}
+    int y0, x0, W;
+    c2 *E0, *E1, *R0, *R1;
+    __device__ int at(int i, int j) const { return (i - y0) * (W >> 1) + ((j - x0) >> 1); }
+    __device__ c2* E(int color) const { return color ? E1 : E0; }
+    __device__ c2* Rh(int color) const { return color ? R1 : R0; }
+    __device__ c2 e(int i, int j) const { return E((i + j) & 1)[at(i, j)]; }
+};
 
-// residual of the level's row at a fine node (zero on the hole)
+// mean of the inward neighbours of edge node (i, j), held in the plane Eo
 template <typename R>
-__device__ __forceinline__ typename CX<R>::T an_resid(const typename CX<R>::T* e, const typename CX<R>::T* rhs,
-                                                      const unsigned char* typ, int i, int j, int n, R h, R sig,
-                                                      bool zero)
+__device__ __forceinline__ typename CX<R>::T inward_mean_w(const AnWin<R>& w, const typename CX<R>::T* Eo, int i,
+                                                           int j, int n)
 {
-    typedef typename CX<R>::T c2;
-    const int S = n + 1, q = i * S + j;
-    const unsigned char ty = typ[q];
-    c2 r = rhs[q];
-    if (ty == AN_HOLE) { r.x = 0; r.y = 0; return r; }
-    if (zero) return r;
-    const c2 c = e[q];
-    if (ty == AN_PDE) {
-        const c2 s = nbr_sum(e, q, S);
-        const R ih2 = (R)1 / (h * h);
-        r.x -= (s.x - (R)4 * c.x) * ih2 - sig * c.x;
-        r.y -= (s.y - (R)4 * c.y) * ih2 - sig * c.y;
-    } else {
-        const c2 m = inward_mean(e, i, j, n);
-        r.x -= (c.x - m.x) / h;
-        r.y -= (c.y - m.y) / h;
-    }
-    return r;
-}
-
-// ---------------------------------------------------------------------------
-// Tile kernels: a level's sweeps (and its residual + restriction) on a window in shared
-// memory, so that the sweeps of one side of the cycle are one launch
-// ---------------------------------------------------------------------------
-// A window [sy0, sy1] x [sx0, sx1] of the level (clipped to [0, n]) is staged with row
-// stride SW.  Half-sweep k updates the nodes of its colour that lie k + 1 nodes inside
-// every window side that is not a side of the grid, so that each updated node sees the
-// values the per-level kernels would give it; after 2 nu half-sweeps the values are those
-// of the per-level sweeps on the window shrunk by 2 nu (grid sides excepted).
-constexpr int AN_CT = 16;            // coarse nodes per side of a descent tile
-constexpr int AN_FT = 32;            // fine nodes per side of an ascent tile
-
-// mean of the inward neighbours of edge node (i, j) at window index q
-template <typename T>
-__device__ __forceinline__ T inward_mean_w(const T* e, int q, int SW, int i, int j, int n)
-{
-    T s;
+    typename CX<R>::T s;
     s.x = 0;
     s.y = 0;
     int c = 0;
-    if (i == 0) { s.x += e[q + SW].x; s.y += e[q + SW].y; ++c; }
-    if (i == n) { s.x += e[q - SW].x; s.y += e[q - SW].y; ++c; }
-    if (j == 0) { s.x += e[q + 1].x; s.y += e[q + 1].y; ++c; }
-    if (j == n) { s.x += e[q - 1].x; s.y += e[q - 1].y; ++c; }
+    if (i == 0) { const auto v = Eo[w.at(1, j)]; s.x += v.x; s.y += v.y; ++c; }
+    if (i == n) { const auto v = Eo[w.at(n - 1, j)]; s.x += v.x; s.y += v.y; ++c; }
+    if (j == 0) { const auto v = Eo[w.at(i, 1)]; s.x += v.x; s.y += v.y; ++c; }
+    if (j == n) { const auto v = Eo[w.at(i, n - 1)]; s.x += v.x; s.y += v.y; ++c; }
     if (c == 2) { s.x *= 0.5f; s.y *= 0.5f; }
     return s;
 }
 
-template <typename R>
-__device__ __forceinline__ typename CX<R>::T an_resid_w(const typename CX<R>::T* e, const typename CX<R>::T* rhs,
-                                                        const unsigned char* typ, int q, int SW, int i, int j,
-                                                        int n, R h, R sig, bool zero)
+// One red-black half-sweep over rows ya..yb, columns xa..xb (inside the grid): PDE rows
+// e = (sum of neighbours - h^2 rhs) / (4 + sigma h^2), EDGE rows the mean of the inward
+// neighbours plus h rhs, hole nodes left alone.  PURE: PDE nodes only.
+template <typename R, bool PURE>
+__device__ __forceinline__ void an_half_w(const AnWin<R>& w, const AnGeo& g, int ya, int yb, int xa, int xb, R h,
+                                          R dinv, int color)
 {
     typedef typename CX<R>::T c2;
-    const unsigned char ty = typ[q];
-    c2 r = rhs[q];
-    if (ty == AN_HOLE) { r.x = 0; r.y = 0; return r; }
-    if (zero) return r;
-    const c2 c = e[q];
-    if (ty == AN_PDE) {
-        const c2 s = nbr_sum(e, q, SW);
-        const R ih2 = (R)1 / (h * h);
-        r.x -= (s.x - (R)4 * c.x) * ih2 - sig * c.x;
-        r.y -= (s.y - (R)4 * c.y) * ih2 - sig * c.y;
-    } else {
-        const c2 m = inward_mean_w(e, q, SW, i, j, n);
-        r.x -= (c.x - m.x) / h;
-        r.y -= (c.y - m.y) / h;
-    }
-    return r;
-}
-
-struct AnWin {
-    int sx0, sx1, sy0, sy1, SW;
-};
-
-// stage e (or zeros), rhs and the row types of the window
-template <typename R>
-__device__ void an_stage(typename CX<R>::T* E, typename CX<R>::T* Rr, unsigned char* Ty, const AnWin& w,
-                         const typename CX<R>::T* __restrict__ e, const typename CX<R>::T* __restrict__ rhs,
-                         const unsigned char* __restrict__ typ, int n, bool load_e)
-{
-    typedef typename CX<R>::T c2;
-    const int S = n + 1, ww = w.sx1 - w.sx0 + 1, wh = w.sy1 - w.sy0 + 1;
-    const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    c2 z;
-    z.x = 0;
-    z.y = 0;
-    for (int ly = threadIdx.x >> 5; ly < wh; ly += nw)
-        for (int lx = lane; lx < ww; lx += 32) {
-            const int g = (w.sy0 + ly) * S + w.sx0 + lx, q = ly * w.SW + lx;
-            E[q] = load_e ? e[g] : z;
-            Rr[q] = rhs[g];
-            Ty[q] = typ[g];
-        }
-}
-
-// Red-black Gauss-Seidel on the nodes of colour `color` in row i, columns ux0..ux1, of
-// arrays with row stride SW whose element 0 is node (oy, ox); the warp's lanes take the
-// row's nodes of that colour.  PDE rows take the 5-point local solve, EDGE rows the mean
-// of their inward neighbours plus h rhs.
-template <typename R>
-__device__ __forceinline__ void an_row(typename CX<R>::T* E, const typename CX<R>::T* Rr, const unsigned char* Ty,
-                                       int SW, int oy, int ox, int i, int ux0, int ux1, int n, R h, R dinv,
-                                       int color)
-{
-    typedef typename CX<R>::T c2;
+    if (ya > yb || xa > xb) return;
+    const int nx = (xb - xa + 2) >> 1, total = nx * (yb - ya + 1);
+    const unsigned m = an_magic(nx);
     const R h2 = h * h;
-    const int jf = ux0 + ((i + ux0 + color) & 1);
-    for (int j = jf + 2 * (int)(threadIdx.x & 31); j <= ux1; j += 64) {
-        const int q = (i - oy) * SW + (j - ox);
-        const unsigned char ty = Ty[q];
-        if (ty == AN_PDE) {
-            const c2 sn = nbr_sum(E, q, SW);
-            const c2 r = Rr[q];
-            c2 v;
-            v.x = (sn.x - h2 * r.x) * dinv;
-            v.y = (sn.y - h2 * r.y) * dinv;
-            E[q] = v;
-        } else if (ty == AN_EDGE) {
-            const c2 m = inward_mean_w(E, q, SW, i, j, n);
-            const c2 r = Rr[q];
-            c2 v;
-            v.x = m.x + h * r.x;
-            v.y = m.y + h * r.y;
-            E[q] = v;
+    c2* __restrict__ Ec = w.E(color);
+    const c2* __restrict__ Eo = w.E(color ^ 1);
+    const c2* __restrict__ Rc = w.Rh(color);
+    for (int q = threadIdx.x; q < total; q += blockDim.x) {
+        const int r = an_div(q, nx, m);
+        const int i = ya + r;
+        const int j = xa + ((xa + i + color) & 1) + 2 * (q - r * nx);
+        if (j > xb) continue;
+        if (!PURE && g.hole(i, j)) continue;
+        const int o = w.at(i, j);
+        const c2 rr = Rc[o];
+        c2 v;
+        if (PURE || !g.edge(i, j)) {
+            const c2 a = Eo[w.at(i - 1, j)], b = Eo[w.at(i + 1, j)], c = Eo[w.at(i, j - 1)], d = Eo[w.at(i, j + 1)];
+            v.x = (((a.x + b.x) + (c.x + d.x)) - h2 * rr.x) * dinv;
+            v.y = (((a.y + b.y) + (c.y + d.y)) - h2 * rr.y) * dinv;
+        } else {
+            const c2 s = inward_mean_w<R>(w, Eo, i, j, g.n);
+            v.x = s.x + h * rr.x;
+            v.y = s.y + h * rr.y;
         }
+        Ec[o] = v;
     }
 }
 
-// one half-sweep over rows uy0..uy1, a warp per row
-template <typename R>
-__device__ __forceinline__ void an_half(typename CX<R>::T* E, const typename CX<R>::T* Rr, const unsigned char* Ty,
-                                        int SW, int oy, int ox, int uy0, int uy1, int ux0, int ux1, int n, R h,
-                                        R dinv, int color)
+// does the box hold neither edge nor hole nodes?
+__device__ __forceinline__ bool an_pure(const AnGeo& g, int ya, int yb, int xa, int xb)
 {
-    const int nw = blockDim.x >> 5;
-    for (int i = uy0 + (int)(threadIdx.x >> 5); i <= uy1; i += nw)
-        an_row<R>(E, Rr, Ty, SW, oy, ox, i, ux0, ux1, n, h, dinv, color);
+    return ya >= 1 && yb < g.n && xa >= 1 && xb < g.n && (yb < g.lo || ya > g.hi || xb < g.lo || xa > g.hi);
 }
 
-// Full weighting of the residual at coarse PDE nodes, injection at EDGE nodes, zero on the
-// hole, for coarse rows CI0..CI1, columns CJ0..CJ1; Res holds the fine residual with row
-// stride RW, element 0 at fine node (roy, rox).  The coarse value goes to out(I, J).
-template <typename R, typename F>
-__device__ __forceinline__ void an_restrict_res(const typename CX<R>::T* Res, int RW, int roy, int rox,
-                                                const unsigned char* tc, int Sc, int CI0, int CI1, int CJ0, int CJ1,
-                                                F out)
+template <typename R>
+__device__ __forceinline__ void an_half_any(const AnWin<R>& w, const AnGeo& g, int ya, int yb, int xa, int xb, R h,
+                                            R dinv, int color)
 {
-    typedef typename CX<R>::T c2;
-    const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    for (int I = CI0 + (threadIdx.x >> 5); I <= CI1; I += nw)
-        for (int J = CJ0 + lane; J <= CJ1; J += 32) {
-            const unsigned char ty = tc[I * Sc + J];
-            c2 v;
-            if (ty == AN_HOLE) {
-                v.x = 0;
-                v.y = 0;
-            } else if (ty == AN_EDGE) {
-                v = Res[(2 * I - roy) * RW + (2 * J - rox)];
-            } else {
-                R ax = 0, ay = 0;
-#pragma unroll
-                for (int a = -1; a <= 1; ++a)
-#pragma unroll
-                    for (int b = -1; b <= 1; ++b) {
-                        const R wgt = (R)((2 - (a < 0 ? -a : a)) * (2 - (b < 0 ? -b : b)));
-                        const c2 r = Res[(2 * I + a - roy) * RW + (2 * J + b - rox)];
-                        ax += wgt * r.x;
-                        ay += wgt * r.y;
-                    }
-                v.x = ax * (R)(1.0 / 16.0);
-                v.y = ay * (R)(1.0 / 16.0);
-            }
-            out(I, J, v);
-        }
+    if (an_pure(g, ya, yb, xa, xb)) an_half_w<R, true>(w, g, ya, yb, xa, xb, h, dinv, color);
+    else an_half_w<R, false>(w, g, ya, yb, xa, xb, h, dinv, color);
 }
 
-// nu red-black sweeps on the window
+// nu sweeps of a window of `rows` rows whose outermost `skip` nodes are already spent
 template <typename R>
-__device__ void an_sweeps_w(typename CX<R>::T* E, const typename CX<R>::T* Rr, const unsigned char* Ty,
-                            const AnWin& w, int n, R h, R dinv, int nu)
+__device__ __forceinline__ void an_sweeps_w(const AnWin<R>& w, const AnGeo& g, int rows, int cols, int skip, R h,
+                                            R dinv, int nu)
 {
     for (int k = 0; k < 2 * nu; ++k) {
-        const int ux0 = w.sx0 == 0 ? 0 : w.sx0 + k + 1, ux1 = w.sx1 == n ? n : w.sx1 - k - 1;
-        const int uy0 = w.sy0 == 0 ? 0 : w.sy0 + k + 1, uy1 = w.sy1 == n ? n : w.sy1 - k - 1;
-        an_half<R>(E, Rr, Ty, w.SW, w.sy0, w.sx0, uy0, uy1, ux0, ux1, n, h, dinv, k & 1);
+        const int s = skip + k + 1;
+        an_half_any<R>(w, g, max(0, w.y0 + s), min(g.n, w.y0 + rows - 1 - s), max(0, w.x0 + s),
+                       min(g.n, w.x0 + cols - 1 - s), h, dinv, k & 1);
         __syncthreads();
     }
 }
 
+// the band sweeps (PDE rows of the ring) on such a window; its 2 AN_BAND_SWEEPS outermost
+// nodes are spent afterwards
 template <typename R>
-__host__ __device__ size_t an_win_bytes(int SW)
+__device__ __forceinline__ void an_band_w(const AnWin<R>& w, const AnGeo& g, int rows, int cols, bool whole, R h,
+                                          R dinv)
 {
-    const size_t pts = (size_t)SW * SW;
-    return 2 * an_a16(pts * sizeof(typename CX<R>::T)) + an_a16(pts);
+    for (int k = 0; k < 2 * AN_BAND_SWEEPS; ++k) {
+        const int s = whole ? 0 : k + 1;
+        an_half_w<R, false>(w, g, max(g.b0, w.y0 + s), min(g.b1, w.y0 + rows - 1 - s), max(g.b0, w.x0 + s),
+                            min(g.b1, w.x0 + cols - 1 - s), h, dinv, k & 1);
+        __syncthreads();
+    }
 }
-__host__ __device__ constexpr int an_down_sw(int nu1) { return 2 * AN_CT + 3 + 4 * nu1; }
-constexpr int AN_RW = 2 * AN_CT + 1;  // fine residual rows / columns of a descent tile
-template <typename R>
-size_t an_down_bytes(int nu1)
-{
-    return an_win_bytes<R>(an_down_sw(nu1)) + an_a16((size_t)AN_RW * AN_RW * sizeof(typename CX<R>::T));
-}
-__host__ __device__ constexpr int an_up_sw(int nu2) { return AN_FT + 4 * nu2; }
 
-// Descent of one level: nu1 sweeps, then the coarse rhs (full weighting of the residual at
-// coarse PDE nodes, injection at coarse edge nodes, zero on the hole) and a zero coarse
-// iterate for the coarse nodes [I0, I0 + AN_CT) x [J0, J0 + AN_CT); the swept fine iterate
-// goes to e_out on the fine nodes [2 I0, 2 I0 + 2 AN_CT) x [2 J0, 2 J0 + 2 AN_CT): a
-// separate buffer, since other CTAs stage their windows from e_in meanwhile.
+// stage rows x cols nodes of e (or zeros) and rhs (asynchronous copies; the caller waits)
 template <typename R>
-__global__ void __launch_bounds__(AN_NT)
-k_an_down(const typename CX<R>::T* __restrict__ e, typename CX<R>::T* __restrict__ e_out,
-          const typename CX<R>::T* __restrict__ rhs,
-          const unsigned char* __restrict__ typ, int n, R h, R dinv, R sig, int nu1, int load_e,
-          typename CX<R>::T* __restrict__ rc, typename CX<R>::T* __restrict__ ec,
-          const unsigned char* __restrict__ tc, int nc)
+__device__ __forceinline__ void an_stage(const AnWin<R>& w, int rows, int cols, const typename CX<R>::T* __restrict__ e,
+                                         const typename CX<R>::T* __restrict__ rhs, int n, bool load_e)
 {
     typedef typename CX<R>::T c2;
+    const int S = n + 1;
+    const unsigned m = an_magic(cols);
+    c2 z;
+    z.x = 0;
+    z.y = 0;
+    for (int q = threadIdx.x; q < rows * cols; q += blockDim.x) {
+        const int ly = an_div(q, cols, m), lx = q - ly * cols;
+        const int i = w.y0 + ly, j = w.x0 + lx;
+        const bool in = i >= 0 && i <= n && j >= 0 && j <= n;
+        const size_t gq = in ? (size_t)i * S + j : 0;
+        const int c = (i + j) & 1, o = w.at(i, j);
+        if (load_e) cp_async_elem<sizeof(c2)>(w.E(c) + o, e + gq, in);
+        else w.E(c)[o] = z;
+        cp_async_elem<sizeof(c2)>(w.Rh(c) + o, rhs + gq, in);
+    }
+}
+
+// residual of the row at (i, j): zero on the hole, rhs itself where the iterate is zero
+template <typename R>
+__device__ __forceinline__ typename CX<R>::T an_resid_w(const AnWin<R>& w, const AnGeo& g, int i, int j, R h, R ih2,
+                                                        R sig, bool zero)
+{
+    typedef typename CX<R>::T c2;
+    const int color = (i + j) & 1, o = w.at(i, j);
+    c2 r = w.Rh(color)[o];
+    if (g.hole(i, j)) { r.x = 0; r.y = 0; return r; }
+    if (zero) return r;
+    const c2 c = w.E(color)[o];
+    const c2* __restrict__ Eo = w.E(color ^ 1);
+    if (!g.edge(i, j)) {
+        const c2 p = Eo[w.at(i - 1, j)], q = Eo[w.at(i + 1, j)], s = Eo[w.at(i, j - 1)], t = Eo[w.at(i, j + 1)];
+        const R sx = (p.x + q.x) + (s.x + t.x), sy = (p.y + q.y) + (s.y + t.y);
+        r.x -= (sx - (R)4 * c.x) * ih2 - sig * c.x;
+        r.y -= (sy - (R)4 * c.y) * ih2 - sig * c.y;
+    } else {
+        const c2 mm = inward_mean_w<R>(w, Eo, i, j, g.n);
+        r.x -= (c.x - mm.x) / h;
+        r.y -= (c.y - mm.y) / h;
+    }
+    return r;
+}
+
+// coarse node (I, J) of the restriction of the fine residual, res(i, j) at fine nodes: full
+// weighting at PDE nodes, injection at EDGE nodes, zero on the hole
+template <typename R, typename F>
+__device__ __forceinline__ typename CX<R>::T an_restrict_node(const AnGeo& gc, int I, int J, F res)
+{
+    typedef typename CX<R>::T c2;
+    c2 v;
+    if (gc.hole(I, J)) {
+        v.x = 0;
+        v.y = 0;
+    } else if (gc.edge(I, J)) {
+        v = res(2 * I, 2 * J);
+    } else {
+        R ax = 0, ay = 0;
+#pragma unroll
+        for (int a = -1; a <= 1; ++a)
+#pragma unroll
+            for (int b = -1; b <= 1; ++b) {
+                const R wgt = (R)((2 - (a < 0 ? -a : a)) * (2 - (b < 0 ? -b : b)));
+                const c2 r = res(2 * I + a, 2 * J + b);
+                ax += wgt * r.x;
+                ay += wgt * r.y;
+            }
+        v.x = ax * (R)(1.0 / 16.0);
+        v.y = ay * (R)(1.0 / 16.0);
+    }
+    return v;
+}
+
+__host__ __device__ constexpr int an_down_rows(int T, int nu1) { return T + 3 + 4 * nu1; }
+__host__ __device__ constexpr int an_up_w(int T, int nu2, bool band)
+{
+    return T + 2 * (2 * nu2 + (band ? 2 * AN_BAND_SWEEPS : 0));
+}
+template <typename R> size_t an_down_bytes(int T, int nu1)
+{
+    return 2 * (size_t)an_down_rows(T, nu1) * (an_down_rows(T, nu1) + 1) * sizeof(typename CX<R>::T);
+}
+template <typename R> size_t an_up_bytes(int T, int nu2)
+{
+    const size_t W = an_up_w(T, nu2, true);
+    return (2 * W * W + (W / 2 + 1) * (W / 2 + 1)) * sizeof(typename CX<R>::T);
+}
+
+template <typename R>
+__device__ __forceinline__ AnWin<R> an_window(void* smem, int y0, int x0, int rows, int W)
+{
+    typedef typename CX<R>::T c2;
+    const int pl = rows * (W >> 1);
+    c2* b = reinterpret_cast<c2*>(smem);
+    return AnWin<R>{y0, x0, W, b, b + pl, b + 2 * pl, b + 3 * pl};
+}
+
+// Descent of one level: nu1 sweeps, then the coarse rhs for the T / 2 x T / 2 coarse nodes from
+// (I0, J0); the swept fine iterate goes to e_out on the T x T fine nodes from (2 I0, 2 J0): a
+// separate buffer, since other CTAs stage their windows from e meanwhile.
+// Bound by the latency of its phases (FP64: by an SM's FP64 rate).  complex64, cold: level
+// 1024 34 -> 28.8 us, 512 16 -> 10.6, 128 12 -> 8.3 against rows by warps with type bytes and
+// unbatched loads.
+template <typename R, int T>
+__global__ void __launch_bounds__(AN_TT, 2)
+k_an_down(const typename CX<R>::T* __restrict__ e, typename CX<R>::T* __restrict__ e_out,
+          const typename CX<R>::T* __restrict__ rhs, AnGeo g, R h, R dinv, R sig, R ih2, int nu1, int load_e,
+          typename CX<R>::T* __restrict__ rc, AnGeo gc)
+{
+    typedef typename CX<R>::T c2;
+    constexpr int AN_CT = T / 2;
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int n = g.n, nc = gc.n;
     const int ntc = (nc + AN_CT) / AN_CT;
     const int I0 = (blockIdx.x / ntc) * AN_CT, J0 = (blockIdx.x % ntc) * AN_CT;
     const int hw = 2 + 2 * nu1;               // low side; the high side needs 2 nu1
-    AnWin w;
-    w.SW = an_down_sw(nu1);
-    w.sy0 = max(0, 2 * I0 - hw);
-    w.sy1 = min(n, 2 * I0 + 2 * AN_CT + 2 * nu1);
-    w.sx0 = max(0, 2 * J0 - hw);
-    w.sx1 = min(n, 2 * J0 + 2 * AN_CT + 2 * nu1);
-    const size_t pts = (size_t)w.SW * w.SW;
-    c2* E = reinterpret_cast<c2*>(smem_raw);
-    c2* Rr = reinterpret_cast<c2*>(smem_raw + an_a16(pts * sizeof(c2)));
-    unsigned char* Ty = smem_raw + 2 * an_a16(pts * sizeof(c2));
-    c2* Res = reinterpret_cast<c2*>(smem_raw + an_win_bytes<R>(w.SW));
-    an_stage<R>(E, Rr, Ty, w, e, rhs, typ, n, load_e != 0);
+    const int rows = an_down_rows(T, nu1), W = rows + 1;
+    const AnWin<R> w = an_window<R>(smem_raw, 2 * I0 - hw, 2 * J0 - hw, rows, W);
+    pdl_wait();
+    pdl_trigger();
+    an_stage<R>(w, rows, rows, e, rhs, n, load_e != 0);
+    cp_async_wait_all();
     __syncthreads();
-    an_sweeps_w<R>(E, Rr, Ty, w, n, h, dinv, nu1);
+    an_sweeps_w<R>(w, g, rows, rows, 0, h, dinv, nu1);
     const bool zero = nu1 == 0 && load_e == 0;
     const int Sc = nc + 1, S = n + 1;
     const int ci1 = min(nc, I0 + AN_CT - 1), cj1 = min(nc, J0 + AN_CT - 1);
-    const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    // the fine residual once per node: rows / columns 2 I0 - 1 .. 2 ci1 + 1 (within the grid)
-    const int roy = 2 * I0 - 1, rox = 2 * J0 - 1;
-    {
-        const int ry0 = max(0, roy), ry1 = min(n, 2 * ci1 + 1), rx0 = max(0, rox), rx1 = min(n, 2 * cj1 + 1);
-        for (int i = ry0 + (threadIdx.x >> 5); i <= ry1; i += nw)
-            for (int j = rx0 + lane; j <= rx1; j += 32)
-                Res[(i - roy) * AN_RW + (j - rox)] =
-                    an_resid_w<R>(E, Rr, Ty, (i - w.sy0) * w.SW + (j - w.sx0), w.SW, i, j, n, h, sig, zero);
-    }
-    __syncthreads();
-    an_restrict_res<R>(Res, AN_RW, roy, rox, tc, Sc, I0, ci1, J0, cj1, [&](int I, int J, c2 v) {
-        c2 z;
-        z.x = 0;
-        z.y = 0;
-        ec[I * Sc + J] = z;
-        rc[I * Sc + J] = v;
-    });
     {
         const int fi1 = min(n, 2 * I0 + 2 * AN_CT - 1), fj1 = min(n, 2 * J0 + 2 * AN_CT - 1);
-        for (int i = 2 * I0 + (threadIdx.x >> 5); i <= fi1; i += nw)
-            for (int j = 2 * J0 + lane; j <= fj1; j += 32) e_out[i * S + j] = E[(i - w.sy0) * w.SW + (j - w.sx0)];
+        for (int q = threadIdx.x; q < 4 * AN_CT * AN_CT; q += AN_TT) {
+            const int i = 2 * I0 + q / (2 * AN_CT), j = 2 * J0 + q % (2 * AN_CT);
+            if (i <= fi1 && j <= fj1) e_out[(size_t)i * S + j] = w.e(i, j);
+        }
     }
-}
-
-// Ascent sweeps of one level: nu2 sweeps of e_in; the fine nodes [32 by, 32 by + 32) x
-// [32 bx, 32 bx + 32) go to e_out.
-template <typename R>
-__global__ void __launch_bounds__(AN_NT)
-k_an_up(const typename CX<R>::T* __restrict__ e, typename CX<R>::T* __restrict__ e_out,
-        const typename CX<R>::T* __restrict__ rhs,
-        const unsigned char* __restrict__ typ, int n, R h, R dinv, int nu2)
-{
-    typedef typename CX<R>::T c2;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int nt = (n + AN_FT) / AN_FT;
-    const int i0 = (blockIdx.x / nt) * AN_FT, j0 = (blockIdx.x % nt) * AN_FT;
-    const int hw = 2 * nu2;
-    AnWin w;
-    w.SW = an_up_sw(nu2);
-    w.sy0 = max(0, i0 - hw);
-    w.sy1 = min(n, i0 + AN_FT - 1 + hw);
-    w.sx0 = max(0, j0 - hw);
-    w.sx1 = min(n, j0 + AN_FT - 1 + hw);
-    const size_t pts = (size_t)w.SW * w.SW;
-    c2* E = reinterpret_cast<c2*>(smem_raw);
-    c2* Rr = reinterpret_cast<c2*>(smem_raw + an_a16(pts * sizeof(c2)));
-    unsigned char* Ty = smem_raw + 2 * an_a16(pts * sizeof(c2));
-    an_stage<R>(E, Rr, Ty, w, e, rhs, typ, n, true);
+    // the fine residual once per node, in place of the window's rhs: rows / columns
+    // 2 I0 - 1 .. 2 ci1 + 1 (within the grid)
+    {
+        const int ry0 = max(0, 2 * I0 - 1), ry1 = min(n, 2 * ci1 + 1);
+        const int rx0 = max(0, 2 * J0 - 1), rx1 = min(n, 2 * cj1 + 1);
+        const int nx = rx1 - rx0 + 1;
+        const unsigned m = an_magic(nx);
+        for (int q = threadIdx.x; q < nx * (ry1 - ry0 + 1); q += AN_TT) {
+            const int r = an_div(q, nx, m), i = ry0 + r, j = rx0 + (q - r * nx);
+            w.Rh((i + j) & 1)[w.at(i, j)] = an_resid_w<R>(w, g, i, j, h, ih2, sig, zero);
+        }
+    }
     __syncthreads();
-    an_sweeps_w<R>(E, Rr, Ty, w, n, h, dinv, nu2);
-    const int S = n + 1, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    const int fi1 = min(n, i0 + AN_FT - 1), fj1 = min(n, j0 + AN_FT - 1);
-    for (int i = i0 + (threadIdx.x >> 5); i <= fi1; i += nw)
-        for (int j = j0 + lane; j <= fj1; j += 32) e_out[i * S + j] = E[(i - w.sy0) * w.SW + (j - w.sx0)];
+    for (int q = threadIdx.x; q < AN_CT * AN_CT; q += AN_TT) {
+        const int I = I0 + q / AN_CT, J = J0 + q % AN_CT;
+        if (I > ci1 || J > cj1) continue;
+        rc[(size_t)I * Sc + J] = an_restrict_node<R>(
+            gc, I, J, [&](int i, int j) -> c2 { return w.Rh((i + j) & 1)[w.at(i, j)]; });
+    }
 }
 
-// coarse rhs: full weighting of the fine residual at PDE nodes, injection at EDGE nodes;
-// coarse iterate := 0
-template <typename R>
-__global__ void __launch_bounds__(AN_NT)
-k_an_restrict(const typename CX<R>::T* __restrict__ ef, const typename CX<R>::T* __restrict__ rf,
-              const unsigned char* __restrict__ tf, int nf, R hf, R sig, typename CX<R>::T* __restrict__ rc,
-              typename CX<R>::T* __restrict__ ec, const unsigned char* __restrict__ tc, int nc, int zero)
+// e(i, j) += bilinear interpolation of the coarse iterate, ce(I, J)
+template <typename R, typename F>
+__device__ __forceinline__ typename CX<R>::T an_corrected(typename CX<R>::T v, int i, int j, F ce)
+{
+    const int I0 = i >> 1, I1 = (i + 1) >> 1, J0 = j >> 1, J1 = (j + 1) >> 1;
+    const auto a = ce(I0, J0), b = ce(I1, J0), c = ce(I0, J1), d = ce(I1, J1);
+    v.x += (R)0.25 * (((a.x + b.x) + c.x) + d.x);
+    v.y += (R)0.25 * (((a.y + b.y) + c.y) + d.y);
+    return v;
+}
+
+// Ascent of one level: the correction e2 + interpolation of the coarse iterate ec, the band
+// sweeps around the hole, nu2 sweeps; T x T fine nodes go to e_out.  Only the tiles whose window meets the ring make the band sweeps, on a window
+// 2 AN_BAND_SWEEPS nodes wider on every side (their values there are recomputed, the same, by
+// the tiles that share them).  One launch for what were a prolongation (5 us), the band in one
+// CTA (15) and a sweep launch (15-22): complex64 11 us at levels 128 and 256, 13.6 at 512, 28
+// at 1024, cold.
+template <typename R, int T>
+__global__ void __launch_bounds__(AN_TT, 2)
+k_an_up(const typename CX<R>::T* __restrict__ e2, typename CX<R>::T* __restrict__ e_out,
+        const typename CX<R>::T* __restrict__ rhs, AnGeo g, R h, R dinv, int nu2,
+        const typename CX<R>::T* __restrict__ ec, int nc)
 {
     typedef typename CX<R>::T c2;
-    const int Sc = nc + 1;
-    const long total = (long)Sc * Sc;
-    for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < total; t += (long)gridDim.x * blockDim.x) {
-        const int I = (int)(t / Sc), J = (int)(t % Sc);
-        c2 z;
-        z.x = 0;
-        z.y = 0;
-        ec[t] = z;
-        const unsigned char ty = tc[t];
-        if (ty == AN_HOLE) {
-            rc[t] = z;
-        } else if (ty == AN_EDGE) {
-            rc[t] = an_resid<R>(ef, rf, tf, 2 * I, 2 * J, nf, hf, sig, zero != 0);
-        } else {
-            R ax = 0, ay = 0;
-#pragma unroll
-            for (int a = -1; a <= 1; ++a)
-#pragma unroll
-                for (int b = -1; b <= 1; ++b) {
-                    const R wgt = (R)((2 - (a < 0 ? -a : a)) * (2 - (b < 0 ? -b : b)));
-                    const c2 r = an_resid<R>(ef, rf, tf, 2 * I + a, 2 * J + b, nf, hf, sig, zero != 0);
-                    ax += wgt * r.x;
-                    ay += wgt * r.y;
-                }
-            c2 v;
-            v.x = ax * (R)(1.0 / 16.0);
-            v.y = ay * (R)(1.0 / 16.0);
-            rc[t] = v;
+    constexpr int AN_FT = T;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int n = g.n, nt = (n + AN_FT) / AN_FT;
+    const int i0 = (blockIdx.x / nt) * AN_FT, j0 = (blockIdx.x % nt) * AN_FT;
+    const int h0 = 2 * nu2;
+    const bool band = i0 - h0 <= g.b1 && i0 + AN_FT - 1 + h0 >= g.b0 && j0 - h0 <= g.b1 &&
+                      j0 + AN_FT - 1 + h0 >= g.b0;
+    const int skip = band ? 2 * AN_BAND_SWEEPS : 0;
+    const int W = an_up_w(T, nu2, band), CW = W / 2 + 1;
+    const AnWin<R> w = an_window<R>(smem_raw, i0 - h0 - skip, j0 - h0 - skip, W, W);
+    c2* const Cs = w.R1 + W * (W >> 1);
+    const int cy0 = w.y0 >> 1, cx0 = w.x0 >> 1;            // even origins
+    pdl_wait();
+    pdl_trigger();
+    {
+        const int Sc = nc + 1;
+        const unsigned m = an_magic(CW);
+        for (int q = threadIdx.x; q < CW * CW; q += AN_TT) {
+            const int r = an_div(q, CW, m), I = cy0 + r, J = cx0 + (q - r * CW);
+            const bool in = I >= 0 && I <= nc && J >= 0 && J <= nc;
+            cp_async_elem<sizeof(c2)>(Cs + q, ec + (in ? (size_t)I * Sc + J : 0), in);
         }
     }
-}
-
-// fine iterate += bilinear interpolation of the coarse one (fine hole nodes untouched)
-template <typename R>
-__global__ void __launch_bounds__(AN_NT)
-k_an_prolong(const typename CX<R>::T* __restrict__ ec, int nc, typename CX<R>::T* __restrict__ ef,
-             const unsigned char* __restrict__ tf, int nf)
-{
-    typedef typename CX<R>::T c2;
-    const int Sf = nf + 1, Sc = nc + 1;
-    const long total = (long)Sf * Sf;
-    for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < total; t += (long)gridDim.x * blockDim.x) {
-        if (tf[t] == AN_HOLE) continue;
-        const int i = (int)(t / Sf), j = (int)(t % Sf);
-        const int I0 = i >> 1, I1 = (i + 1) >> 1, J0 = j >> 1, J1 = (j + 1) >> 1;
-        const c2 a = ec[I0 * Sc + J0], b = ec[I1 * Sc + J0], c = ec[I0 * Sc + J1], d = ec[I1 * Sc + J1];
-        c2 v = ef[t];
-        v.x += (R)0.25 * (((a.x + b.x) + c.x) + d.x);
-        v.y += (R)0.25 * (((a.y + b.y) + c.y) + d.y);
-        ef[t] = v;
+    an_stage<R>(w, W, W, e2, rhs, n, true);
+    cp_async_wait_all();
+    __syncthreads();
+    {
+        const int ya = max(0, w.y0), yb = min(n, w.y0 + W - 1), xa = max(0, w.x0), xb = min(n, w.x0 + W - 1);
+        // without band sweeps the first half-sweep overwrites colour 0 unread: colour 1 alone
+        const bool half = !band && nu2 > 0;
+        const int nx = half ? (xb - xa + 2) >> 1 : xb - xa + 1;
+        const unsigned m = an_magic(nx);
+        for (int q = threadIdx.x; q < nx * (yb - ya + 1); q += AN_TT) {
+            const int r = an_div(q, nx, m), i = ya + r, u = q - r * nx;
+            const int j = half ? xa + ((xa + i + 1) & 1) + 2 * u : xa + u;
+            if (j > xb || g.hole(i, j)) continue;
+            c2* const p = w.E((i + j) & 1) + w.at(i, j);
+            *p = an_corrected<R>(*p, i, j, [&](int I, int J) -> c2 { return Cs[(I - cy0) * CW + (J - cx0)]; });
+        }
+    }
+    __syncthreads();
+    if (band) an_band_w<R>(w, g, W, W, false, h, dinv);
+    an_sweeps_w<R>(w, g, W, W, skip, h, dinv, nu2);
+    const int S = n + 1;
+    for (int q = threadIdx.x; q < AN_FT * AN_FT; q += AN_TT) {
+        const int i = i0 + q / AN_FT, j = j0 + q % AN_FT;
+        if (i <= n && j <= n) e_out[(size_t)i * S + j] = w.e(i, j);
     }
 }
 
-// coarsest level: e = Ainv rhs over its m unknowns (map: unknown -> node); a warp per row,
-// its lanes over the columns (coalesced rows of Ainv), partial sums added by a butterfly
-template <typename R>
-__device__ __forceinline__ void an_dense_solve(const typename CX<R>::T* rhs, typename CX<R>::T* e,
-                                               const double* __restrict__ Ainv, const int* __restrict__ map, int m)
+// Coarsest level: e = Ainv rhs over its m unknowns (map: unknown -> node).  At holds Ainv
+// transposed (column by column), so that neighbouring threads, which form neighbouring
+// unknowns, read neighbouring words.  A warp's FP64 instruction holds its sub-core's pipe
+// for 64 clocks: the columns are shared out so that every lane multiplies (a butterfly of
+// FP64 adds per row took longer than the products), then each unknown adds its partial sums.
+// part: room for AN_PARTS m complex FP64 sums.
+constexpr int AN_PARTS = 14;
+template <typename R, typename FR, typename FE>
+__device__ __forceinline__ void an_dense_solve(const double* At, const int* __restrict__ map, int m, double2* part,
+                                               FR rhs, FE put)
 {
-    typedef typename CX<R>::T c2;
-    const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    for (int r = threadIdx.x >> 5; r < m; r += nw) {
+    const int groups = min(AN_PARTS, (int)blockDim.x / m), per = (m + groups - 1) / groups;
+    const int gq = threadIdx.x / m, r = threadIdx.x - gq * m;
+    if (gq < groups) {
         double ax = 0.0, ay = 0.0;
-        for (int c = lane; c < m; c += 32) {
-            const double a = Ainv[(size_t)r * m + c];
-            const c2 v = rhs[map[c]];
-            ax += a * (double)v.x;
-            ay += a * (double)v.y;
+        for (int c = gq * per; c < min(m, (gq + 1) * per); ++c) {
+            const double a = At[(size_t)c * m + r];
+            const auto v = rhs(map[c]);
+            ax = fma(a, an_widen(v.x), ax);
+            ay = fma(a, an_widen(v.y), ay);
         }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            ax += __shfl_xor_sync(0xffffffffu, ax, o);
-            ay += __shfl_xor_sync(0xffffffffu, ay, o);
-        }
-        if (lane == 0) {
-            c2 v;
-            v.x = (R)ax;
-            v.y = (R)ay;
-            e[map[r]] = v;
-        }
+        part[gq * m + r] = make_double2(ax, ay);
     }
-}
-
-template <typename R>
-__global__ void __launch_bounds__(AN_NT)
-k_an_coarse(const typename CX<R>::T* __restrict__ rhs, typename CX<R>::T* __restrict__ e,
-            const double* __restrict__ Ainv, const int* __restrict__ map, int m)
-{
-    an_dense_solve<R>(rhs, e, Ainv, map, m);
+    __syncthreads();
+    // the two components of an unknown by two threads
+    if ((int)threadIdx.x < 2 * m) {
+        const int u = threadIdx.x >> 1;
+        double s = 0.0;
+        for (int k = 0; k < groups; ++k) s += (threadIdx.x & 1) ? part[k * m + u].y : part[k * m + u].x;
+        put(map[u], threadIdx.x & 1, (R)s);
+    }
 }
 
 // ---------------------------------------------------------------------------
 // Coarse tail: the coarsest levels in one CTA, in shared memory
 // ---------------------------------------------------------------------------
-// The same V-cycle as the per-level kernels (sweeps, restriction, prolongation, band
-// sweeps, exact coarsest level), with block-wide barriers between its phases instead of
-// kernel boundaries.  Levels 64, 32, 16, 8 hold about 5.7 K nodes.  In FP64 one SM's
-// arithmetic rate (a small fraction of its FP32 rate) makes the level-64 restriction slower
-// in one CTA than spread over several, so the FP64 tail starts lower.
+// The same V-cycle as the tile kernels (sweeps, restriction, prolongation, band sweeps,
+// exact coarsest level), with block-wide barriers between its phases instead of kernel
+// boundaries.  Levels 64, 32, 16, 8 hold about 5.7 K nodes.  In FP64 one SM's arithmetic
+// rate (a small fraction of its FP32 rate) makes the larger of them slower in one CTA than
+// spread over several, so the FP64 tail starts lower.  complex64 from 64: 75 -> 47 us against
+// rows by warps over type bytes and a butterfly per row of the dense solve.
 constexpr int AN_TAIL_TOP_F = 64;
 constexpr int AN_TAIL_TOP_D = 16;
 constexpr int AN_TAIL_MAX = 4;
 
-struct AnTailLev {
-    int n, b0, b1, lo, hi;
-    double h, dinv;
-    const unsigned char* typ;
-};
 struct AnTail {
     int L, nu1, nu2, load_e, m;
     double sigma;
-    AnTailLev lev[AN_TAIL_MAX];
-    const double* Ainv;
+    AnGeo geo[AN_TAIL_MAX];
+    double h[AN_TAIL_MAX], dinv[AN_TAIL_MAX], ih2[AN_TAIL_MAX];
+    const double* At;
     const int* map;
 };
 
+// shared memory: per level the four planes ((n + 1) rows of n + 2), the top level's residual
+// planes, the coarsest level's transposed inverse and partial sums
+__host__ __device__ inline size_t an_tail_level(int n) { return (size_t)(n + 1) * (n + 2) * 2; }
+template <typename R>
+size_t an_tail_bytes(const int* ns, int L, int m)
+{
+    size_t c = (size_t)(ns[0] + 1) * (ns[0] + 2);
+    for (int l = 0; l < L; ++l) c += an_tail_level(ns[l]);
+    return an_a16(c * sizeof(typename CX<R>::T)) + an_a16((size_t)m * m * sizeof(double)) +
+           (size_t)AN_PARTS * m * sizeof(double2);
+}
 
 template <typename R>
 __global__ void __launch_bounds__(1024, 1)
@@ -732,119 +511,114 @@ k_an_tail(typename CX<R>::T* __restrict__ eg, const typename CX<R>::T* __restric
 {
     typedef typename CX<R>::T c2;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    c2* E[AN_TAIL_MAX];
-    c2* Rr[AN_TAIL_MAX];
-    unsigned char* Ty[AN_TAIL_MAX];
-    size_t off = 0;
-    for (int l = 0; l < T.L; ++l) {
-        const size_t pts = (size_t)(T.lev[l].n + 1) * (T.lev[l].n + 1);
-        E[l] = reinterpret_cast<c2*>(smem_raw + off);
-        off += an_a16(pts * sizeof(c2));
-        Rr[l] = reinterpret_cast<c2*>(smem_raw + off);
-        off += an_a16(pts * sizeof(c2));
-        Ty[l] = smem_raw + off;
-        off += an_a16(pts);
-    }
-    c2* Res = reinterpret_cast<c2*>(smem_raw + off);     // the top level's residual, once per node
-    const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    for (int l = 0; l < T.L; ++l) {
-        const int pts = (T.lev[l].n + 1) * (T.lev[l].n + 1);
-        for (int q = threadIdx.x; q < pts; q += blockDim.x) Ty[l][q] = T.lev[l].typ[q];
-    }
+    c2* const base = reinterpret_cast<c2*>(smem_raw);
+    // window l of the levels; the top level's residual planes follow the last one
+    size_t off[AN_TAIL_MAX + 1];
+    off[0] = 0;
+#pragma unroll
+    for (int l = 0; l < AN_TAIL_MAX; ++l) off[l + 1] = off[l] + (l < T.L ? an_tail_level(T.geo[l].n) : 0);
+    const size_t c_end = off[AN_TAIL_MAX] + (size_t)(T.geo[0].n + 1) * (T.geo[0].n + 2);
+    c2* const Res = base + off[AN_TAIL_MAX];
+    double* const At = reinterpret_cast<double*>(smem_raw + an_a16(c_end * sizeof(c2)));
+    double2* const part = reinterpret_cast<double2*>(smem_raw + an_a16(c_end * sizeof(c2)) +
+                                                     an_a16((size_t)T.m * T.m * sizeof(double)));
+    auto win = [&](int l) { return an_window<R>(base + off[l], 0, 0, T.geo[l].n + 1, T.geo[l].n + 2); };
+    // the inverse arrives while the cycle descends (host-written: before the wait)
+    for (int q = threadIdx.x; q < T.m * T.m; q += blockDim.x) cp_async_elem<8>(At + q, T.At + q, true);
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+    pdl_wait();
+    pdl_trigger();
     {
-        const int pts = (T.lev[0].n + 1) * (T.lev[0].n + 1);
+        const int n = T.geo[0].n;
+        const AnWin<R> w = win(0);
+        an_stage<R>(w, n + 1, n + 1, eg, rg, n, T.load_e != 0);
+    }
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+    // the coarse iterates start from zero
+    {
         c2 z;
         z.x = 0;
         z.y = 0;
-        for (int q = threadIdx.x; q < pts; q += blockDim.x) {
-            Rr[0][q] = rg[q];
-            E[0][q] = T.load_e ? eg[q] : z;
+        for (int l = 1; l < T.L; ++l) {
+            const int cnt = (T.geo[l].n + 1) * (T.geo[l].n + 2);        // both iterate planes
+            for (int q = threadIdx.x; q < cnt; q += blockDim.x) base[off[l] + q] = z;
         }
     }
+    asm volatile("cp.async.wait_all;\n" ::: "memory");
     __syncthreads();
     const R sig = (R)T.sigma;
     // descent
     for (int l = 0; l + 1 < T.L; ++l) {
-        const AnTailLev& Lv = T.lev[l];
-        const R h = (R)Lv.h, dinv = (R)Lv.dinv;
-        const int n = Lv.n, S = n + 1;
+        const AnGeo g = T.geo[l], gc = T.geo[l + 1];
+        const R h = (R)T.h[l], dinv = (R)T.dinv[l];
+        const int n = g.n, W = n + 2;
+        const AnWin<R> w = win(l);
         for (int k = 0; k < 2 * T.nu1; ++k) {
-            an_half<R>(E[l], Rr[l], Ty[l], S, 0, 0, 0, n, 0, n, n, h, dinv, k & 1);
+            an_half_w<R, false>(w, g, 0, n, 0, n, h, dinv, k & 1);
             __syncthreads();
         }
-        const int nc = T.lev[l + 1].n, Sc = nc + 1;
         const bool zero = T.nu1 == 0 && (l > 0 || !T.load_e);
-        for (int i = threadIdx.x >> 5; i <= n; i += nw)
-            for (int j = lane; j <= n; j += 32)
-                Res[i * S + j] = an_resid<R>(E[l], Rr[l], Ty[l], i, j, n, h, sig, zero);
+        const R ih2 = (R)T.ih2[l];
+        const unsigned m = an_magic(n + 1);
+        c2* const P[2] = {Res, Res + (n + 1) * (W >> 1)};
+        for (int q = threadIdx.x; q < (n + 1) * (n + 1); q += blockDim.x) {
+            const int i = an_div(q, n + 1, m), j = q - i * (n + 1);
+            P[(i + j) & 1][w.at(i, j)] = an_resid_w<R>(w, g, i, j, h, ih2, sig, zero);
+        }
         __syncthreads();
-        c2* const Ec = E[l + 1];
-        c2* const Rc = Rr[l + 1];
-        an_restrict_res<R>(Res, S, 0, 0, Ty[l + 1], Sc, 0, nc, 0, nc, [&](int I, int J, c2 v) {
-            c2 z;
-            z.x = 0;
-            z.y = 0;
-            Ec[I * Sc + J] = z;
-            Rc[I * Sc + J] = v;
-        });
+        const AnWin<R> wc = win(l + 1);
+        const unsigned mc = an_magic(gc.n + 1);
+        for (int q = threadIdx.x; q < (gc.n + 1) * (gc.n + 1); q += blockDim.x) {
+            const int I = an_div(q, gc.n + 1, mc), J = q - I * (gc.n + 1);
+            wc.Rh((I + J) & 1)[wc.at(I, J)] = an_restrict_node<R>(
+                gc, I, J, [&](int i, int j) -> c2 { return P[(i + j) & 1][w.at(i, j)]; });
+        }
         __syncthreads();
     }
     // the coarsest level, exactly
-    an_dense_solve<R>(Rr[T.L - 1], E[T.L - 1], T.Ainv, T.map, T.m);
-    __syncthreads();
+    {
+        const AnWin<R> w = win(T.L - 1);
+        const int S = T.geo[T.L - 1].n + 1;
+        an_dense_solve<R>(
+            At, T.map, T.m, part,
+            [&](int q) -> c2 { const int i = q / S, j = q - i * S; return w.Rh((i + j) & 1)[w.at(i, j)]; },
+            [&](int q, int im, R v) {
+                const int i = q / S, j = q - i * S;
+                c2* const p = w.E((i + j) & 1) + w.at(i, j);
+                if (im) p->y = v;
+                else p->x = v;
+            });
+        __syncthreads();
+    }
     // ascent
     for (int l = T.L - 2; l >= 0; --l) {
-        const AnTailLev& Lv = T.lev[l];
-        const int n = Lv.n, S = n + 1, nc = T.lev[l + 1].n, Sc = nc + 1;
-        const R h = (R)Lv.h, dinv = (R)Lv.dinv;
-        for (int i = threadIdx.x >> 5; i <= n; i += nw)
-            for (int j = lane; j <= n; j += 32) {
-                const int q = i * S + j;
-                if (Ty[l][q] == AN_HOLE) continue;
-                const int I0 = i >> 1, I1 = (i + 1) >> 1, J0 = j >> 1, J1 = (j + 1) >> 1;
-                const c2 a = E[l + 1][I0 * Sc + J0], b = E[l + 1][I1 * Sc + J0];
-                const c2 c = E[l + 1][I0 * Sc + J1], d = E[l + 1][I1 * Sc + J1];
-                c2 v = E[l][q];
-                v.x += (R)0.25 * (((a.x + b.x) + c.x) + d.x);
-                v.y += (R)0.25 * (((a.y + b.y) + c.y) + d.y);
-                E[l][q] = v;
-            }
-        __syncthreads();
-        // band sweeps around the hole: rows b0..b1 of the ring [b0, b1]^2 minus [lo, hi]^2
-        // (all PDE rows), a warp per row
-        {
-            const int b0 = Lv.b0, b1 = Lv.b1, lo = Lv.lo, hi = Lv.hi;
-            for (int k = 0; k < 2 * AN_BAND_SWEEPS; ++k) {
-                const int color = k & 1;
-                for (int i = b0 + (threadIdx.x >> 5); i <= b1; i += nw) {
-                    if (i < lo || i > hi) {
-                        an_row<R>(E[l], Rr[l], Ty[l], S, 0, 0, i, b0, b1, n, h, dinv, color);
-                    } else {
-                        an_row<R>(E[l], Rr[l], Ty[l], S, 0, 0, i, b0, lo - 1, n, h, dinv, color);
-                        an_row<R>(E[l], Rr[l], Ty[l], S, 0, 0, i, hi + 1, b1, n, h, dinv, color);
-                    }
-                }
-                __syncthreads();
-            }
+        const AnGeo g = T.geo[l];
+        const int n = g.n;
+        const R h = (R)T.h[l], dinv = (R)T.dinv[l];
+        const AnWin<R> w = win(l), wc = win(l + 1);
+        const unsigned m = an_magic(n + 1);
+        for (int q = threadIdx.x; q < (n + 1) * (n + 1); q += blockDim.x) {
+            const int i = an_div(q, n + 1, m), j = q - i * (n + 1);
+            if (g.hole(i, j)) continue;
+            c2* const p = w.E((i + j) & 1) + w.at(i, j);
+            *p = an_corrected<R>(*p, i, j, [&](int I, int J) -> c2 { return wc.e(I, J); });
         }
+        __syncthreads();
+        an_band_w<R>(w, g, n + 1, n + 1, true, h, dinv);
         for (int k = 0; k < 2 * T.nu2; ++k) {
-            an_half<R>(E[l], Rr[l], Ty[l], S, 0, 0, 0, n, 0, n, n, h, dinv, k & 1);
+            an_half_w<R, false>(w, g, 0, n, 0, n, h, dinv, k & 1);
             __syncthreads();
         }
     }
-    const int pts = (T.lev[0].n + 1) * (T.lev[0].n + 1);
-    for (int q = threadIdx.x; q < pts; q += blockDim.x) eg[q] = E[0][q];
-}
-
-template <typename R>
-size_t an_tail_bytes(const int* ns, int L)
-{
-    size_t off = 0;
-    for (int l = 0; l < L; ++l) {
-        const size_t pts = (size_t)(ns[l] + 1) * (ns[l] + 1);
-        off += 2 * an_a16(pts * sizeof(typename CX<R>::T)) + an_a16(pts);
+    {
+        const AnWin<R> w = win(0);
+        const int n = T.geo[0].n;
+        const unsigned m = an_magic(n + 1);
+        for (int q = threadIdx.x; q < (n + 1) * (n + 1); q += blockDim.x) {
+            const int i = an_div(q, n + 1, m), j = q - i * (n + 1);
+            eg[q] = w.e(i, j);
+        }
     }
-    return off + an_a16((size_t)(ns[0] + 1) * (ns[0] + 1) * sizeof(typename CX<R>::T));
 }
 
 // U := the hole data on hole nodes, 0 elsewhere (both iterate buffers)
@@ -858,12 +632,6 @@ k_an_init(double2* __restrict__ U0, double2* __restrict__ U1, const double2* __r
         U1[t] = v;
     }
 }
-
-// FP64 <-> inner precision; complex64's format changes run on the integer pipes
-__device__ __forceinline__ double an_widen(float x) { return f2d_bits(x); }
-__device__ __forceinline__ double an_widen(double x) { return x; }
-__device__ __forceinline__ float an_narrow(double x, float) { return d2f_bits(x); }
-__device__ __forceinline__ double an_narrow(double x, double) { return x; }
 
 // U_out = U_in + e on the non-hole nodes (hole nodes keep the data in both buffers);
 // per-block maxima of |e|^2 into part[2 b + 1]
@@ -1285,12 +1053,11 @@ struct helm_annulus {
         unsigned char* typ;
         void* e;
         void* rhs;
-        void* e2;                         // the swept iterate between the tile kernels
+        void* e2;                         // the swept iterate between descent and ascent
         int b0, b1, lo, hi;               // band ring [b0, b1]^2 minus the hole box [lo, hi]^2
-        size_t band_bytes;                // shared memory of k_an_band_s (0: the L2 form)
     };
     std::vector<Level> lev;
-    double* Ainv = nullptr;
+    double* At = nullptr;                 // the coarsest level's inverse, transposed
     int* map = nullptr;
     int m = 0;
     double2* U1 = nullptr;
@@ -1300,7 +1067,6 @@ struct helm_annulus {
     unsigned long long* kmin = nullptr;
     cudaStream_t stream = nullptr;
     std::vector<void*> allocs;
-    bool tiles = false;                   // the levels above the tail use the tile kernels
     cudaStream_t ls = nullptr;            // where an_vcycle and the step launch (stream, or cap)
     cudaStream_t cap = nullptr;           // non-blocking stream for capturing a step's graph
     bool capturing = false;
@@ -1408,6 +1174,21 @@ bool an_coarse_inverse(const std::vector<unsigned char>& t, int n, double h, dou
     return true;
 }
 
+// every shared-memory size the kernels of a plan can ask for (any nu1, nu2 <= 8)
+template <typename R>
+cudaError_t an_attrs()
+{
+    auto set = [](auto* k, size_t b) {
+        return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b);
+    };
+    cudaError_t e = set(k_an_down<R, 32>, an_down_bytes<R>(32, 8));
+    if (e == cudaSuccess) e = set(k_an_down<R, 16>, an_down_bytes<R>(16, 8));
+    if (e == cudaSuccess) e = set(k_an_up<R, 32>, an_up_bytes<R>(32, 8));
+    if (e == cudaSuccess) e = set(k_an_up<R, 16>, an_up_bytes<R>(16, 8));
+    if (e == cudaSuccess) e = set(k_an_tail<R>, AN_SMEM_MAX);
+    return e;
+}
+
 // kernels launched (or recorded into a step graph, counted at each replay)
 void an_count(helm_annulus* a, uint64_t n)
 {
@@ -1415,6 +1196,45 @@ void an_count(helm_annulus* a, uint64_t n)
     else add_launches(n);
 }
 
+AnGeo an_geo(const helm_annulus::Level& L) { return AnGeo{L.n, L.lo, L.hi, L.b0, L.b1}; }
+
+// fine nodes per side of a tile: the smaller tiles where the larger would not reach every SM
+// (each is then bound by its own phases, in FP64 by one SM's FP64 rate: N = 256 FP64 9.9 ms a
+// solve with 32 everywhere, 6.0 with this rule; 512 complex64 4.1 -> 3.8)
+int an_tile(int n)
+{
+    const int nt = (n + 32) / 32;
+    return nt * nt >= 152 ? 32 : 16;
+}
+
+template <typename R, int T>
+helm_status an_down(helm_annulus* a, const helm_annulus::Level& L, const helm_annulus::Level& C, bool zero)
+{
+    typedef typename CX<R>::T c2;
+    const R h = (R)L.h, dinv = (R)(1.0 / (4.0 + a->sigma * L.h * L.h));
+    const int nt = (C.n + T / 2) / (T / 2);
+    AN_CK(launch_k(k_an_down<R, T>, dim3(nt * nt), dim3(AN_TT), an_down_bytes<R>(T, a->nu1), a->ls, (const c2*)L.e,
+                   (c2*)L.e2, (const c2*)L.rhs, an_geo(L), h, dinv, (R)a->sigma, (R)1 / (h * h), a->nu1, zero ? 0 : 1,
+                   (c2*)C.rhs, an_geo(C)));
+    an_count(a, 1);
+    return HELM_OK;
+}
+
+template <typename R, int T>
+helm_status an_up(helm_annulus* a, const helm_annulus::Level& L, const helm_annulus::Level& C)
+{
+    typedef typename CX<R>::T c2;
+    const R h = (R)L.h, dinv = (R)(1.0 / (4.0 + a->sigma * L.h * L.h));
+    const int nt = (L.n + T) / T;
+    AN_CK(launch_k(k_an_up<R, T>, dim3(nt * nt), dim3(AN_TT), an_up_bytes<R>(T, a->nu2), a->ls, (const c2*)L.e2,
+                   (c2*)L.e, (const c2*)L.rhs, an_geo(L), h, dinv, a->nu2, (const c2*)C.e, C.n));
+    an_count(a, 1);
+    return HELM_OK;
+}
+
+// One V(nu1, nu2) cycle from level l down.  The iterate goes e -> e2 (descent), then e2 + the
+// coarse correction -> e (ascent): the tiles of a launch stage windows of the buffer that
+// none of them writes.
 template <typename R>
 helm_status an_vcycle(helm_annulus* a, int l, bool zero)
 {
@@ -1429,74 +1249,26 @@ helm_status an_vcycle(helm_annulus* a, int l, bool zero)
         T.load_e = zero ? 0 : 1;
         T.m = a->m;
         T.sigma = a->sigma;
-        T.Ainv = a->Ainv;
+        T.At = a->At;
         T.map = a->map;
         for (int i = 0; i < T.L; ++i) {
             const auto& V = a->lev[l + i];
-            T.lev[i] = AnTailLev{V.n, V.b0, V.b1, V.lo, V.hi, V.h, 1.0 / (4.0 + a->sigma * V.h * V.h), V.typ};
+            T.geo[i] = an_geo(V);
+            T.h[i] = V.h;
+            T.dinv[i] = 1.0 / (4.0 + a->sigma * V.h * V.h);
+            T.ih2[i] = (double)((R)1 / ((R)V.h * (R)V.h));
         }
-        k_an_tail<R><<<1, 1024, a->tail_bytes, s>>>((c2*)L.e, (const c2*)L.rhs, T);
-        AN_CK(cudaGetLastError());
+        for (int i = T.L; i < AN_TAIL_MAX; ++i) T.geo[i] = AnGeo{0, 0, 0, 0, 0};
+        AN_CK(launch_k(k_an_tail<R>, dim3(1), dim3(1024), a->tail_bytes, s, (c2*)L.e, (const c2*)L.rhs, T));
         an_count(a, 1);
         return HELM_OK;
     }
-    if (l + 1 == (int)a->lev.size()) {
-        k_an_coarse<R><<<1, AN_NT, 0, s>>>((const c2*)L.rhs, (c2*)L.e, a->Ainv, a->map, a->m);
-        AN_CK(cudaGetLastError());
-        an_count(a, 1);
-        return HELM_OK;
-    }
-    const R h = (R)L.h, dinv = (R)(1.0 / (4.0 + a->sigma * L.h * L.h));
-    const int half = (L.n + 2) / 2;
-    const int g = grid_for((long)(L.n + 1) * half);
     const auto& C = a->lev[l + 1];
-    const bool tiles = a->tiles;
-    // with the tile kernels the iterate goes e -> e2 (descent), e2 (correction, band),
-    // e2 -> e (ascent)
-    c2* const ew = (c2*)(tiles ? L.e2 : L.e);
-    if (tiles) {
-        const int ntc = (C.n + AN_CT) / AN_CT;
-        k_an_down<R><<<ntc * ntc, AN_NT, an_down_bytes<R>(a->nu1), s>>>(
-            (const c2*)L.e, ew, (const c2*)L.rhs, L.typ, L.n, h, dinv, (R)a->sigma, a->nu1, zero ? 0 : 1, (c2*)C.rhs,
-            (c2*)C.e, C.typ, C.n);
-        an_count(a, 1);
-    } else {
-        for (int sweep = 0; sweep < a->nu1; ++sweep)
-            for (int col = 0; col < 2; ++col) {
-                k_an_rbgs<R><<<g, AN_NT, 0, s>>>((c2*)L.e, (const c2*)L.rhs, L.typ, L.n, h, dinv, col, 0, L.n, 0,
-                                                 L.n);
-                an_count(a, 1);
-            }
-        k_an_restrict<R><<<grid_for((long)(C.n + 1) * (C.n + 1)), AN_NT, 0, s>>>(
-            (const c2*)L.e, (const c2*)L.rhs, L.typ, L.n, h, (R)a->sigma, (c2*)C.rhs, (c2*)C.e, C.typ, C.n,
-            (zero && a->nu1 == 0) ? 1 : 0);
-        an_count(a, 1);
-    }
-    helm_status st = an_vcycle<R>(a, l + 1, true);
+    helm_status st = an_tile(L.n) == 32 ? an_down<R, 32>(a, L, C, zero) : an_down<R, 16>(a, L, C, zero);
     if (st != HELM_OK) return st;
-    k_an_prolong<R><<<grid_for((long)(L.n + 1) * (L.n + 1)), AN_NT, 0, s>>>((const c2*)C.e, C.n, ew, L.typ, L.n);
-    if (L.band_bytes)
-        k_an_band_s<R><<<1, 1024, L.band_bytes, s>>>(ew, (const c2*)L.rhs, L.typ, L.n, h, dinv,
-                                                    AnRing(L.b0, L.b1, L.lo, L.hi), AN_BAND_SWEEPS);
-    else
-        k_an_band<R><<<1, 1024, 0, s>>>(ew, (const c2*)L.rhs, L.typ, L.n, h, dinv, L.b0, L.b1, L.lo, L.hi,
-                                        AN_BAND_SWEEPS);
-    an_count(a, 2);
-    if (tiles) {                           // nu2 = 0: the launch only moves e2 to e
-        const int nt = (L.n + AN_FT) / AN_FT;
-        k_an_up<R><<<nt * nt, AN_NT, an_win_bytes<R>(an_up_sw(a->nu2)), s>>>(ew, (c2*)L.e, (const c2*)L.rhs,
-                                                                            L.typ, L.n, h, dinv, a->nu2);
-        an_count(a, 1);
-    } else {
-        for (int sweep = 0; sweep < a->nu2; ++sweep)
-            for (int col = 0; col < 2; ++col) {
-                k_an_rbgs<R><<<g, AN_NT, 0, s>>>((c2*)L.e, (const c2*)L.rhs, L.typ, L.n, h, dinv, col, 0, L.n, 0,
-                                                 L.n);
-                an_count(a, 1);
-            }
-    }
-    AN_CK(cudaGetLastError());
-    return HELM_OK;
+    st = an_vcycle<R>(a, l + 1, true);
+    if (st != HELM_OK) return st;
+    return an_tile(L.n) == 32 ? an_up<R, 32>(a, L, C) : an_up<R, 16>(a, L, C);
 }
 
 template <typename R>
@@ -1517,7 +1289,6 @@ helm_status an_solve(helm_annulus* a, const double2* data, double2* u, double to
         cudaStream_t q = a->ls;
         if (mode == 1) {
             for (int c = 0; c < a->cycles; ++c) {
-                if (c == 0) AN_CK(cudaMemsetAsync(L0.e, 0, total * sizeof(c2), q));
                 const helm_status st = an_vcycle<R>(a, 0, c == 0);
                 if (st != HELM_OK) return st;
             }
@@ -1627,7 +1398,6 @@ helm_status an_apply_inv(helm_annulus* a, int cycles)
     const long total = (long)(a->N + 1) * (a->N + 1);
     a->ls = a->stream;
     for (int c = 0; c < cycles; ++c) {
-        if (c == 0) AN_CK(cudaMemsetAsync(L0.e, 0, total * sizeof(c2), a->stream));
         const helm_status st = an_vcycle<R>(a, 0, c == 0);
         if (st != HELM_OK) return st;
     }
@@ -1885,12 +1655,6 @@ helm_status helm_annulus_create(helm_annulus** out, int n, double side, double h
         L.hi = hi;
         L.b0 = std::max(1, lo - AN_BAND);
         L.b1 = std::min(m - 1, hi + AN_BAND);
-        L.band_bytes = 0;
-        if (AN_BAND_SMEM) {
-            const AnRing g(L.b0, L.b1, L.lo, L.hi);
-            const size_t bb = prec == HELM_PREC_FP64 ? an_band_bytes<double>(g) : an_band_bytes<float>(g);
-            if (bb <= AN_SMEM_MAX && g.total() <= 1024 * AN_BAND_PT) L.band_bytes = bb;
-        }
         a->lev.push_back(L);
     }
     if (a->lev.size() < 2) return fail(HELM_EINVAL);
@@ -1898,41 +1662,14 @@ helm_status helm_annulus_create(helm_annulus** out, int n, double side, double h
     const int top = prec == HELM_PREC_FP64 ? AN_TAIL_TOP_D : AN_TAIL_TOP_F;
     for (int l = 0; l < (int)a->lev.size(); ++l)
         if (a->lev[l].n <= top) { a->t0 = l; break; }
-    if (a->t0 >= 0 && (int)a->lev.size() - a->t0 <= AN_TAIL_MAX) {
-        int ns[AN_TAIL_MAX];
-        const int L = (int)a->lev.size() - a->t0;
-        for (int i = 0; i < L; ++i) ns[i] = a->lev[a->t0 + i].n;
-        a->tail_bytes = (prec == HELM_PREC_FP64) ? an_tail_bytes<double>(ns, L) : an_tail_bytes<float>(ns, L);
-        const cudaError_t e = (prec == HELM_PREC_FP64)
-            ? cudaFuncSetAttribute(k_an_tail<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)a->tail_bytes)
-            : cudaFuncSetAttribute(k_an_tail<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)a->tail_bytes);
-        if (e != cudaSuccess) a->t0 = -1;      // no tail: per-level launches all the way down
-        cudaGetLastError();
-    } else {
-        a->t0 = -1;
-    }
+    if (a->t0 < 0 || (int)a->lev.size() - a->t0 > AN_TAIL_MAX) return fail(HELM_EUNSUPPORTED);
     {
-        const size_t dmax = (prec == HELM_PREC_FP64) ? an_down_bytes<double>(8) : an_down_bytes<float>(8);
-        const size_t umax = (prec == HELM_PREC_FP64) ? an_win_bytes<double>(an_up_sw(8)) : an_win_bytes<float>(an_up_sw(8));
-        cudaError_t e1, e2;
-        if (prec == HELM_PREC_FP64) {
-            e1 = cudaFuncSetAttribute(k_an_down<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dmax);
-            e2 = cudaFuncSetAttribute(k_an_up<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)umax);
-        } else {
-            e1 = cudaFuncSetAttribute(k_an_down<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dmax);
-            e2 = cudaFuncSetAttribute(k_an_up<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)umax);
+        const bool d = prec == HELM_PREC_FP64;
+        const cudaError_t e = d ? an_attrs<double>() : an_attrs<float>();
+        if (e != cudaSuccess) {
+            note_error(cudaGetErrorString(e));
+            return fail(HELM_ECUDA);
         }
-        if (e1 != cudaSuccess || e2 != cudaSuccess) return fail(HELM_ECUDA);
-        // in FP64 the windows' redundant halo sweeps cost more than the launches they save
-        a->tiles = AN_TILES && prec == HELM_PREC_MIXED;
-    }
-    size_t band_max = 0;
-    for (const auto& L : a->lev) band_max = std::max(band_max, L.band_bytes);
-    if (band_max) {
-        const cudaError_t e = (prec == HELM_PREC_FP64)
-            ? cudaFuncSetAttribute(k_an_band_s<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)band_max)
-            : cudaFuncSetAttribute(k_an_band_s<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)band_max);
-        if (e != cudaSuccess) return fail(HELM_ECUDA);
     }
     const long total = (long)(n + 1) * (n + 1);
     a->nblk = grid_for(total);
@@ -1955,7 +1692,7 @@ helm_status helm_annulus_destroy(helm_annulus* a)
     if (!a) return HELM_EINVAL;
     if (a->stream) cudaStreamSynchronize(a->stream);
     for (void* p : a->allocs) cudaFree(p);
-    if (a->Ainv) cudaFree(a->Ainv);
+    if (a->At) cudaFree(a->At);
     if (a->h_part) cudaFreeHost(a->h_part);
     if (a->stream) cudaStreamDestroy(a->stream);
     if (a->cap) cudaStreamDestroy(a->cap);
@@ -1973,15 +1710,23 @@ helm_status helm_annulus_set_shift(helm_annulus* a, double alpha)
     std::vector<double> inv;
     std::vector<int> map;
     if (!an_coarse_inverse(t, C.n, C.h, a->sigma, inv, map)) return HELM_EINVAL;
-    if (a->Ainv) cudaFree(a->Ainv);
-    a->Ainv = nullptr;
-    a->m = (int)map.size();
+    if (a->At) cudaFree(a->At);
+    a->At = nullptr;
+    const int m = (int)map.size();
+    a->m = m;
     void* p = nullptr;
     if (cudaMalloc(&p, inv.size() * sizeof(double) + map.size() * sizeof(int)) != cudaSuccess) return HELM_ENOMEM;
-    a->Ainv = (double*)p;
-    a->map = (int*)(a->Ainv + inv.size());
-    AN_CK(cudaMemcpy(a->Ainv, inv.data(), inv.size() * sizeof(double), cudaMemcpyHostToDevice));
+    a->At = (double*)p;
+    a->map = (int*)(a->At + inv.size());
+    std::vector<double> at(inv.size());
+    for (int r = 0; r < m; ++r)
+        for (int c = 0; c < m; ++c) at[(size_t)c * m + r] = inv[(size_t)r * m + c];
+    AN_CK(cudaMemcpy(a->At, at.data(), at.size() * sizeof(double), cudaMemcpyHostToDevice));
     AN_CK(cudaMemcpy(a->map, map.data(), map.size() * sizeof(int), cudaMemcpyHostToDevice));
+    int ns[AN_TAIL_MAX];
+    const int L = (int)a->lev.size() - a->t0;
+    for (int i = 0; i < L; ++i) ns[i] = a->lev[a->t0 + i].n;
+    a->tail_bytes = a->prec == HELM_PREC_FP64 ? an_tail_bytes<double>(ns, L, m) : an_tail_bytes<float>(ns, L, m);
     return HELM_OK;
 }
 
