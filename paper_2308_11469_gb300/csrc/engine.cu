@@ -211,6 +211,14 @@ struct Engine {
     int* d_ctrl = nullptr;                     // [0] steps done, [1] step budget, [2] go, [3] arrivals, [4] launch's steps
     int* h_ctrl = nullptr;                     // pinned mirror
     InstState* h_state = nullptr;              // pinned mirror (cap entries)
+    // behind it: a plan's solve leaves its histories there (relres, then increments from
+    // HIST_OUT + 1), when it made at most HIST_OUT steps
+    static constexpr int HIST_OUT = 1024;
+    double* h_hist() const { return reinterpret_cast<double*>(h_state + cap); }
+    // what instance 0's device descriptor and state hold for standalone cycles (an active
+    // state at step 0): repeated cycles upload nothing
+    InstDesc vc_desc{};
+    bool vc_ready = false;
     // page-locked staging of a starting instance's descriptor and state (a copy from
     // pageable memory would wait for the stream; a slot is restaged only after its previous
     // instance retired, behind a stream synchronisation)
@@ -328,7 +336,7 @@ struct Engine {
         InstState* nh = nullptr;
         HELM_CK(cudaMalloc(&nd, sizeof(InstDesc) * nc));
         HELM_CK(cudaMalloc(&ns, sizeof(InstState) * nc));
-        HELM_CK(cudaMallocHost(&nh, sizeof(InstState) * nc));
+        HELM_CK(cudaMallocHost(&nh, sizeof(InstState) * nc + (2 * HIST_OUT + 1) * sizeof(double)));
         InstDesc* hd = nullptr;
         InstState* hs = nullptr;
         HELM_CK(cudaMallocHost(&hd, sizeof(InstDesc) * nc));
@@ -941,28 +949,28 @@ struct Engine {
         return HELM_OK;
     }
 
-    // Run outer steps until every active instance has finished or `budget` steps ran.
-    // Returns the number of steps executed (read back after the stream drains).
-    helm_status run(cudaStream_t s, int budget, int* steps_done)
+    // A plan's solve, on its single instance: descriptor and state as kernel arguments, all
+    // outer steps in one launch, results through page-locked memory, one synchronisation
+    // (the caller's).
+    helm_status solve(cudaStream_t s)
     {
-        helm_status st = prepare();
-        if (st != HELM_OK) return st;
-        h_ctrl[0] = 0;
-        h_ctrl[1] = budget > 0 ? budget : INT_MAX;
-        h_ctrl[2] = 1;
-        h_ctrl[3] = 0;
-        HELM_CK(cudaMemcpyAsync(d_ctrl, h_ctrl, 4 * sizeof(int), cudaMemcpyHostToDevice, s));
+        const Instance* in = slots[0];
+        vc_ready = false;
+        HELM_CK(launch_begin(in->d, d_desc, d_state, d_ctrl, s));
+        // the instance's tile list names instance 0; the last tile records relres_0 and the
+        // initial status
+        HELM_CK(launch_residual(D, prec, d_desc, d_state, in->d_res0, in->nres0, 0, s, nullptr, 0, 0, 0, 0,
+                                in->d.damp != 0.0 ? 1 : 0));
         if (small_cs) {
-            st = enqueue_step(s);
+            const helm_status st = enqueue_step(s);
             if (st != HELM_OK) return st;
         } else {
             HELM_CK(cudaGraphLaunch(exec, s));
         }
-        HELM_CK(cudaMemcpyAsync(h_ctrl, d_ctrl, 3 * sizeof(int), cudaMemcpyDeviceToHost, s));
-        HELM_CK(cudaMemcpyAsync(h_state, d_state, sizeof(InstState) * cap, cudaMemcpyDeviceToHost, s));
+        const long S = in->d.n + 2, count = (D == 3) ? S * S * S : S * S;
+        HELM_CK(launch_finish(in->d, d_state, count, h_state, h_hist(), HIST_OUT, s));
         HELM_CK(cudaStreamSynchronize(s));
-        if (steps_done) *steps_done = h_ctrl[0];
-        g_launches += step_launches(h_ctrl[0]);
+        g_launches += 3 + step_launches(h_state[0].it);
         return HELM_OK;
     }
 };
@@ -1348,24 +1356,17 @@ helm_status helm_solve_ex(helm_plan* p, const void* f, const void* g, void* u, d
     in.d.damp = p->damp;
     helm_status st = p->eng.prepare();
     if (st != HELM_OK) return st;
-    st = p->eng.start_instance(0, p->stream);
-    if (st != HELM_OK) return st;
-    int steps = 0;
-    st = p->eng.run(p->stream, 0, &steps);
+    st = p->eng.solve(p->stream);
     if (st != HELM_OK) return st;
     const InstState s = p->eng.h_state[0];
-    if (s.it & 1) HELM_CK(cudaMemcpyAsync(u, in.d.u[1], ub, cudaMemcpyDeviceToDevice, p->stream));
-    if (res_hist) HELM_CK(cudaMemcpyAsync(res_hist, in.d.hist, (s.it + 1) * sizeof(double),
-                                          cudaMemcpyDeviceToHost, p->stream));
-    if (einf_hist && s.it > 0)
-        HELM_CK(cudaMemcpyAsync(einf_hist, in.d.einf, s.it * sizeof(double), cudaMemcpyDeviceToHost,
-                                p->stream));
-    HELM_CK(cudaStreamSynchronize(p->stream));
-    // leave the slot idle so standalone V-cycles see a known state
-    InstState idle;
-    memset(&idle, 0, sizeof idle);
-    idle.status = HELM_ST_IDLE;
-    HELM_CK(cudaMemcpy(p->eng.d_state, &idle, sizeof idle, cudaMemcpyHostToDevice));
+    if (s.it <= Engine::HIST_OUT) {
+        const double* h = p->eng.h_hist();
+        if (res_hist) memcpy(res_hist, h, (s.it + 1) * sizeof(double));
+        if (einf_hist) memcpy(einf_hist, h + Engine::HIST_OUT + 1, s.it * sizeof(double));
+    } else {
+        if (res_hist) HELM_CK(cudaMemcpy(res_hist, in.d.hist, (s.it + 1) * sizeof(double), cudaMemcpyDeviceToHost));
+        if (einf_hist) HELM_CK(cudaMemcpy(einf_hist, in.d.einf, s.it * sizeof(double), cudaMemcpyDeviceToHost));
+    }
     if (iters) *iters = s.it;
     return (helm_status)s.status;
 }
@@ -1520,6 +1521,7 @@ helm_status helm_spectral_radius(helm_plan* p, int max_iters, double tol, int cy
     if (!p || max_iters < 1 || !(tol >= 0.0) || cycles < 1 || cycles > 64) return HELM_EINVAL;
     Engine& E = p->eng;
     const int pr = p->prec == HELM_PREC_FP64 ? 0 : 1;
+    E.vc_ready = false;
     // one V-cycle of the plan's schedule from the current iterate, on instance 0
     const int sc = E.cycles;
     E.cycles = 1;
@@ -1587,34 +1589,34 @@ helm_status poisson_vcycle(helm_plan* p, const void* rhs, void* e, int nu1, int 
     E.nu1 = nu1;
     E.nu2 = nu2;
     E.cycles = 1;
-    helm_status st = E.rebuild_plan();
-    E.nu1 = s1;
-    E.nu2 = s2;
+    // the launch plan of this schedule (kept beside the solves' plans)
+    E.dirty = true;
+    helm_status st = E.prepare_plan();
     E.cycles = sc;
     E.dirty = true;
-    E.plan_sig.clear();
-    E.graph_sig.clear();
+    auto restore = [&]() { E.nu1 = s1; E.nu2 = s2; };
+    if (st != HELM_OK) { restore(); return st; }
+    if (!E.vc_ready || memcmp(&E.vc_desc, &p->inst.d, sizeof(InstDesc)) != 0) {
+        InstState act;
+        memset(&act, 0, sizeof act);
+        act.status = HELM_ST_ACTIVE;
+        if (cudaMemcpyAsync(E.d_desc, &p->inst.d, sizeof(InstDesc), cudaMemcpyHostToDevice, p->stream) != cudaSuccess ||
+            cudaMemcpyAsync(E.d_state, &act, sizeof act, cudaMemcpyHostToDevice, p->stream) != cudaSuccess) {
+            restore();
+            HELM_CK(cudaGetLastError());
+            return HELM_ECUDA;
+        }
+        memcpy(&E.vc_desc, &p->inst.d, sizeof(InstDesc));
+        E.vc_ready = true;
+    }
+    const int pr = p->prec == HELM_PREC_FP64 ? 0 : 1;
+    if (launch_pack(p->D, pr, E.d_desc, 0, p->n, rhs, e, p->stream) != cudaSuccess) st = HELM_ECUDA;
+    if (st == HELM_OK) st = E.enqueue(E.vcyc_plain, p->stream, false);
+    restore();
     if (st != HELM_OK) return st;
-    InstState act;
-    memset(&act, 0, sizeof act);
-    act.status = HELM_ST_ACTIVE;
-    HELM_CK(cudaMemcpyAsync(E.d_desc, &p->inst.d, sizeof(InstDesc), cudaMemcpyHostToDevice, p->stream));
-    HELM_CK(cudaMemcpyAsync(E.d_state, &act, sizeof act, cudaMemcpyHostToDevice, p->stream));
-    HELM_CK(launch_pack(p->D, p->prec == HELM_PREC_FP64 ? 0 : 1, E.d_desc, 0, p->n, rhs, 1, p->stream));
-    HELM_CK(launch_pack(p->D, p->prec == HELM_PREC_FP64 ? 0 : 1, E.d_desc, 0, p->n, e, 0, p->stream));
-    E.nu1 = nu1;
-    E.nu2 = nu2;
-    st = E.enqueue(E.vcyc_plain, p->stream, false);
-    E.nu1 = s1;
-    E.nu2 = s2;
-    if (st != HELM_OK) return st;
-    HELM_CK(launch_unpack(p->D, p->prec == HELM_PREC_FP64 ? 0 : 1, E.d_desc, 0, p->n, e, p->stream));
-    InstState idle;
-    memset(&idle, 0, sizeof idle);
-    idle.status = HELM_ST_IDLE;
-    HELM_CK(cudaMemcpyAsync(E.d_state, &idle, sizeof idle, cudaMemcpyHostToDevice, p->stream));
+    HELM_CK(launch_unpack(p->D, pr, E.d_desc, 0, p->n, e, p->stream));
     HELM_CK(cudaStreamSynchronize(p->stream));
-    g_launches += E.vcyc_plain.size() + 3;
+    g_launches += E.vcyc_plain.size() + 2;
     return HELM_OK;
 }
 

@@ -164,6 +164,12 @@ struct WsInit {
     int tx, ty, tz, pad;
 };
 cudaError_t launch_init_workspaces(const WsInit* recs, int count, cudaStream_t s);
+// start and end of a plan's solve (one instance): descriptor, state, step control ctrl[0..3]
+// and wall rings from the host's d; state and histories (of up to cap steps) to page-locked
+// host memory and the last iterate (count values) to the caller's buffer
+cudaError_t launch_begin(const InstDesc& d, InstDesc* dst, InstState* st, int* ctrl, cudaStream_t s);
+cudaError_t launch_finish(const InstDesc& d, const InstState* st, long count, InstState* h_st, double* h_hist, int cap,
+                          cudaStream_t s);
 // u[0] and u[1] rings := g ring
 cudaError_t launch_set_ring(int D, const InstDesc* insts, int inst, int n, cudaStream_t s);
 // the same for the m instances insts[slots[j]] (device list), all of size n
@@ -171,8 +177,8 @@ cudaError_t launch_set_ring_many(int D, const InstDesc* insts, const int* slots,
 // the residual tiles (tx x ty x tz each) of instances slots[0 .. m) into items, in order
 cudaError_t launch_fill_res_many(ResItem* items, const int* slots, int m, int tx, int ty, int tz, cudaStream_t s);
 // interior tight <-> level-0 padded/pitched, inner precision
-cudaError_t launch_pack(int D, int prec, const InstDesc* insts, int inst, int n,
-                        const void* src, int which /*0 = e, 1 = rhs*/, cudaStream_t s);
+cudaError_t launch_pack(int D, int prec, const InstDesc* insts, int inst, int n, const void* rhs, const void* e,
+                        cudaStream_t s);
 cudaError_t launch_unpack(int D, int prec, const InstDesc* insts, int inst, int n,
                           void* dst, cudaStream_t s);
 

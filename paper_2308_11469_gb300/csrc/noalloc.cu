@@ -190,8 +190,7 @@ extern "C" helm_status poisson_vcycle_noalloc(int ndim, int n, double h, int pre
     NA_CK(cudaMemsetAsync(base + OFF_LEVELS, 0, off - OFF_LEVELS, sm));
     k_noalloc_header<<<1, 256, 0, sm>>>(header, base);
     NA_CK(cudaGetLastError());
-    NA_CK(launch_pack(D, pr, dd, 0, n, rhs, 1, sm));
-    NA_CK(launch_pack(D, pr, dd, 0, n, e, 0, sm));
+    NA_CK(launch_pack(D, pr, dd, 0, n, rhs, e, sm));
     auto pts = [&](int m) { return (D == 3) ? (long)m * m * m : (long)m * m; };
     if (fused) {
         for (int l = 0; l < lt; ++l)

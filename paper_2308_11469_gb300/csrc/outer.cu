@@ -775,9 +775,66 @@ __global__ void k_fill_res_many(ResItem* __restrict__ items, const int* __restri
     }
 }
 
+// Start of a plan's solve: its descriptor (a kernel argument: no copy from host memory), a
+// fresh state and the step control, and the wall ring of both iterate buffers.
+template <int D>
+__global__ void k_begin(const __grid_constant__ InstDesc d, InstDesc* __restrict__ dst, InstState* __restrict__ st,
+                        int* __restrict__ ctrl)
+{
+    pdl_wait();
+    if (blockIdx.x == 0) {
+        const int* src = reinterpret_cast<const int*>(&d);
+        for (int i = threadIdx.x; i < (int)(sizeof(InstDesc) / sizeof(int)); i += blockDim.x)
+            reinterpret_cast<int*>(dst)[i] = src[i];
+        if (threadIdx.x == 0) {
+            InstState s = {};
+            s.status = HELM_ST_ACTIVE;
+            *st = s;
+            ctrl[0] = 0;
+            ctrl[1] = 0x7fffffff;
+            ctrl[2] = 1;
+            ctrl[3] = 0;
+        }
+    }
+    // the ring face by face (edges more than once, with the same value)
+    const long S = d.n + 2, face = (D == 3) ? S * S : S, N1 = S - 1;
+    for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < 2 * D * face; t += (long)gridDim.x * blockDim.x) {
+        const long side = t / face, r = t - side * face, a = r % S, b = r / S, c = (side & 1) ? N1 : 0;
+        long q;
+        if (side < 2) q = (D == 3) ? (c * S + b) * S + a : c * S + a;
+        else if (side < 4) q = (D == 3) ? (b * S + c) * S + a : a * S + c;
+        else q = (b * S + a) * S + c;
+        const double2 v = d.g[q];
+        d.u[0][q] = v;
+        d.u[1][q] = v;
+    }
+}
+
+// End of a plan's solve: the state and (up to `cap` steps) the histories into page-locked host
+// memory, relres first, the increments from cap + 1, and the last iterate into the caller's
+// buffer when it lives in the library's.
+__global__ void __launch_bounds__(256)
+k_finish(const InstState* __restrict__ st, const double* __restrict__ hist, const double* __restrict__ einf,
+         double2* __restrict__ u0, const double2* __restrict__ u1, long count, InstState* h_st, double* h_hist, int cap)
+{
+    const int it = st->it;
+    if (blockIdx.x == 0) {
+        if (threadIdx.x == 0) *h_st = *st;
+        if (it <= cap)
+            for (int i = threadIdx.x; i <= it; i += blockDim.x) {
+                h_hist[i] = hist[i];
+                if (i < it) h_hist[cap + 1 + i] = einf[i];
+            }
+    }
+    if (it & 1)
+        for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < count; i += (long)gridDim.x * blockDim.x)
+            u0[i] = u1[i];
+}
+
+// interior tight rhs and e -> level 0
 template <int D, typename R>
-__global__ void k_pack(const InstDesc* __restrict__ insts, int inst, const void* __restrict__ src,
-                       int which)
+__global__ void k_pack(const InstDesc* __restrict__ insts, int inst, const void* __restrict__ rhs,
+                       const void* __restrict__ e)
 {
     pdl_wait();
     pdl_trigger();
@@ -786,14 +843,14 @@ __global__ void k_pack(const InstDesc* __restrict__ insts, int inst, const void*
     const LevelDesc L = I.lev[0];
     const int n = L.n;
     const long total = (D == 3) ? (long)n * n * n : (long)n * n;
-    c2* dst = (c2*)(which ? L.rhs : L.e);
-    const c2* s = (const c2*)src;
     for (long q = blockIdx.x * (long)blockDim.x + threadIdx.x; q < total;
          q += (long)gridDim.x * blockDim.x) {
         const int x = (int)(q % n) + 1;
         const int y = (int)((q / n) % n) + 1;
         const int z = (D == 3) ? (int)(q / ((long)n * n)) + 1 : 0;
-        dst[((D == 3) ? ((long)z * L.rows + y) : (long)y) * L.pitch + xslot<D>(x, L.pitch)] = s[q];
+        const long o = ((D == 3) ? ((long)z * L.rows + y) : (long)y) * L.pitch + xslot<D>(x, L.pitch);
+        ((c2*)L.rhs)[o] = ((const c2*)rhs)[q];
+        ((c2*)L.e)[o] = ((const c2*)e)[q];
     }
 }
 
@@ -1286,15 +1343,30 @@ cudaError_t launch_fill_res_many(ResItem* items, const int* slots, int m, int tx
     return cudaGetLastError();
 }
 
-cudaError_t launch_pack(int D, int prec, const InstDesc* insts, int inst, int n, const void* src,
-                        int which, cudaStream_t s)
+cudaError_t launch_pack(int D, int prec, const InstDesc* insts, int inst, int n, const void* rhs, const void* e,
+                        cudaStream_t s)
 {
     const long work = (D == 3) ? (long)n * n * n : (long)n * n;
     const int nb = blocks_for(work);
-    if (D == 2 && prec == 0) launch_k(k_pack<2, double>, dim3(nb), dim3(256), 0, s, insts, inst, src, which);
-    else if (D == 2) launch_k(k_pack<2, float>, dim3(nb), dim3(256), 0, s, insts, inst, src, which);
-    else if (prec == 0) launch_k(k_pack<3, double>, dim3(nb), dim3(256), 0, s, insts, inst, src, which);
-    else launch_k(k_pack<3, float>, dim3(nb), dim3(256), 0, s, insts, inst, src, which);
+    if (D == 2 && prec == 0) launch_k(k_pack<2, double>, dim3(nb), dim3(256), 0, s, insts, inst, rhs, e);
+    else if (D == 2) launch_k(k_pack<2, float>, dim3(nb), dim3(256), 0, s, insts, inst, rhs, e);
+    else if (prec == 0) launch_k(k_pack<3, double>, dim3(nb), dim3(256), 0, s, insts, inst, rhs, e);
+    else launch_k(k_pack<3, float>, dim3(nb), dim3(256), 0, s, insts, inst, rhs, e);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_begin(const InstDesc& d, InstDesc* dst, InstState* st, int* ctrl, cudaStream_t s)
+{
+    const long S = d.n + 2, work = (d.D == 3) ? 6 * S * S : 4 * S;
+    if (d.D == 2) launch_k(k_begin<2>, dim3(blocks_for(work)), dim3(256), 0, s, d, dst, st, ctrl);
+    else launch_k(k_begin<3>, dim3(blocks_for(work)), dim3(256), 0, s, d, dst, st, ctrl);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_finish(const InstDesc& d, const InstState* st, long count, InstState* h_st, double* h_hist, int cap,
+                          cudaStream_t s)
+{
+    k_finish<<<blocks_for(count), 256, 0, s>>>(st, d.hist, d.einf, d.u[0], d.u[1], count, h_st, h_hist, cap);
     return cudaGetLastError();
 }
 
