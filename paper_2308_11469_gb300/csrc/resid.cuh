@@ -4,6 +4,7 @@
 #include "launch.h"
 #include "fp_bits.cuh"
 #include "fixed_lap.cuh"
+#include "fixed_win.cuh"
 
 namespace helm {
 namespace {
@@ -290,22 +291,6 @@ __device__ __forceinline__ int fx_scale(int emax_raw)
 __device__ __forceinline__ longlong2 fx_fix2(double2 v, int emax)
 {
     return make_longlong2(fx_fix(v.x, emax), fx_fix(v.y, emax));
-}
-
-__device__ __forceinline__ int fx_exp2(double2 v) { return max(fx_exp(v.x), fx_exp(v.y)); }
-
-// largest of the threads' exponents (one shared word per warp; the caller's barrier
-// follows before any thread reads the result)
-template <int NT>
-__device__ __forceinline__ int block_max_exp(int ex, int* sx)
-{
-    ex = __reduce_max_sync(0xffffffffu, ex);
-    if ((threadIdx.x & 31) == 0) sx[threadIdx.x >> 5] = ex;
-    __syncthreads();
-    int m = sx[0];
-#pragma unroll
-    for (int w = 1; w < NT / 32; ++w) m = max(m, sx[w]);
-    return m;
 }
 
 // The residual window of a tile is its (TX + 2) x (TY + 2) nodes; its 1-node ring has

@@ -24,12 +24,48 @@
 #include "launch.h"
 #include "pdl.cuh"
 #include "sweep2d.cuh"
+#include "fixed_win.cuh"
+
+#include <type_traits>
 
 namespace helm {
 namespace {
 
 constexpr int NT = SW_NT;
 constexpr int NW = SW_NW;
+
+// half_sweep_flat / sweeps_flat on fixed-point planes (R0, R1: h^2 rhs)
+template <int W, int TX, int TY, int RING, int COLOR>
+__device__ __forceinline__ void half_sweep_fx(longlong2* E0, longlong2* E1, const longlong2* R0, const longlong2* R1,
+                                              int gx0, int gy0, int x0, int y0, int n)
+{
+    typedef Planes<W> PL;
+    constexpr int NX = (TX + 2 * RING) / 2, NY = TY + 2 * RING;
+    longlong2* __restrict__ Ec = COLOR ? E1 : E0;
+    const longlong2* __restrict__ Eo = COLOR ? E0 : E1;
+    const longlong2* __restrict__ Rc = COLOR ? R1 : R0;
+    const int xr = x0 - RING;
+    for (int q = threadIdx.x; q < NX * NY; q += NT) {
+        const int j = q / NX, i = q - j * NX;
+        const int gy = y0 - RING + j;
+        const int gx = xr + (((xr + gy) & 1) ^ COLOR) + 2 * i;
+        if (gy < 1 || gy > n || gx < 1 || gx > n) continue;
+        const int lx = gx - gx0, ly = gy - gy0;
+        const int o = PL::at(lx, ly);
+        Ec[o] = fx_gs(Eo[PL::at(lx - 1, ly)], Eo[PL::at(lx + 1, ly)], Eo[PL::at(lx, ly - 1)], Eo[PL::at(lx, ly + 1)],
+                      Rc[o]);
+    }
+}
+template <int W, int TX, int TY, int RING, int NS, int COLOR = 0>
+__device__ __forceinline__ void sweeps_fx(longlong2* E0, longlong2* E1, const longlong2* R0, const longlong2* R1,
+                                          int gx0, int gy0, int x0, int y0, int n)
+{
+    if constexpr (NS > 0) {
+        half_sweep_fx<W, TX, TY, RING, COLOR>(E0, E1, R0, R1, gx0, gy0, x0, y0, n);
+        __syncthreads();
+        sweeps_fx<W, TX, TY, RING - 1, NS - 1, COLOR ^ 1>(E0, E1, R0, R1, gx0, gy0, x0, y0, n);
+    }
+}
 
 template <typename R, int NU, int TX, int TY>
 __global__ void __launch_bounds__(NT)
@@ -86,6 +122,85 @@ k_down2d(const InstDesc* __restrict__ insts, const InstState* __restrict__ st,
         cp_async_elem<sizeof(c2)>((c ? R1 : R0) + o, gr + g, in);
     }
     cp_async_wait_all();
+    if constexpr (std::is_same<R, double>::value) {
+        // fixed point (fixed_win.cuh): each thread puts the words it staged on the window's
+        // scale, four times the largest value's (the residual of an iterate grown by nu1 sweeps
+        // is below 25 times it, a row of the full weighting four times that)
+        __shared__ int sx[NW];
+        const FxH2 hh(L.h);
+        int ex = 0;
+        if (sigma == 0.0)
+            for (int q = threadIdx.x; q < W * HH; q += NT) {
+                const int ly = q / W, lx = q - ly * W, o = PL::at(lx, ly);
+                const bool c = (lx + ly + cpar) & 1;
+                const int er = fx_exp2((c ? R1 : R0)[o]);
+                ex = max(ex, er ? er + hh.add : 0);
+                if (!zero) ex = max(ex, fx_exp2((c ? E1 : E0)[o]));
+            }
+        const int em = block_max_exp<NW * 32>(ex, sx) + 2;
+        if (sigma == 0.0 && hh.usable(em)) {
+            longlong2* const F0 = reinterpret_cast<longlong2*>(E0);
+            longlong2* const F1 = reinterpret_cast<longlong2*>(E1);
+            longlong2* const G0 = reinterpret_cast<longlong2*>(R0);
+            longlong2* const G1 = reinterpret_cast<longlong2*>(R1);
+            for (int q = threadIdx.x; q < W * HH; q += NT) {
+                const int ly = q / W, lx = q - ly * W, o = PL::at(lx, ly);
+                const bool c = (lx + ly + cpar) & 1;
+                (c ? G1 : G0)[o] = hh.q2((c ? R1 : R0)[o], em);
+                if (!zero) (c ? F1 : F0)[o] = fx_q2((c ? E1 : E0)[o], em);
+            }
+            __syncthreads();
+            sweeps_fx<W, TX, TY, 2 * NU + 1, 2 * NU>(F0, F1, G0, G1, gx0, gy0, x0, y0, n);
+            if (!(NU == 0 && zero)) {
+                c2* __restrict__ ge2 = (c2*)L.e2;
+                for (int q = threadIdx.x; q < TX * TY; q += NT) {
+                    const int ty = q / TX, tx = q - ty * TX, gx = x0 + tx, gy = y0 + ty;
+                    const int lx = tx + H, ly = ty + H;
+                    if (gx <= n && gy <= n)
+                        ge2[(size_t)gy * P + gx] = fx_d2((((lx + ly + cpar) & 1) ? F1 : F0)[PL::at(lx, ly)], em);
+                }
+                // h^2 residual on the tile plus a 1-node ring, in place of h^2 rhs
+                constexpr int NX = (TX + 2) / 2, NY = TY + 2;
+                for (int q = threadIdx.x; q < 2 * NX * NY; q += NT) {
+                    const int color = q >= NX * NY, qq = q - color * (NX * NY);
+                    const int jy = qq / NX, i = qq - jy * NX;
+                    const int gy = y0 - 1 + jy;
+                    const int gx = x0 - 1 + (((x0 - 1 + gy) & 1) ^ color) + 2 * i;
+                    if (gy < 1 || gy > n || gx < 1 || gx > n) continue;
+                    const longlong2* __restrict__ Fo = color ? F0 : F1;
+                    const int ly = gy - gy0, lx = gx - gx0, o = PL::at(lx, ly);
+                    const longlong2 f = (color ? F1 : F0)[o];
+                    const longlong2 a = Fo[PL::at(lx - 1, ly)], b = Fo[PL::at(lx + 1, ly)];
+                    const longlong2 u = Fo[PL::at(lx, ly - 1)], d = Fo[PL::at(lx, ly + 1)];
+                    longlong2* const r = (color ? G1 : G0) + o;
+                    *r = make_longlong2(r->x - (((a.x + b.x) + (u.x + d.x)) - 4 * f.x),
+                                        r->y - (((a.y + b.y) + (u.y + d.y)) - 4 * f.y));
+                }
+                __syncthreads();
+            }
+            // full weighting: rows first, each rounded to a quarter
+            c2* __restrict__ cr = (c2*)C.rhs;
+            const int nc = C.n, Xa = (x0 + 1) >> 1, Ya = (y0 + 1) >> 1, PC = C.pitch;
+            for (int q = threadIdx.x; q < (TX / 2) * (TY / 2); q += NT) {
+                const int cy = q / (TX / 2), cx = q - cy * (TX / 2), Y = Ya + cy, X = Xa + cx;
+                if (Y > nc || X > nc) continue;
+                const int lx = 2 * X - gx0, ly = 2 * Y - gy0;
+                longlong2 t[3];
+#pragma unroll
+                for (int dy = -1; dy <= 1; ++dy) {
+                    const bool c = (lx + ly + dy + cpar) & 1;
+                    const longlong2 m = (c ? G1 : G0)[PL::at(lx, ly + dy)];
+                    const longlong2 a = (c ? G0 : G1)[PL::at(lx - 1, ly + dy)];
+                    const longlong2 b = (c ? G0 : G1)[PL::at(lx + 1, ly + dy)];
+                    t[dy + 1] = make_longlong2(fx_shr<2>((a.x + b.x) + 2 * m.x), fx_shr<2>((a.y + b.y) + 2 * m.y));
+                }
+                // (t0 + 2 t1 + t2) / 4 of h^2 times the coarse rhs
+                const longlong2 v = make_longlong2((t[0].x + t[2].x) + 2 * t[1].x, (t[0].y + t[2].y) + 2 * t[1].y);
+                cr[(size_t)Y * PC + X] = hh.over(v, em - 2);
+            }
+            return;
+        }
+    }
     __syncthreads();
     const R h2 = (R)(L.h * L.h);
     const R dinv = (R)L.dinv;                      // 1 / (4 + sigma h^2)
@@ -237,6 +352,65 @@ k_up2d(const InstDesc* __restrict__ insts, const InstState* __restrict__ st,
         cp_async_elem<sizeof(c2)>((c ? R1 : R0) + o, gr + g, in);
     }
     cp_async_wait_all();
+    if constexpr (std::is_same<R, double>::value) {
+        // fixed point (fixed_win.cuh): after the correction the iterate is at most twice the
+        // window's largest value, after nu2 sweeps at most 2 + nu2 / 2 times it
+        __shared__ int sx[NW];
+        const FxH2 hh(L.h);
+        int ex = 0;
+        const bool plain = L.dinv == 0.25;         // no shift
+        if (plain) {
+            for (int q = threadIdx.x; q < CW * CH; q += NT) ex = max(ex, fx_exp2(Cs[q]));
+            for (int q = threadIdx.x; q < W * HH; q += NT) {
+                const int ly = q / W, lx = q - ly * W, o = PL::at(lx, ly);
+                const bool c = (lx + ly + cpar) & 1;
+                const int er = fx_exp2((c ? R1 : R0)[o]);
+                ex = max(ex, er ? er + hh.add : 0);
+                if (!e2z) ex = max(ex, fx_exp2((c ? E1 : E0)[o]));
+            }
+        }
+        const int em = block_max_exp<NW * 32>(ex, sx);
+        if (plain && hh.usable(em)) {
+            longlong2* const F0 = reinterpret_cast<longlong2*>(E0);
+            longlong2* const F1 = reinterpret_cast<longlong2*>(E1);
+            longlong2* const G0 = reinterpret_cast<longlong2*>(R0);
+            longlong2* const G1 = reinterpret_cast<longlong2*>(R1);
+            longlong2* const Fc = reinterpret_cast<longlong2*>(Cs);
+            for (int q = threadIdx.x; q < CW * CH; q += NT) Fc[q] = fx_q2(Cs[q], em);
+            for (int q = threadIdx.x; q < W * HH; q += NT) {
+                const int ly = q / W, lx = q - ly * W, o = PL::at(lx, ly);
+                const bool c = (lx + ly + cpar) & 1;
+                (c ? G1 : G0)[o] = hh.q2((c ? R1 : R0)[o], em);
+                if (!e2z) (c ? F1 : F0)[o] = fx_q2((c ? E1 : E0)[o], em);
+            }
+            __syncthreads();
+            // with sweeps to come colour 0 is overwritten unread: colour 1 alone
+            constexpr int NX = NU ? W / 2 : W;
+            for (int q = threadIdx.x; q < NX * HH; q += NT) {
+                const int ly = q / NX, i = q - ly * NX;
+                const int lx = NU ? 2 * i + ((ly + cpar + 1) & 1) : i;
+                const int gx = gx0 + lx, gy = gy0 + ly;
+                if (gy < 1 || gy > n || gx < 1 || gx > n) continue;
+                const int Y0 = (gy >> 1) - cy0, Y1 = ((gy + 1) >> 1) - cy0;
+                const int X0 = (gx >> 1) - cx0, X1 = ((gx + 1) >> 1) - cx0;
+                const longlong2 a = Fc[Y0 * CW + X0], b = Fc[Y0 * CW + X1];
+                const longlong2 c = Fc[Y1 * CW + X0], d = Fc[Y1 * CW + X1];
+                longlong2* const p = (((lx + ly + cpar) & 1) ? F1 : F0) + PL::at(lx, ly);
+                p->x += fx_shr<2>((a.x + b.x) + (c.x + d.x));
+                p->y += fx_shr<2>((a.y + b.y) + (c.y + d.y));
+            }
+            __syncthreads();
+            sweeps_fx<W, TX, TY, 2 * NU - 1, 2 * NU>(F0, F1, G0, G1, gx0, gy0, x0, y0, n);
+            c2* __restrict__ ge = (c2*)L.e;
+            for (int q = threadIdx.x; q < TX * TY; q += NT) {
+                const int ty = q / TX, tx = q - ty * TX, gx = x0 + tx, gy = y0 + ty;
+                const int lx = tx + H, ly = ty + H;
+                if (gx <= n && gy <= n)
+                    ge[(size_t)gy * P + gx] = fx_d2((((lx + ly + cpar) & 1) ? F1 : F0)[PL::at(lx, ly)], em);
+            }
+            return;
+        }
+    }
     __syncthreads();
     // correction: e2 + multilinear interpolation of the coarse iterate (interior nodes)
     for (int q = threadIdx.x; q < W * HH; q += NT) {
@@ -300,6 +474,28 @@ k_restrict_rhs2d(const InstDesc* __restrict__ insts, const InstState* __restrict
     const c2* __restrict__ gr = (const c2*)lev_rhs(L, item.level, sv.it);
     const size_t P = L.pitch;
     const size_t o = (size_t)(2 * Y) * P + 2 * X;
+    if constexpr (std::is_same<R, double>::value) {
+        // fixed point (fixed_win.cuh) on the nine values' own scale
+        c2 r[9];
+        int ex = 0;
+#pragma unroll
+        for (int k = 0; k < 9; ++k) {
+            r[k] = __ldg(gr + (o + (ptrdiff_t)(k / 3 - 1) * (ptrdiff_t)P + (k % 3 - 1)));
+            ex = max(ex, fx_exp2(r[k]));
+        }
+        if (fx_usable(ex)) {
+            longlong2 s = make_longlong2(0, 0);
+#pragma unroll
+            for (int k = 0; k < 9; ++k) {
+                const longlong2 f = fx_q2(r[k], ex);
+                const int w = (k / 3 == 1) + (k % 3 == 1);
+                s.x += f.x << w;
+                s.y += f.y << w;
+            }
+            ((c2*)C.rhs)[(size_t)Y * C.pitch + X] = fx_d2(s, ex - 4);
+            return;
+        }
+    }
     R ax = 0, ay = 0;
 #pragma unroll
     for (int dy = -1; dy <= 1; ++dy) {
@@ -373,6 +569,50 @@ k_restrict2_rhs2d(const InstDesc* __restrict__ insts, const InstState* __restric
                      : "memory");
     }
     asm volatile("cp.async.wait_all;\n" ::: "memory");
+    if constexpr (std::is_same<R, double>::value) {
+        // fixed point (fixed_win.cuh): the weights' sums are exact, level l + 1 is kept rounded
+        // to its scale for level l + 2
+        __shared__ int sx[R2NT / 32];
+        int ex = 0;
+        for (int q = threadIdx.x; q < R2W0 * CPR; q += R2NT) ex = max(ex, fx_exp2(W0[q]));
+        const int em = block_max_exp<R2NT>(ex, sx);
+        if (fx_usable(em)) {
+            longlong2* const F0 = reinterpret_cast<longlong2*>(W0);
+            longlong2* const F1 = reinterpret_cast<longlong2*>(W1);
+            for (int q = threadIdx.x; q < R2W0 * CPR; q += R2NT) F0[q] = fx_q2(W0[q], em);
+            __syncthreads();
+            auto weigh = [](const longlong2* w, int pitch) -> longlong2 {      // centre *w
+                longlong2 s = make_longlong2(0, 0);
+#pragma unroll
+                for (int dy = -1; dy <= 1; ++dy) {
+                    const longlong2 a = w[dy * pitch - 1], m = w[dy * pitch], b = w[dy * pitch + 1];
+                    const long long tx = (a.x + b.x) + 2 * m.x, ty = (a.y + b.y) + 2 * m.y;
+                    s.x += dy ? tx : 2 * tx;
+                    s.y += dy ? ty : 2 * ty;
+                }
+                return s;
+            };
+            c2* __restrict__ g1 = (c2*)L1.rhs;
+            const int P1 = L1.pitch;
+            for (int q = threadIdx.x; q < R2W1 * R2W1; q += R2NT) {
+                const int y1 = q / R2W1, x1 = q % R2W1;
+                const int X1 = 2 * X2a - 1 + x1, Y1 = 2 * Y2a - 1 + y1;
+                longlong2 s = make_longlong2(0, 0);
+                if (X1 <= n1 && Y1 <= n1) {
+                    s = weigh(F0 + (2 * y1 + 2) * R2W0 + 2 * x1 + 2, R2W0);
+                    if (x1 < 2 * R2T && y1 < 2 * R2T) g1[(size_t)Y1 * P1 + X1] = fx_d2(s, em - 4);
+                }
+                F1[q] = make_longlong2(fx_shr<4>(s.x), fx_shr<4>(s.y));
+            }
+            __syncthreads();
+            c2* __restrict__ g2 = (c2*)L2.rhs;
+            const int x2 = threadIdx.x % R2T, y2 = threadIdx.x / R2T;
+            const int X2 = X2a + x2, Y2 = Y2a + y2;
+            if (y2 < R2T && X2 <= n2 && Y2 <= n2)
+                g2[(size_t)Y2 * L2.pitch + X2] = fx_d2(weigh(F1 + (2 * y2 + 1) * R2W1 + 2 * x2 + 1, R2W1), em - 4);
+            return;
+        }
+    }
     __syncthreads();
     // level l+1 window: node (2 X2a - 1 + x1, 2 Y2a - 1 + y1); its fine node (2 X1 + dx, ...)
     // is window element (2 x1 + 2 + dx, 2 y1 + 2 + dy)
