@@ -24,6 +24,7 @@
 #include "launch.h"
 #include "pdl.cuh"
 #include "tail_levels.cuh"
+#include "fixed_win.cuh"
 
 namespace helm {
 namespace {
@@ -36,8 +37,102 @@ __device__ float g_xtab[XTAB_FLOATS];
 __device__ float g_ytab[YTAB_FLOATS];
 __device__ double g_ztab[ZTAB_DOUBLES];
 
+// FP64 tail of level 31 in fixed point (fixed_win.cuh), a thread per node: sweeps, residual,
+// full weighting and correction as integer sums on the level's scale, level 15 solved exactly
+// in FP64.  The ascent's scale also covers level 15's solution.  false (nothing written): a
+// value is out of the scales' range, the FP64 code takes over.
+__device__ __noinline__ bool tail_fx31(const LevelDesc& L0, const double2* __restrict__ gr, bool le, int nu1, int nu2,
+                                       unsigned char* smem)
+{
+    constexpr int N = 31, S = N + 2, NC = ZN, SC = NC + 2;
+    __shared__ int sx[TNT / 32];
+    longlong2* const F = reinterpret_cast<longlong2*>(smem);             // iterate, zero ring
+    longlong2* const G = F + S * S;                                      // h^2 residual
+    double2* const Ec = reinterpret_cast<double2*>(G + S * S);           // level 15 (ix layout)
+    double2* const Rc = Ec + SC * SC;
+    longlong2* const Fc = G;                                             // (the residual is dead by then)
+    double* const scr = reinterpret_cast<double*>(Rc + SC * SC);
+    static_assert(((size_t)2 * S * S + 2 * SC * SC) * 16 + ZSCR_DOUBLES * 8 <= tail_bytes<2, double, N>(), "shared memory");
+    const int t = threadIdx.x;
+    const bool own = t < N * N;
+    const int y = t / N + 1, x = t % N + 1, o = y * S + x;
+    double2* __restrict__ ge = (double2*)L0.e;
+    const FxH2 hh(L0.h);
+    double2 r = make_double2(0.0, 0.0), e = r;
+    if (own) {
+        r = gr[(size_t)y * L0.pitch + x];
+        if (le) e = ge[(size_t)y * L0.pitch + x];
+    }
+    for (int i = t; i < ZTAB_DOUBLES; i += TNT) scr[i] = g_ztab[i];
+    for (int i = t; i < S * S; i += TNT) F[i] = make_longlong2(0, 0);
+    for (int i = t; i < SC * SC; i += TNT) Ec[i] = make_double2(0.0, 0.0);
+    const int er = fx_exp2(r);
+    const int em = block_max_exp<TNT>(max(er ? er + hh.add : 0, fx_exp2(e)), sx) + 2;
+    if (!hh.usable(em)) return false;
+    longlong2 g = make_longlong2(0, 0);
+    if (own) {
+        g = hh.q2(r, em);
+        if (le) F[o] = fx_q2(e, em);
+    }
+    __syncthreads();
+    const int color = (x + y) & 1;
+    auto sweeps = [&](int nu) {
+        for (int s = 0; s < 2 * nu; ++s) {
+            if (own && color == (s & 1)) F[o] = fx_gs(F[o - 1], F[o + 1], F[o - S], F[o + S], g);
+            __syncthreads();
+        }
+    };
+    sweeps(nu1);
+    if (own) {
+        longlong2 q = g;
+        if (nu1 > 0 || le) {
+            const longlong2 c = F[o], a = F[o - 1], b = F[o + 1], u = F[o - S], d = F[o + S];
+            q.x -= ((a.x + b.x) + (u.x + d.x)) - 4 * c.x;
+            q.y -= ((a.y + b.y) + (u.y + d.y)) - 4 * c.y;
+        }
+        G[o] = q;
+    }
+    __syncthreads();
+    const int Y = t / NC + 1, X = t % NC + 1, oc = Y * SC + ix<NC>(X);
+    if (t < NC * NC) {
+        longlong2 w[3];
+#pragma unroll
+        for (int dy = -1; dy <= 1; ++dy) {
+            const longlong2* p = G + (2 * Y + dy) * S + 2 * X;
+            w[dy + 1] = make_longlong2(fx_shr<2>((p[-1].x + p[1].x) + 2 * p[0].x),
+                                       fx_shr<2>((p[-1].y + p[1].y) + 2 * p[0].y));
+        }
+        Rc[oc] = hh.over(make_longlong2((w[0].x + w[2].x) + 2 * w[1].x, (w[0].y + w[2].y) + 2 * w[1].y), em - 2);
+    }
+    __syncthreads();
+    z_solve(Ec, Rc, scr, 2.0 * L0.h, 0.0);
+    const double2 ec = t < SC * SC ? Ec[t] : make_double2(0.0, 0.0);     // ring and layout alike
+    const int ea = max(em, block_max_exp<TNT>(fx_exp2(ec), sx) + 2);
+    if (!hh.usable(ea)) return false;
+    if (t < SC * SC) Fc[t] = fx_q2(ec, ea);
+    if (own) {
+        // from the descent's scale to the ascent's
+        const int d = min(ea - em, 62);
+        auto down = [d](long long v) { return d == 0 ? v : (v + ((1ll << (d - 1)) - 1) + ((v >> d) & 1)) >> d; };
+        g = make_longlong2(down(g.x), down(g.y));
+        const longlong2 f = F[o];
+        F[o] = make_longlong2(down(f.x), down(f.y));
+    }
+    __syncthreads();
+    if (own && (nu2 == 0 || color == 1)) {       // with sweeps to come colour 0 is overwritten unread
+        const int Y0 = y >> 1, Y1 = (y + 1) >> 1, X0 = ix<NC>(x >> 1), X1 = ix<NC>((x + 1) >> 1);
+        const longlong2 a = Fc[Y0 * SC + X0], b = Fc[Y0 * SC + X1], c = Fc[Y1 * SC + X0], d = Fc[Y1 * SC + X1];
+        F[o].x += fx_shr<2>((a.x + b.x) + (c.x + d.x));
+        F[o].y += fx_shr<2>((a.y + b.y) + (c.y + d.y));
+    }
+    __syncthreads();
+    sweeps(nu2);
+    if (own) ge[(size_t)y * L0.pitch + x] = fx_d2(F[o], ea);
+    return true;
+}
+
 template <int D, typename R, int N0>
-__global__ void __launch_bounds__(TNT)
+__global__ void __launch_bounds__(TNT, 1)
 k_tail(const InstDesc* __restrict__ insts, const InstState* __restrict__ st,
        const MgItem* __restrict__ items, int nu1, int nu2, int load_e)
 {
@@ -52,6 +147,11 @@ k_tail(const InstDesc* __restrict__ insts, const InstState* __restrict__ st,
     const InstState sv = st[item.inst];
     if (sv.status != HELM_ST_ACTIVE) return;
     if (L0.n != N0) return;                       // launched for another tail size
+    if constexpr (D == 2 && std::is_same<R, double>::value && N0 == 31) {
+        if (sigma == 0.0 &&
+            tail_fx31(L0, (const double2*)lev_rhs(L0, item.level, sv.it), load_e && item.level == 0, nu1, nu2, smem_raw))
+            return;
+    }
     constexpr int TOT = tail_elems<D, N0>();
     constexpr int S = N0 + 2;
     constexpr int ROWS = (D == 3) ? N0 * N0 : N0;

@@ -89,6 +89,12 @@ template <int NWARPS> __device__ __forceinline__ void tsync() {
 
 template <typename T> __device__ __forceinline__ T cz() { T v; v.x = 0; v.y = 0; return v; }
 
+// FP64 phases number their nodes over all the threads: a warp's FP64 instruction holds its
+// sub-core's pipe for 64 clocks however few lanes it serves, so a warp per row of 15 or 3
+// nodes wastes most of them (3D tail of level 7: 90 us).
+template <typename R> constexpr bool t_flat() { return std::is_same<R, double>::value; }
+template <int NWARPS> __device__ __forceinline__ int t_id() { return NWARPS == 1 ? (int)(threadIdx.x & 31) : (int)threadIdx.x; }
+
 template <int D, typename R, int N, int NWARPS>
 __device__ __forceinline__ void t_sweep(typename C2<R>::T* E, const typename C2<R>::T* Rr, R h2,
                                         R dinv, int color)
@@ -96,13 +102,8 @@ __device__ __forceinline__ void t_sweep(typename C2<R>::T* E, const typename C2<
     typedef typename C2<R>::T c2;
     constexpr int S = N + 2;
     constexpr int ROWS = (D == 3) ? N * N : N;
-    const int lane = threadIdx.x & 31;
-    for (int r = threadIdx.x >> 5; r < ROWS; r += NWARPS) {
-        const int y = r % N + 1;
-        const int z = (D == 3) ? r / N + 1 : 0;
-        const int xs = 1 + (((1 + y + z) & 1) ^ color);
-        const int x = xs + 2 * lane;          // N <= 63: one pass of 32 lanes covers the row
-        if (x > N) continue;
+    // node x of grid row r (y, z), xs the first x of the colour in that row
+    auto node = [&](int y, int z, int xs, int x) {
         const int row = ((D == 3) ? (z * S + y) : y) * S;
         // x has the row's colour parity p; its west / east neighbours the other one
         constexpr int HE = Lv<D, N>::HE;
@@ -121,6 +122,24 @@ __device__ __forceinline__ void t_sweep(typename C2<R>::T* E, const typename C2<
         v.x = (sx - h2 * rr.x) * dinv;
         v.y = (sy - h2 * rr.y) * dinv;
         E[o] = v;
+    };
+    if constexpr (t_flat<R>()) {
+        constexpr int NXH = (N + 1) / 2;                 // nodes of a colour in a row, at most
+        for (int q = t_id<NWARPS>(); q < ROWS * NXH; q += 32 * NWARPS) {
+            const int r = q / NXH, i = q % NXH;
+            const int y = r % N + 1, z = (D == 3) ? r / N + 1 : 0;
+            const int xs = 1 + (((1 + y + z) & 1) ^ color), x = xs + 2 * i;
+            if (x <= N) node(y, z, xs, x);
+        }
+    } else {
+        const int lane = threadIdx.x & 31;
+        for (int r = threadIdx.x >> 5; r < ROWS; r += NWARPS) {
+            const int y = r % N + 1;
+            const int z = (D == 3) ? r / N + 1 : 0;
+            const int xs = 1 + (((1 + y + z) & 1) ^ color);
+            const int x = xs + 2 * lane;          // N <= 63: one pass of 32 lanes covers the row
+            if (x <= N) node(y, z, xs, x);
+        }
     }
 }
 
@@ -138,9 +157,12 @@ __device__ __forceinline__ void t_restrict(const typename C2<R>::T* E, const typ
     constexpr int ROWS = (D == 3) ? NC * NC : NC;
     const R ih2 = (R)1 / (h * h);
     const R scale = (D == 3) ? (R)(1.0 / 64.0) : (R)(1.0 / 16.0);
-    const int X = (threadIdx.x & 31) + 1;
-    if (X > NC) return;
-    for (int r = threadIdx.x >> 5; r < ROWS; r += NWARPS) {
+    constexpr bool FLAT = t_flat<R>();
+    const int lane = threadIdx.x & 31;
+    if (!FLAT && lane >= NC) return;
+    for (int q = FLAT ? t_id<NWARPS>() : (int)(threadIdx.x >> 5); q < (FLAT ? ROWS * NC : ROWS);
+         q += FLAT ? 32 * NWARPS : NWARPS) {
+        const int r = FLAT ? q / NC : q, X = (FLAT ? q % NC : lane) + 1;
         const int Y = r % NC + 1;
         const int Z = (D == 3) ? r / NC + 1 : 0;
         R ax = 0, ay = 0;
@@ -195,37 +217,46 @@ __device__ __forceinline__ void t_prolong(typename C2<R>::T* E, const typename C
     constexpr int SC = NC + 2;
     constexpr int HE = Lv<D, N>::HE;
     constexpr int ROWS = (D == 3) ? N * N : N;
-    const int lane = threadIdx.x & 31;
     const R w = (D == 3) ? (R)0.125 : (R)0.25;
-    for (int r = threadIdx.x >> 5; r < ROWS; r += NWARPS) {
-        const int y = r % N + 1;
-        const int z = (D == 3) ? r / N + 1 : 0;
+    // node x = 2 q + par of grid row (y, z)
+    auto node = [&](int y, int z, int q, int par) {
         const int row = ((D == 3) ? (z * S + y) : y) * S;
         const int y0 = y >> 1, y1 = (y + 1) >> 1;
         const int z0 = z >> 1, z1 = (z + 1) >> 1;
+        const int c0 = ix<NC>(q), c1 = par ? ix<NC>(q + 1) : c0;
+        R vx = 0, vy = 0;
 #pragma unroll
-        for (int par = 0; par < 2; ++par) {
-            const int q = lane + (par ? 0 : 1);
-            if (2 * q + par > N) continue;
-            const int c0 = ix<NC>(q), c1 = par ? ix<NC>(q + 1) : c0;
-            R vx = 0, vy = 0;
+        for (int iz = 0; iz < (D == 3 ? 2 : 1); ++iz)
 #pragma unroll
-            for (int iz = 0; iz < (D == 3 ? 2 : 1); ++iz)
+            for (int iy = 0; iy < 2; ++iy) {
+                const int Z = iz ? z1 : z0, Y = iy ? y1 : y0;
+                const int crow = ((D == 3) ? (Z * SC + Y) : Y) * SC;
+                const c2 a = Ec[crow + c0], b = Ec[crow + c1];
+                vx += a.x;
+                vy += a.y;
+                vx += b.x;
+                vy += b.y;
+            }
+        const int o = row + (par ? HE : 0) + q;
+        c2 v = E[o];
+        v.x += w * vx;
+        v.y += w * vy;
+        E[o] = v;
+    };
+    if constexpr (t_flat<R>()) {
+        for (int t = t_id<NWARPS>(); t < ROWS * N; t += 32 * NWARPS) {
+            const int r = t / N, x = t % N + 1;
+            node(r % N + 1, (D == 3) ? r / N + 1 : 0, x >> 1, x & 1);
+        }
+    } else {
+        const int lane = threadIdx.x & 31;
+        for (int r = threadIdx.x >> 5; r < ROWS; r += NWARPS) {
+            const int y = r % N + 1, z = (D == 3) ? r / N + 1 : 0;
 #pragma unroll
-                for (int iy = 0; iy < 2; ++iy) {
-                    const int Z = iz ? z1 : z0, Y = iy ? y1 : y0;
-                    const int crow = ((D == 3) ? (Z * SC + Y) : Y) * SC;
-                    const c2 a = Ec[crow + c0], b = Ec[crow + c1];
-                    vx += a.x;
-                    vy += a.y;
-                    vx += b.x;
-                    vy += b.y;
-                }
-            const int o = row + (par ? HE : 0) + q;
-            c2 v = E[o];
-            v.x += w * vx;
-            v.y += w * vy;
-            E[o] = v;
+            for (int par = 0; par < 2; ++par) {
+                const int q = lane + (par ? 0 : 1);
+                if (2 * q + par <= N) node(y, z, q, par);
+            }
         }
     }
 }
@@ -407,6 +438,10 @@ __device__ __forceinline__ void y_solve(float2* E, const float2* Rr, float* scr,
 // walls: e = c S (W o (S r S)) S, c = -h^2 / (n+1)^2, W_ab = 1 / (s_a + s_b + sigma h^2 / 4)
 __device__ __forceinline__ void z_solve(double2* E, const double2* Rr, const double* scr, double h, double sigma)
 {
+    // The basis is symmetric or antisymmetric about the middle, S_a(16-j) = (-1)^(a+1) S_aj, so
+    // each product runs over sums (odd a) or differences (even a) of mirrored inputs: 8 terms an
+    // output instead of 15, on the FP64 pipe that bounds it.  A product's result is left folded
+    // along the next one's axis by its own threads after a barrier.
     const double* Sm = scr;
     const double* sv = scr + ZN * ZP;
     double2* T1 = reinterpret_cast<double2*>(const_cast<double*>(scr) + ZTAB_DOUBLES);
@@ -415,52 +450,57 @@ __device__ __forceinline__ void z_solve(double2* E, const double2* Rr, const dou
     const double tau = 0.25 * sigma * h * h;
     const int t = threadIdx.x;
     const bool act = t < ZN * ZN;
-    const int a = t / ZN, b = t % ZN;
+    const int a = t / ZN, b = t % ZN;                // 0-based: basis function a + 1
+    constexpr int M = ZN / 2;                        // 7: the middle index
     auto at = [](int y, int x) { return (y + 1) * (ZN + 2) + ix<ZN>(x + 1); };
-    if (act) {                                   // T1[a][b] = sum_y S[a][y] r[y][b]
+    // rows j and 14 - j of the fold hold sum and difference; the middle row stays
+    auto fold = [&](auto get, auto put) {
+        if (t < M * ZN) {
+            const int j = t / ZN, k = t % ZN;
+            const double2 u = get(j, k), v = get(ZN - 1 - j, k);
+            put(j, k, make_double2(u.x + v.x, u.y + v.y));
+            put(ZN - 1 - j, k, make_double2(u.x - v.x, u.y - v.y));
+        }
+    };
+    // sum_j S[f][j] in[j] from the folded inputs get(j)
+    auto dot = [&](int f, auto get) {
         double ax = 0.0, ay = 0.0;
-        for (int y = 0; y < ZN; ++y) {
-            const double s = Sm[a * ZP + y];
-            const double2 v = Rr[at(y, b)];
+        const bool odd = (f & 1) == 0;               // basis function f + 1 odd
+#pragma unroll
+        for (int j = 0; j < M; ++j) {
+            const double s = Sm[f * ZP + j];
+            const double2 v = get(odd ? j : ZN - 1 - j);
             ax = fma(s, v.x, ax);
             ay = fma(s, v.y, ay);
         }
-        T1[a * ZP + b] = make_double2(ax, ay);
-    }
-    __syncthreads();
-    if (act) {                                   // T2[a][b] = c W_ab sum_x T1[a][x] S[x][b]
-        double ax = 0.0, ay = 0.0;
-        for (int x = 0; x < ZN; ++x) {
-            const double s = Sm[x * ZP + b];
-            const double2 v = T1[a * ZP + x];
-            ax = fma(v.x, s, ax);
-            ay = fma(v.y, s, ay);
+        if (odd) {
+            const double s = Sm[f * ZP + M];
+            const double2 v = get(M);
+            ax = fma(s, v.x, ax);
+            ay = fma(s, v.y, ay);
         }
+        return make_double2(ax, ay);
+    };
+    fold([&](int j, int k) { return Rr[at(j, k)]; }, [&](int j, int k, double2 v) { T1[j * ZP + k] = v; });
+    if (t < ZN) T1[M * ZP + t] = Rr[at(M, t)];
+    __syncthreads();
+    if (act) T2[a * ZP + b] = dot(a, [&](int j) { return T1[j * ZP + b]; });               // S r
+    __syncthreads();
+    fold([&](int j, int k) { return T2[k * ZP + j]; }, [&](int j, int k, double2 v) { T2[k * ZP + j] = v; });
+    __syncthreads();
+    if (act) {                                                                              // c W o (S r S)
+        const double2 v = dot(b, [&](int j) { return T2[a * ZP + j]; });
         const double w = c / (sv[a] + sv[b] + tau);
-        T2[a * ZP + b] = make_double2(w * ax, w * ay);
+        T1[a * ZP + b] = make_double2(w * v.x, w * v.y);
     }
     __syncthreads();
-    if (act) {                                   // T1[a][b] = sum_y S[a][y] T2[y][b]
-        double ax = 0.0, ay = 0.0;
-        for (int y = 0; y < ZN; ++y) {
-            const double s = Sm[a * ZP + y];
-            const double2 v = T2[y * ZP + b];
-            ax = fma(s, v.x, ax);
-            ay = fma(s, v.y, ay);
-        }
-        T1[a * ZP + b] = make_double2(ax, ay);
-    }
+    fold([&](int j, int k) { return T1[j * ZP + k]; }, [&](int j, int k, double2 v) { T1[j * ZP + k] = v; });
     __syncthreads();
-    if (act) {                                   // E[a][b] = sum_x T1[a][x] S[x][b]
-        double ax = 0.0, ay = 0.0;
-        for (int x = 0; x < ZN; ++x) {
-            const double s = Sm[x * ZP + b];
-            const double2 v = T1[a * ZP + x];
-            ax = fma(v.x, s, ax);
-            ay = fma(v.y, s, ay);
-        }
-        E[at(a, b)] = make_double2(ax, ay);
-    }
+    if (act) T2[a * ZP + b] = dot(a, [&](int j) { return T1[j * ZP + b]; });               // S (...)
+    __syncthreads();
+    fold([&](int j, int k) { return T2[k * ZP + j]; }, [&](int j, int k, double2 v) { T2[k * ZP + j] = v; });
+    __syncthreads();
+    if (act) E[at(a, b)] = dot(b, [&](int j) { return T2[a * ZP + j]; });                  // (S (...)) S
     __syncthreads();
 }
 
