@@ -45,6 +45,14 @@ cudaError_t launch_restrict(int D, int prec, const InstDesc* insts, const InstSt
 cudaError_t launch_prolong(int D, int prec, const InstDesc* insts, const InstState* st,
                            const MgItem* items, int nitems, int work, cudaStream_t s, int mode = 0,
                            int skip0 = 0);
+// the 3D FP64 forms of these three (vcycle3d64.cu), called by them
+cudaError_t setup_3d64();
+cudaError_t launch_rbgs64(const InstDesc* insts, const InstState* st, const MgItem* items, int nitems, int work,
+                          int color, int mode, cudaStream_t s);
+cudaError_t launch_restrict64(const InstDesc* insts, const InstState* st, const MgItem* items, int nitems, int work,
+                              cudaStream_t s, int mode);
+cudaError_t launch_prolong64(const InstDesc* insts, const InstState* st, const MgItem* items, int nitems, int work,
+                             cudaStream_t s, int mode, int skip0);
 // zero the iterate of the listed levels (ring included)
 cudaError_t launch_zero(int D, int prec, const InstDesc* insts, const InstState* st,
                         const MgItem* items, int nitems, int work, cudaStream_t s);

@@ -107,7 +107,7 @@ k_rbgs(const InstDesc* __restrict__ insts, const InstState* __restrict__ st,
 // x-neighbours at j, j+1 (odd x) or j-1, j (even x).  No shared-memory word is written by the
 // sweep; results go straight to global memory.
 template <typename R> struct Rb3p {
-    static constexpr int TY = sizeof(R) == 4 ? 8 : 4;      // rows per CTA (a warp per row)
+    static constexpr int TY = 8;                           // rows per CTA (a warp per row)
     static constexpr int L = 1;                            // planes in flight
     static constexpr int OS = L + 3, RS = L + 1;           // ring slots
     static constexpr int MAX_HP = 264;                     // pitch / 2 of n = 511
@@ -542,7 +542,7 @@ template <int D, typename R>
 static cudaError_t carve()
 {
     cudaError_t e;
-    if (D == 3 && sizeof(R) == 4) {                        // the z-marching forms are complex64 only
+    if constexpr (D == 3 && sizeof(R) == 4) {              // the z-marching forms are complex64 only
         if ((e = max_carveout(k_restrict3p<R>)) != cudaSuccess) return e;
         if ((e = cudaFuncSetAttribute(k_restrict3p<R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)Rs3p<R>::bytes(Rs3p<float>::MAX_P))) != cudaSuccess)
@@ -552,9 +552,13 @@ static cudaError_t carve()
                                       (int)Rb3p<R>::bytes(Rb3p<float>::MAX_HP))) != cudaSuccess)
             return e;
     }
-    if ((e = max_carveout(k_rbgs<D, R>)) != cudaSuccess) return e;
-    if ((e = max_carveout(k_restrict<D, R>)) != cudaSuccess) return e;
-    if ((e = max_carveout(k_prolong<D, R>)) != cudaSuccess) return e;
+    if constexpr (D == 3 && sizeof(R) == 8) {              // FP64 has its own level kernels
+        if ((e = setup_3d64()) != cudaSuccess) return e;
+    } else {
+        if ((e = max_carveout(k_rbgs<D, R>)) != cudaSuccess) return e;
+        if ((e = max_carveout(k_restrict<D, R>)) != cudaSuccess) return e;
+        if ((e = max_carveout(k_prolong<D, R>)) != cudaSuccess) return e;
+    }
     return max_carveout(k_zero<D, R>);
 }
 
@@ -568,11 +572,12 @@ cudaError_t launch_rbgs(int D, int prec, const InstDesc* insts, const InstState*
                         const MgItem* items, int nitems, int work, int color, int mode,
                         cudaStream_t s, int nmax)
 {
+    if (D == 3 && prec == 0) return launch_rbgs64(insts, st, items, nitems, work, color, mode, s);
     // 3D plain half-sweeps of levels 127 .. 511: the plane-marching form
     const int hp = (nmax + 2 + 15) / 16 * 8;
-    if (D == 3 && prec != 0 && mode == 0 && nmax >= 127 && hp <= Rb3p<float>::MAX_HP) {
-        const int ty = prec == 0 ? Rb3p<double>::TY : Rb3p<float>::TY;
-        const size_t sm = prec == 0 ? Rb3p<double>::bytes(hp) : Rb3p<float>::bytes(hp);
+    if (D == 3 && mode == 0 && nmax >= 127 && hp <= Rb3p<float>::MAX_HP) {
+        const int ty = Rb3p<float>::TY;
+        const size_t sm = Rb3p<float>::bytes(hp);
         const int per_sm = (int)(227 * 1024 / (sm + 1024));
         const int nyb = (nmax + ty - 1) / ty;
         // z chunks so that the launch is about one wave of resident CTAs
@@ -581,14 +586,12 @@ cudaError_t launch_rbgs(int D, int prec, const InstDesc* insts, const InstState*
         const int zchunk = (nmax + nzc - 1) / nzc;
         nzc = (nmax + zchunk - 1) / zchunk;
         dim3 g(nyb * nzc, nitems);
-        if (prec == 0) launch_k(k_rbgs3p<double>, g, dim3(32 * ty), sm, s, insts, st, items, color, zchunk);
-        else launch_k(k_rbgs3p<float>, g, dim3(32 * ty), sm, s, insts, st, items, color, zchunk);
+        launch_k(k_rbgs3p<float>, g, dim3(32 * ty), sm, s, insts, st, items, color, zchunk);
         return cudaGetLastError();
     }
     dim3 g = mg_grid(work, nitems);
     if (D == 2 && prec == 0) launch_k(k_rbgs<2, double>, dim3(g), dim3(256), 0, s, insts, st, items, color, mode);
     else if (D == 2) launch_k(k_rbgs<2, float>, dim3(g), dim3(256), 0, s, insts, st, items, color, mode);
-    else if (prec == 0) launch_k(k_rbgs<3, double>, dim3(g), dim3(256), 0, s, insts, st, items, color, mode);
     else launch_k(k_rbgs<3, float>, dim3(g), dim3(256), 0, s, insts, st, items, color, mode);
     return cudaGetLastError();
 }
@@ -596,10 +599,11 @@ cudaError_t launch_rbgs(int D, int prec, const InstDesc* insts, const InstState*
 cudaError_t launch_restrict(int D, int prec, const InstDesc* insts, const InstState* st,
                             const MgItem* items, int nitems, int work, cudaStream_t s, int mode, int nmax)
 {
+    if (D == 3 && prec == 0) return launch_restrict64(insts, st, items, nitems, work, s, mode);
     // 3D complex64 restriction of the rhs alone (every iterate of the launch zero) from fine
     // levels 127 .. 511: the z-marching form
     const int pitch = (nmax + 2 + 15) / 16 * 16;
-    if (D == 3 && prec != 0 && mode == 2 && nmax >= 127 && pitch <= Rs3p<float>::MAX_P) {
+    if (D == 3 && mode == 2 && nmax >= 127 && pitch <= Rs3p<float>::MAX_P) {
         const int nc = (nmax - 1) / 2;
         const size_t sm = Rs3p<float>::bytes(pitch);
         const int per_sm = (int)(227 * 1024 / (sm + 1024));
@@ -615,7 +619,6 @@ cudaError_t launch_restrict(int D, int prec, const InstDesc* insts, const InstSt
     dim3 g = mg_grid(work, nitems);
     if (D == 2 && prec == 0) launch_k(k_restrict<2, double>, dim3(g), dim3(256), 0, s, insts, st, items, mode);
     else if (D == 2) launch_k(k_restrict<2, float>, dim3(g), dim3(256), 0, s, insts, st, items, mode);
-    else if (prec == 0) launch_k(k_restrict<3, double>, dim3(g), dim3(256), 0, s, insts, st, items, mode);
     else launch_k(k_restrict<3, float>, dim3(g), dim3(256), 0, s, insts, st, items, mode);
     return cudaGetLastError();
 }
@@ -623,10 +626,10 @@ cudaError_t launch_restrict(int D, int prec, const InstDesc* insts, const InstSt
 cudaError_t launch_prolong(int D, int prec, const InstDesc* insts, const InstState* st,
                            const MgItem* items, int nitems, int work, cudaStream_t s, int mode, int skip0)
 {
+    if (D == 3 && prec == 0) return launch_prolong64(insts, st, items, nitems, work, s, mode, skip0);
     dim3 g = mg_grid(work, nitems);
     if (D == 2 && prec == 0) launch_k(k_prolong<2, double>, dim3(g), dim3(256), 0, s, insts, st, items, mode, skip0);
     else if (D == 2) launch_k(k_prolong<2, float>, dim3(g), dim3(256), 0, s, insts, st, items, mode, skip0);
-    else if (prec == 0) launch_k(k_prolong<3, double>, dim3(g), dim3(256), 0, s, insts, st, items, mode, skip0);
     else launch_k(k_prolong<3, float>, dim3(g), dim3(256), 0, s, insts, st, items, mode, skip0);
     return cudaGetLastError();
 }

@@ -97,3 +97,32 @@ def test_iterate_larger_than_the_result_and_nan():
     assert _error(n, 1.0 / (n + 1), r, e0, (2, 2)) <= 10 * 2.0 ** -53 * 512
     r[7, 9] = complex("nan")
     assert np.isnan(_run(n, 1.0 / (n + 1), r, e0, (2, 2))).any()
+
+
+@pytest.mark.parametrize("n", [1, 3, 7, 15, 31, 63])
+@pytest.mark.parametrize("nu", [(0, 2), (2, 2), (2, 0)])
+@pytest.mark.parametrize("kind", ["rough", "smooth", "patch"])
+def test_3d_error_is_fp64s_own(n, nu, kind):
+    # (a node's last update and correction: 7 + 8 terms, 14 roundings of half an ulp)
+    from paper_2308_11469_gb300 import binding as B
+    h = (0.7 if kind == "smooth" else 1.0) / (n + 1)
+    rng = np.random.default_rng(n)
+    if kind == "rough":
+        r = rng.standard_normal((n,) * 3) + 1j * rng.standard_normal((n,) * 3)
+    elif kind == "smooth":
+        s = np.sin(np.pi * np.arange(1, n + 1) / (n + 1))
+        r = (1 - 2j) * s[:, None, None] * s[None, :, None] * s[None, None, :]
+    else:
+        r = np.zeros((n,) * 3, dtype=complex)
+        r[n // 2, n // 2, n // 3:n // 3 + 2] = 1.0 - 2.0j
+    plan = B.helm_plan_create(3, n, h, 1.0, prec=B.HELM_PREC_FP64)
+    e = torch.zeros((n,) * 3, dtype=torch.complex128, device="cuda")
+    B.poisson_vcycle(plan, torch.from_numpy(r).cuda(), e, *nu)
+    B.helm_plan_destroy(plan)
+    got, num, den = e.cpu().numpy(), LD(0), LD(0)
+    for part in ("real", "imag"):
+        E = np.zeros((n + 2,) * 3, dtype=LD)
+        mg.vcycle(E, getattr(r, part).astype(LD), LD(h), *nu)
+        num += ((getattr(got, part).astype(LD) - E[1:-1, 1:-1, 1:-1]) ** 2).sum()
+        den += (E ** 2).sum()
+    assert float(np.sqrt(num / den)) <= 14 * 2.0 ** -53
