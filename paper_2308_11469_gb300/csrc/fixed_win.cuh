@@ -67,6 +67,33 @@ __device__ __forceinline__ int block_max_exp(int ex, int* sx)
 // derived from it)?
 __device__ __forceinline__ bool fx_usable(int emax) { return emax >= FX_EMIN + 8 && emax <= FX_EMAX - 8; }
 
+// v 2^(1080 - emax) truncated (fx_fix without its range test)
+__device__ __forceinline__ long long fx_qt(double v, int emax)
+{
+    const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
+    const unsigned mh = (hi & 0x000fffffu) | 0x00100000u;
+    unsigned long long m = ((unsigned long long)__funnelshift_l(lo, mh, 10) << 32) | (lo << 10);
+    asm("shr.u64 %0, %0, %1;" : "+l"(m) : "r"(emax + 5 - (int)((hi >> 20) & 0x7ffu)));
+    const long long sg = (long long)((int)hi >> 31);
+    return ((long long)m ^ sg) - sg;
+}
+
+// v 2^(emax - 1080) rounded to nearest, ties to even, in the inner precision; binary32 results
+// below the normal range become zero (as d2f_bits does)
+__device__ __forceinline__ double fx_inner(long long v, int emax, double) { return fx_to_double(v, emax); }
+__device__ __forceinline__ float fx_inner(long long v, int emax, float)
+{
+    const unsigned long long a = (unsigned long long)(v < 0 ? -v : v);
+    const int lz = __clzll((long long)a);
+    const unsigned long long m = a << (lz & 63);          // leading 1 at bit 63
+    // 32 bits with the rest folded into the last one: the rounding to 24 sees the same
+    const unsigned b = __float_as_uint(__uint2float_rn((unsigned)(m >> 32) | ((unsigned)m != 0u)));
+    // b = top * 2^0 with top in [2^31, 2^32]; the value is top * 2^(32 - lz + emax - 1080)
+    const int E = (int)(b >> 23) + 32 - lz + emax - 1080;
+    const unsigned f = (unsigned)E - 1u < 254u ? ((unsigned)E << 23) | (b & 0x007fffffu) : (E >= 255 ? 0x7f800000u : 0u);
+    return __uint_as_float(a == 0ull ? 0u : f | ((unsigned)(v >> 32) & 0x80000000u));
+}
+
 // h^2 as a scale: the exponents h^2 adds to a value's (exactly for a power of two, else at most)
 struct FxH2 {
     double h2;

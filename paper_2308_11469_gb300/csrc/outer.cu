@@ -542,13 +542,165 @@ k_upres2d(const InstDesc* __restrict__ insts, InstState* __restrict__ st,
 // three-plane ring of shared memory (1-node halo in x and y)
 // ---------------------------------------------------------------------------
 constexpr int T3X = 32, T3Y = 8, T3Z = 16;
-// resident CTAs per SM of the 3D residual (40 registers at 6): at 255^3 477 -> 396 us per
-// launch against 4 CTAs of 64 registers; fetching each plane one plane ahead into
-// registers measured slower (412 / 432 / 485 us at 4 / 5 / 6 CTAs), and so did a two-deep
-// cp.async ring of the next planes' words in shared memory (425 against 385 us: 5 CTAs
-// per SM, and the copies' issue cost on a kernel bound by its integer work)
-constexpr int RES3D_CTAS = 6;
+// Resident CTAs per SM of the 3D residual: 64 registers at 4, which hold a column's planes and
+// the next plane's words in flight (255^3 complex64 solve 15.2 ms on per-plane scales, 6 CTAs;
+// on the instance's scale with 3, 4, 5 CTAs 14.0, 14.0, 16.5; three warps of their own for the
+// ring 15.6, the ring's next words in registers 14.0 at 3 and 15.4 at 4).
+constexpr int RES3D_CTAS = 4;
 constexpr int P3 = (T3X + 2) * (T3Y + 2);
+constexpr int RING3 = 2 * (T3X + 2) + 2 * T3Y;
+
+// Per-step form (u_{N+1} = u_N + e_N and r_{N+1}), with h^2 a power of two and the whole
+// instance on one fixed-point scale: four times the largest value of u_N (InstState::uex).  A
+// thread keeps its column's values of planes z - 1, z, z + 1 in registers; a plane's window goes
+// through two slots of shared memory, one barrier a plane, and no exponent has to be reduced or
+// shifted to.  f - k^2 u (+ i p u) is formed in FP64 and joins the numerator in fixed point, so
+// h^2 r is one exact sum, rounded once to the inner precision:
+//   h^2 r = h^2 (f - k^2 u + i p u) - (sum of neighbours - 6 u).
+// One unit is 2^-56 of the instance's largest value (FP64 rounds its terms at 2^-53 of their
+// own).  Values beyond the scale (an iterate growing more than fourfold in a step, a source or a
+// wall far above it, an infinity or a NaN) are seen in the largest exponent the tile meets:
+// false, and the tile is redone on per-plane scales.
+// About 330 integer instructions and 4.7 FP64 operations a point (577 and 6.7 on per-plane
+// scales); bound by its load and barrier latency: 255^3 complex64 382 -> 330 us a launch, 3.2 TB/s
+// of its 64 bytes a point.
+template <typename R, bool DAMP>
+__device__ __forceinline__ bool residual3d_tile_scaled(const InstDesc& I, const InstState& s, const ResItem item,
+                                                       longlong2 (*U)[P3], int* sx, int add, R& r2_out, R& em_out,
+                                                       int& ex_out)
+{
+    typedef typename C2<R>::T c2;
+    double2* const Ru = reinterpret_cast<double2*>(U[2]);     // (the third slot is free here)
+    c2* const Re = reinterpret_cast<c2*>(Ru + RING3);
+    static_assert(RING3 * (sizeof(double2) + sizeof(c2)) <= sizeof(U[2]), "raw ring words");
+    const int n = I.n;
+    // (32-bit offsets: n <= 1023)
+    const unsigned S = n + 2, SP = S * S, NP = (unsigned)n * n;
+    const double2* __restrict__ uin = (s.it & 1) ? I.u[1] : I.u[0];
+    double2* __restrict__ uout = (double2*)((s.it & 1) ? I.u[0] : I.u[1]);
+    const double2* __restrict__ f = I.f;
+    const LevelDesc L0 = I.lev[0];
+    const c2* __restrict__ e = (const c2*)L0.e;
+    c2* __restrict__ rhs = (c2*)L0.rhs;            // (a 3D level has one right-hand side)
+    const unsigned P = L0.pitch, PL = P * L0.rows;
+    const double mk2 = -I.k2, damp = I.damp;
+    const int em = s.uex + 2;
+    const int x0 = 1 + item.tx * T3X, y0 = 1 + item.ty * T3Y, z0 = 1 + item.tz * T3Z;
+    const int z1 = min(z0 + T3Z - 1, n);
+    const int lx = (threadIdx.x & 31) + 1, ly = (threadIdx.x >> 5) + 1;
+    const int gx = x0 + lx - 1, gy = y0 + ly - 1;
+    const bool live = gx <= n && gy <= n;
+    const bool inw = gx <= n + 1 && gy <= n + 1;   // a wall node at most
+    const int o = ly * (T3X + 2) + lx;
+    // offsets of the own node in a plane of u, of e and of f
+    const unsigned uo = inw ? gy * S + gx : 0, eo = live ? gy * P + xslot<3>(gx, (int)P) : 0;
+    const unsigned fo = live ? (unsigned)(gy - 1) * n + (gx - 1) : 0;
+    // threads below the ring's size also stage one of its nodes, through shared memory (their
+    // own slots: no barrier between the copy and its reader)
+    const bool ring = threadIdx.x < RING3;
+    unsigned ur = 0, er = 0;
+    int ro = 0;
+    bool rin = false, rint = false;
+    if (ring) {
+        int rlx, rly;
+        ring_node<T3X, T3Y>(threadIdx.x, rlx, rly);
+        const int rx = x0 - 1 + rlx, ry = y0 - 1 + rly;
+        rin = rx <= n + 1 && ry <= n + 1;
+        rint = rin && rx >= 1 && rx <= n && ry >= 1 && ry <= n;
+        ro = rly * (T3X + 2) + rlx;
+        if (rin) ur = ry * S + rx;
+        if (rint) er = ry * P + xslot<3>(rx, (int)P);
+    }
+    unsigned top = 0, gtop = 0;                    // largest high words met (sign off)
+    R r2 = 0, emax2 = 0;
+    auto hi = [](double v) { return (unsigned)__double2hiint(v) & 0x7fffffffu; };
+    // the node's raw words (own: registers), fetched one plane ahead
+    double2 nu = make_double2(0.0, 0.0), nf = nu;
+    c2 ne;
+    auto fetch_ring = [&](int z) {
+        if (ring) {
+            cp_async_elem<16>(Ru + threadIdx.x, uin + z * SP + ur, rin);
+            cp_async_elem<sizeof(c2)>(Re + threadIdx.x, e + z * PL + er, rint);
+        }
+    };
+    auto fetch = [&](int z) {                      // plane z (the walls' included)
+        if (inw) nu = uin[z * SP + uo];
+        ne.x = ne.y = 0;
+        if (live && z >= 1 && z <= n) ne = e[z * PL + eo];
+    };
+    auto sum = [&](double2 v, c2 ev) -> double2 {
+        v.x += Inner<R>::widen(ev.x);
+        v.y += Inner<R>::widen(ev.y);
+        top = max(top, max(hi(v.x), hi(v.y)));
+        return v;
+    };
+    auto fix = [&](double2 v) { return make_longlong2(fx_qt(v.x, em), fx_qt(v.y, em)); };
+    auto stage_ring = [&](int z) {
+        if (ring) {
+            cp_async_wait_all();
+            U[z & 1][ro] = fix(sum(Ru[threadIdx.x], Re[threadIdx.x]));
+        }
+    };
+    fetch_ring(z0);
+    fetch(z0 - 1);
+    longlong2 dn = fix(sum(nu, ne));
+    fetch(z0);
+    if (live) nf = f[(z0 - 1) * NP + fo];
+    double2 cur = sum(nu, ne);
+    if (live) emax2 = abs2(ne);
+    longlong2 fc = fix(cur);
+    U[z0 & 1][o] = fc;
+    stage_ring(z0);
+    if (z0 < z1) fetch_ring(z0 + 1);
+    fetch(z0 + 1);
+    __syncthreads();
+    for (int z = z0; z <= z1; ++z) {
+        const bool more = z < z1;                  // plane z + 1 is this tile's
+        const double2 nxt = sum(nu, ne);
+        if (live && more) emax2 = fmax(emax2, abs2(ne));
+        const longlong2 up = fix(nxt);
+        if (more) {
+            U[(z + 1) & 1][o] = up;
+            stage_ring(z + 1);
+        }
+        double2 g = make_double2(fma(cur.x, mk2, nf.x), fma(cur.y, mk2, nf.y));
+        if (more) {
+            fetch(z + 2);                          // (z + 2 <= n + 1)
+            if (z + 1 < z1) fetch_ring(z + 2);
+            if (live) nf = f[z * NP + fo];
+        }
+        if (live) {
+            const longlong2* Uc = U[z & 1];
+            const longlong2 W = Uc[o - 1], E = Uc[o + 1], So = Uc[o - (T3X + 2)], No = Uc[o + (T3X + 2)];
+            if constexpr (DAMP) {
+                g.x = fma(cur.y, damp, g.x);
+                g.y = fma(cur.x, -damp, g.y);
+            }
+            gtop = max(gtop, max(hi(g.x), hi(g.y)));
+            const long long Gx = fx_qt(g.x, em - add), Gy = fx_qt(g.y, em - add);
+            const long long tx = (Gx - ((W.x + E.x) + (So.x + No.x))) - ((dn.x + up.x) - 6 * fc.x);
+            const long long ty = (Gy - ((W.y + E.y) + (So.y + No.y))) - ((dn.y + up.y) - 6 * fc.y);
+            uout[z * SP + uo] = cur;
+            c2 ri;
+            ri.x = fx_inner(tx, em - add, R());
+            ri.y = fx_inner(ty, em - add, R());
+            rhs[z * PL + eo] = ri;
+            r2 += abs2(ri);
+        }
+        dn = fc;
+        fc = up;
+        cur = nxt;
+        __syncthreads();
+    }
+    const int ex = block_max_exp<NTH>((int)(top >> 20), sx);
+    __syncthreads();
+    const int eg = block_max_exp<NTH>((int)(gtop >> 20), sx);
+    __syncthreads();
+    r2_out = r2;
+    em_out = emax2;
+    ex_out = ex;
+    return ex <= em && (eg == 0 || eg + add <= em);
+}
 
 // The column's planes go through the ring in fixed point
 // (fixed_lap.cuh), each plane on the scale of its own largest exponent; the numerator of
@@ -556,8 +708,9 @@ constexpr int P3 = (T3X + 2) * (T3Y + 2);
 // values shifted down to it), so every node's numerator is exact up to the truncations.
 // Thread t stages the interior node (t mod 32, t / 32) of each plane and keeps it in FP64
 // for its own residual; threads below the ring size stage one ring node each.
+// (not inlined beside the form above, whose registers it would share)
 template <typename R, int MODE, bool DAMP>
-__device__ __forceinline__ void residual3d_tile_fx(const InstDesc* __restrict__ insts,
+__device__ __noinline__ void residual3d_tile_fx(const InstDesc* __restrict__ insts,
                                                    InstState* __restrict__ st, const ResItem item,
                                                    longlong2 (*U)[P3], int* sx, const StepCtl& c)
 {
@@ -575,6 +728,8 @@ __device__ __forceinline__ void residual3d_tile_fx(const InstDesc* __restrict__ 
         if (c.ctrl && item.tx == 0 && item.ty == 0 && item.tz == 0) step_arrive(st, c);
         return;
     }
+    const int tile = (item.tz * I.res_ty + item.ty) * I.res_tx + item.tx;
+    int exm = 0;                                   // largest exponent of the tile's iterate
     const double2* __restrict__ uin = (s.it & 1) ? I.u[1] : I.u[0];
     double2* __restrict__ uout = (double2*)((s.it & 1) ? I.u[0] : I.u[1]);
     const double2* __restrict__ f = I.f;
@@ -618,7 +773,9 @@ __device__ __forceinline__ void residual3d_tile_fx(const InstDesc* __restrict__ 
         mine = node(lx, ly, gz, own && live);
         double2 rv = make_double2(0.0, 0.0);
         if (threadIdx.x < RING) rv = node(rlx, rly, gz, false);
-        const int ep = fx_scale(block_max_exp<NTH>(max(fx_exp2(mine), fx_exp2(rv)), sx));
+        const int raw = block_max_exp<NTH>(max(fx_exp2(mine), fx_exp2(rv)), sx);
+        exm = max(exm, raw);
+        const int ep = fx_scale(raw);
         U[slot][o] = fx_fix2(mine, ep);
         if (threadIdx.x < RING) U[slot][ro] = fx_fix2(rv, ep);
         return ep;
@@ -684,9 +841,8 @@ __device__ __forceinline__ void residual3d_tile_fx(const InstDesc* __restrict__ 
         sc = sn;
         sn = t;
     }
-    const int tile = (item.tz * I.res_ty + item.ty) * I.res_tx + item.tx;
-    if constexpr (MODE == 0) tile_done<double>(I, stp, tile, r2d, b2, MODE, st, c);
-    else tile_done<R>(I, stp, tile, r2, emax2, MODE, st, c);
+    if constexpr (MODE == 0) tile_done<double>(I, stp, tile, r2d, b2, MODE, st, c, exm);
+    else tile_done<R>(I, stp, tile, r2, emax2, MODE, st, c, exm);
 }
 
 // (the start residual, once per solve, also forms ||b||: it runs at 4 CTAs per SM, whose 64
@@ -701,7 +857,25 @@ k_residual3d(const InstDesc* __restrict__ insts, InstState* __restrict__ st,
     pdl_wait();
     pdl_trigger();
     for (int t = blockIdx.x; t < nitems; t += gridDim.x) {
-        residual3d_tile_fx<R, MODE, DAMP>(insts, st, items[t], reinterpret_cast<longlong2(*)[P3]>(U), sx, c);
+        const ResItem item = items[t];
+        longlong2(*const F)[P3] = reinterpret_cast<longlong2(*)[P3]>(U);
+        bool done = false;
+        if constexpr (MODE == 1) {
+            // the whole instance on the scale of its last iterate, where that is known
+            const InstDesc& I = insts[item.inst];
+            const InstState s = st[item.inst];
+            const FxH2 hh(I.h);
+            if (s.status == HELM_ST_ACTIVE && hh.pow2 && s.uex > 0 && s.it > 0 && hh.usable(s.uex + 2) && I.n <= 1023) {
+                R r2, em;
+                int ex;
+                done = residual3d_tile_scaled<R, DAMP>(I, s, item, F, sx, hh.add, r2, em, ex);
+                if (done)
+                    tile_done<R>(I, st + item.inst, (item.tz * I.res_ty + item.ty) * I.res_tx + item.tx, r2, em, MODE,
+                                 st, c, ex);
+                __syncthreads();
+            }
+        }
+        if (!done) residual3d_tile_fx<R, MODE, DAMP>(insts, st, item, F, sx, c);
         __syncthreads();
     }
 }

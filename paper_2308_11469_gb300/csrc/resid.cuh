@@ -204,15 +204,18 @@ __device__ void instance_last(const InstDesc& I, InstState* stp, int mode, const
     block_reduce_v<double, VT>(ta, tm, fa, fm, sa, sm, mode == 0);
     if (threadIdx.x == 0) {
         finalize(I, stp, fa, fm, mode);
-        *I.count = 0u;
+        I.count[0] = 0u;
+        stp->uex = (int)__ldcg(I.count + 1);
+        I.count[1] = 0u;
     }
     if (c.ctrl) step_arrive(st_all, c);
 }
 
-// Write this tile's partials; the last tile of the instance reduces them all.
+// Write this tile's partials; the last tile of the instance reduces them all.  ex: the largest
+// biased exponent of the iterate on the tile (3D).
 template <typename T>
 __device__ void tile_done(const InstDesc& I, InstState* stp, int tile, T ta0, T tm0, int mode,
-                          const InstState* st_all, const StepCtl& c)
+                          const InstState* st_all, const StepCtl& c, int ex = 0)
 {
     __shared__ double sa[NTH / 32], sm[NTH / 32];
     __shared__ int last;
@@ -221,6 +224,7 @@ __device__ void tile_done(const InstDesc& I, InstState* stp, int tile, T ta0, T 
     if (threadIdx.x == 0) {
         I.part[tile] = a;
         I.part[I.nres_blocks + tile] = m;
+        if (ex) atomicMax(I.count + 1, (unsigned)ex);
         __threadfence();
         const unsigned prev = atomicAdd(I.count, 1u);
         last = (prev == (unsigned)(I.nres_blocks - 1));
