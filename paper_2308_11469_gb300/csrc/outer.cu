@@ -229,7 +229,7 @@ k_upres2d(const InstDesc* __restrict__ insts, InstState* __restrict__ st,
     constexpr int UW = TX + 2, UH = TY + 2;
     static_assert(H % 2 == 1 && TX % 2 == 0 && TY % 2 == 0, "gx0, gy0 even");
     typedef Planes<W> PL;
-    static_assert(TY == T2Y && NTH % NTU == 0, "one residual tile, NTH / NTU map threads per thread");
+    static_assert(TY == T2Y && NTH == NTU, "one residual tile, a thread of its map per thread");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ double sa[NTH / 32], sm[NTH / 32];
     __shared__ int last;
@@ -523,7 +523,7 @@ k_upres2d(const InstDesc* __restrict__ insts, InstState* __restrict__ st,
     }
     // the tile's partials in k_residual2d's order, then the instance's ticket
     double ra = 0.0, rm = 0.0;
-    block_reduce_v<R, VT>(r2, em, ra, rm, sa, sm, false);
+    block_reduce<R>(r2[0], em[0], ra, rm, sa, sm, false);
     const int nb = I.nres_blocks;
     if (threadIdx.x == 0) {
         const int tile = by * I.res_tx + bx;
@@ -534,7 +534,7 @@ k_upres2d(const InstDesc* __restrict__ insts, InstState* __restrict__ st,
     }
     __syncthreads();
     if (!last) return;
-    instance_last<VT>(I, stp, 1, st, ctl, sa, sm);
+    instance_last(I, stp, 1, st, ctl, sa, sm);
 }
 
 // ---------------------------------------------------------------------------

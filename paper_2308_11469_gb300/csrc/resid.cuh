@@ -1,6 +1,8 @@
 // Pieces of the outer (FP64) iteration that its kernels share (outer.cu, small2d.cu): the
 // status rule, fixed-order reductions, the step control and the per-node residual.
 #pragma once
+#include <type_traits>
+
 #include "launch.h"
 #include "fp_bits.cuh"
 #include "fixed_lap.cuh"
@@ -32,7 +34,7 @@ template <> struct Inner<double> {
 // relres_N = ||r_N|| / ||b||, b the lifted right-hand side (f minus the wall values'
 // contribution to the stencil): with the paper's zero start r_0 = b and relres_0 = 1; a
 // starting iterate that already solves the system well starts with a small relres.
-// mode 0: `second` is ||b||^2; mode 1: it is max |e|^2.
+// mode 0: `second` is ||b||^2 (mode 1: not used; instance_last records the increment's norm).
 // The outcome after step N (0: the start) with relative residual rel, into s (run, rmin,
 // prev, status).
 __device__ __forceinline__ void status_rule(const InstDesc& I, InstState& s, double rel, int N, bool zero)
@@ -69,57 +71,90 @@ __device__ void finalize(const InstDesc& I, InstState* stp, double norm2, double
         s.it += 1;
         N = s.it;
         rel = norm / s.norm0;
-        I.einf[N - 1] = sqrt(second);
     }
     I.hist[N] = rel;
     status_rule(I, s, rel, N, mode == 0 && norm == 0.0);
     *stp = s;
 }
 
-// Block-wide sums / maxima in a fixed order (xor-shuffle in T, then the warps' values in
-// order, in FP64).  `sum2`: the second channel is summed (mode 0, ||b||^2) instead of
-// maximised (max |e|^2).  Mode 1 reduces its complex64-derived values in FP32, keeping the
-// shuffle tree off the FP64 pipe; the result (thread 0) is FP64 either way.
-// VT > 1: each real thread stands for VT threads of a map VT times the block's size (real
-// thread j for the threads j + blockDim v); virtual warp w + (blockDim / 32) v reduces on
-// real warp w with the same shuffle tree, and the virtual warps' values are summed in
-// order, so the result is that of the larger block.
-template <typename T, int VT = 1>
-__device__ __forceinline__ void block_reduce_v(const T* av, const T* mv, double& ra, double& rm,
-                                               double* sa, double* sm, bool sum2)
+// float -> double, exact for every value, without the FP64 pipe unless it is subnormal
+__device__ __forceinline__ double widen_any(float f)
 {
-    const int nw = (int)(blockDim.x >> 5);
-#pragma unroll
-    for (int v = 0; v < VT; ++v) {
-        T a = av[v], m = mv[v];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            a += __shfl_xor_sync(0xffffffffu, a, o);
-            const T mo = __shfl_xor_sync(0xffffffffu, m, o);
-            m = sum2 ? m + mo : (m > mo ? m : mo);
-        }
-        const int w = (threadIdx.x >> 5) + nw * v;
-        if ((threadIdx.x & 31) == 0) {
-            sa[w] = (double)a;
-            sm[w] = (double)m;
-        }
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        ra = 0.0;
-        rm = 0.0;
-        for (int i = 0; i < nw * VT; ++i) {
-            ra += sa[i];
-            rm = sum2 ? rm + sm[i] : fmax(rm, sm[i]);
-        }
-    }
+    const unsigned mag = __float_as_uint(f) & 0x7fffffffu;
+    return mag - 1u < 0x007fffffu ? (double)f : f2d_bits(f);
 }
 
+// Sum of n floats in order, kept as an unevaluated pair (error-free two-sums: exact to 2^-48 of
+// the sum) so that only the last addition is FP64: a warp's FP64 instruction holds its pipe for
+// 64 clocks, and a thread adding eight warps' values in FP64 kept the whole CTA waiting.
+__device__ __forceinline__ double sum_floats(const float* p, int n)
+{
+    float s = 0.f, c = 0.f;
+    for (int i = 0; i < n; ++i) {
+        const float v = p[i], t = s + v, bb = t - s;
+        c += (s - (t - bb)) + (v - bb);
+        s = t;
+    }
+    return isfinite(s) ? widen_any(s) + widen_any(c) : widen_any(s);
+}
+
+// Block-wide sums / maxima in a fixed order (xor-shuffle in T, then the warps' values in
+// order, in FP64).  `sum2`: the second channel is summed (mode 0, ||b||^2) instead of
+// maximised (max |e|^2, non-negative: FP64 maxima are taken on the bits).  Mode 1 reduces its
+// complex64-derived values in FP32, keeping the shuffle tree off the FP64 pipe; the result
+// (thread 0) is FP64 either way.  live: only the first `live` warps hold values.
 template <typename T>
 __device__ __forceinline__ void block_reduce(T a, T m, double& ra, double& rm, double* sa, double* sm,
-                                             bool sum2)
+                                             bool sum2, int live = 32)
 {
-    block_reduce_v<T, 1>(&a, &m, ra, rm, sa, sm, sum2);
+    const int nw = min((int)(blockDim.x >> 5), live), w = threadIdx.x >> 5;
+    if constexpr (std::is_same<T, float>::value) {
+        float* const fa = reinterpret_cast<float*>(sa);
+        float* const fm = reinterpret_cast<float*>(sm);
+        if (w < nw) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                a += __shfl_xor_sync(0xffffffffu, a, o);
+                const float mo = __shfl_xor_sync(0xffffffffu, m, o);
+                m = m > mo ? m : mo;
+            }
+            if ((threadIdx.x & 31) == 0) {
+                fa[w] = a;
+                fm[w] = m;
+            }
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            float mf = 0.f;
+            for (int i = 0; i < nw; ++i) mf = fmaxf(mf, fm[i]);
+            ra = sum_floats(fa, nw);
+            rm = widen_any(mf);
+        }
+    } else {
+        if (w < nw) {
+            long long mi = __double_as_longlong(m);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                a += __shfl_xor_sync(0xffffffffu, a, o);
+                if (sum2) m += __shfl_xor_sync(0xffffffffu, m, o);
+                else mi = max(mi, __shfl_xor_sync(0xffffffffu, mi, o));
+            }
+            if ((threadIdx.x & 31) == 0) {
+                sa[w] = a;
+                sm[w] = sum2 ? m : __longlong_as_double(mi);
+            }
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            ra = sa[0];
+            rm = sm[0];
+            for (int i = 1; i < nw; ++i) {
+                ra += sa[i];
+                rm = sum2 ? rm + sm[i]
+                          : __longlong_as_double(max(__double_as_longlong(rm), __double_as_longlong(sm[i])));
+            }
+        }
+    }
 }
 
 // End of an outer step, run by one whole CTA once every instance's status is final: is
@@ -178,30 +213,29 @@ __device__ void step_arrive(const InstState* st, const StepCtl& c)
 // leaves sums and maxima of non-negative values unchanged), so a launch with larger CTAs
 // reduces in the same order as the residual kernels.
 // sa, sm: shared scratch of one double per warp of the CTA.
-// VT: threads of the NTH-thread order per real thread (blockDim.x = NTH / VT; sa, sm hold
-// NTH / 32 doubles).
-template <int VT = 1>
 __device__ void instance_last(const InstDesc& I, InstState* stp, int mode, const InstState* st_all,
                               const StepCtl& c, double* sa, double* sm)
 {
     const int nb = I.nres_blocks;
     __threadfence();
-    double ta[VT], tm[VT];
-#pragma unroll
-    for (int v = 0; v < VT; ++v) {
-        ta[v] = 0.0;
-        tm[v] = 0.0;
-        const int t = threadIdx.x + (int)blockDim.x * v;
-        if (t < NTH)
-            for (int b = t; b < nb; b += NTH) {
-                ta[v] += __ldcg(I.part + b);
-                const double x = __ldcg(I.part + nb + b);
-                tm[v] = (mode == 0) ? tm[v] + x : fmax(tm[v], x);
-            }
-    }
+    double ta = 0.0, tm = 0.0;
+    long long ti = 0;
+    if ((int)threadIdx.x < NTH)
+        for (int b = threadIdx.x; b < nb; b += NTH) {
+            ta += __ldcg(I.part + b);
+            const double x = __ldcg(I.part + nb + b);
+            if (mode == 0) tm += x;
+            else ti = max(ti, __double_as_longlong(x));
+        }
+    if (mode != 0) tm = __longlong_as_double(ti);
+    const int it = stp->it;
     __syncthreads();
     double fa = 0.0, fm = 0.0;
-    block_reduce_v<double, VT>(ta, tm, fa, fm, sa, sm, mode == 0);
+    block_reduce<double>(ta, tm, fa, fm, sa, sm, mode == 0, (min(nb, NTH) + 31) >> 5);
+    if (threadIdx.x == 0) sm[0] = fm;
+    __syncthreads();
+    // the increment's norm by another warp, beside relres
+    if (mode != 0 && threadIdx.x == 32) I.einf[it] = sqrt(sm[0]);
     if (threadIdx.x == 0) {
         finalize(I, stp, fa, fm, mode);
         I.count[0] = 0u;
@@ -231,7 +265,7 @@ __device__ void tile_done(const InstDesc& I, InstState* stp, int tile, T ta0, T 
     }
     __syncthreads();
     if (!last) return;
-    instance_last<1>(I, stp, mode, st_all, c, sa, sm);
+    instance_last(I, stp, mode, st_all, c, sa, sm);
 }
 
 // r = f - (Delta_h + k^2 + i p) u at one node: f - k^2 u - (numerator) / h^2, the
@@ -276,13 +310,6 @@ __device__ __forceinline__ double2 helm_resid2d_g(double2 c, longlong2 FC, longl
         r.y = fma(c.x, -damp, r.y);
     }
     return r;
-}
-
-// float -> double, exact for every value, without the FP64 pipe unless it is subnormal
-__device__ __forceinline__ double widen_any(float f)
-{
-    const unsigned mag = __float_as_uint(f) & 0x7fffffffu;
-    return mag - 1u < 0x007fffffu ? (double)f : f2d_bits(f);
 }
 
 // scale exponent of a window from its largest biased exponent (see fixed_lap.cuh); -1:

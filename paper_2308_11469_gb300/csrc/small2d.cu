@@ -217,11 +217,10 @@ k_small2d(const InstDesc* __restrict__ insts, InstState* __restrict__ st, const 
             if (warp == 0) {
                 double a = 0.0;
                 float mf = 0.f;
-                if (lane < NT)
-                    for (int w = 0; w < 8; ++w) {
-                        a += widen_any(sa[8 * lane + w]);
-                        mf = fmaxf(mf, sm[8 * lane + w]);
-                    }
+                if (lane < NT) {
+                    a = sum_floats(sa + 8 * lane, 8);
+                    for (int w = 0; w < 8; ++w) mf = fmaxf(mf, sm[8 * lane + w]);
+                }
 #pragma unroll
                 for (int o = NT / 2; o > 0; o >>= 1) {
                     a += __shfl_xor_sync(0xffffffffu, a, o);
