@@ -484,11 +484,11 @@ constexpr int AN_TAIL_TOP_F = 64;
 constexpr int AN_TAIL_TOP_D = 16;
 constexpr int AN_TAIL_MAX = 4;
 
-struct AnTail {
+template <typename R> struct AnTail {
     int L, nu1, nu2, load_e, m;
-    double sigma;
+    R sigma;
     AnGeo geo[AN_TAIL_MAX];
-    double h[AN_TAIL_MAX], dinv[AN_TAIL_MAX], ih2[AN_TAIL_MAX];
+    R h[AN_TAIL_MAX], dinv[AN_TAIL_MAX], ih2[AN_TAIL_MAX];       // (no conversions in the kernel)
     const double* At;
     const int* map;
 };
@@ -507,7 +507,7 @@ size_t an_tail_bytes(const int* ns, int L, int m)
 
 template <typename R>
 __global__ void __launch_bounds__(1024, 1)
-k_an_tail(typename CX<R>::T* __restrict__ eg, const typename CX<R>::T* __restrict__ rg, AnTail T)
+k_an_tail(typename CX<R>::T* __restrict__ eg, const typename CX<R>::T* __restrict__ rg, AnTail<R> T)
 {
     typedef typename CX<R>::T c2;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -546,11 +546,11 @@ k_an_tail(typename CX<R>::T* __restrict__ eg, const typename CX<R>::T* __restric
     }
     asm volatile("cp.async.wait_all;\n" ::: "memory");
     __syncthreads();
-    const R sig = (R)T.sigma;
+    const R sig = T.sigma;
     // descent
     for (int l = 0; l + 1 < T.L; ++l) {
         const AnGeo g = T.geo[l], gc = T.geo[l + 1];
-        const R h = (R)T.h[l], dinv = (R)T.dinv[l];
+        const R h = T.h[l], dinv = T.dinv[l];
         const int n = g.n, W = n + 2;
         const AnWin<R> w = win(l);
         for (int k = 0; k < 2 * T.nu1; ++k) {
@@ -558,7 +558,7 @@ k_an_tail(typename CX<R>::T* __restrict__ eg, const typename CX<R>::T* __restric
             __syncthreads();
         }
         const bool zero = T.nu1 == 0 && (l > 0 || !T.load_e);
-        const R ih2 = (R)T.ih2[l];
+        const R ih2 = T.ih2[l];
         const unsigned m = an_magic(n + 1);
         c2* const P[2] = {Res, Res + (n + 1) * (W >> 1)};
         for (int q = threadIdx.x; q < (n + 1) * (n + 1); q += blockDim.x) {
@@ -594,7 +594,7 @@ k_an_tail(typename CX<R>::T* __restrict__ eg, const typename CX<R>::T* __restric
     for (int l = T.L - 2; l >= 0; --l) {
         const AnGeo g = T.geo[l];
         const int n = g.n;
-        const R h = (R)T.h[l], dinv = (R)T.dinv[l];
+        const R h = T.h[l], dinv = T.dinv[l];
         const AnWin<R> w = win(l), wc = win(l + 1);
         const unsigned m = an_magic(n + 1);
         for (int q = threadIdx.x; q < (n + 1) * (n + 1); q += blockDim.x) {
@@ -1242,21 +1242,21 @@ helm_status an_vcycle(helm_annulus* a, int l, bool zero)
     const auto& L = a->lev[l];
     cudaStream_t s = a->ls;
     if (l == a->t0) {                      // this level and all coarser ones in one CTA
-        AnTail T{};
+        AnTail<R> T{};
         T.L = (int)a->lev.size() - l;
         T.nu1 = a->nu1;
         T.nu2 = a->nu2;
         T.load_e = zero ? 0 : 1;
         T.m = a->m;
-        T.sigma = a->sigma;
+        T.sigma = (R)a->sigma;
         T.At = a->At;
         T.map = a->map;
         for (int i = 0; i < T.L; ++i) {
             const auto& V = a->lev[l + i];
             T.geo[i] = an_geo(V);
-            T.h[i] = V.h;
-            T.dinv[i] = 1.0 / (4.0 + a->sigma * V.h * V.h);
-            T.ih2[i] = (double)((R)1 / ((R)V.h * (R)V.h));
+            T.h[i] = (R)V.h;
+            T.dinv[i] = (R)(1.0 / (4.0 + a->sigma * V.h * V.h));
+            T.ih2[i] = (R)1 / ((R)V.h * (R)V.h);
         }
         for (int i = T.L; i < AN_TAIL_MAX; ++i) T.geo[i] = AnGeo{0, 0, 0, 0, 0};
         AN_CK(launch_k(k_an_tail<R>, dim3(1), dim3(1024), a->tail_bytes, s, (c2*)L.e, (const c2*)L.rhs, T));

@@ -33,6 +33,10 @@ struct LevelDesc {
     int pad_;
     double h;     // spacing 2^l h
     double dinv;  // 1 / (2D + sigma h^2): the local solve's factor (host-computed)
+    double h2;    // h^2
+    // h, h^2, dinv and 1 / h^2 in FP32, rounded on the host: a warp's conversion or product in
+    // FP64 holds its pipe for 64 clocks, and every thread of every complex64 kernel made three
+    float hf, h2f, dinvf, ih2f;
     void* e;      // padded iterate of (Delta_h - sigma) e = rhs (final iterate of a V-cycle)
     void* rhs;    // right-hand side (same indexing as e)
     void* e2;     // 2D fused path: the pre-smoothed iterate (same indexing as e)
@@ -54,6 +58,7 @@ struct InstDesc {
     double h, k2, tol;
     double ih2, cdiag;          // 1/h^2 and k^2 - 2D/h^2 (the stencil's diagonal)
     double sigma;               // alpha - k^2 >= 0: inner operator Delta_h - sigma
+    float sigf;                 // sigma in FP32
     double damp;                // p >= 0: damping term i p u of Delta u + (i p + k^2) u = f
     double2* u[2];              // u[0] = caller's array, u[1] = library buffer
     const double2* f;
@@ -86,6 +91,23 @@ struct MgItem {
 struct ResItem {
     int inst;
     int tx, ty, tz;
+};
+
+// a level's constants in the precision of a kernel
+template <typename R> struct LevC;
+template <> struct LevC<float> {
+    __host__ __device__ static float h(const LevelDesc& L) { return L.hf; }
+    __host__ __device__ static float h2(const LevelDesc& L) { return L.h2f; }
+    __host__ __device__ static float dinv(const LevelDesc& L) { return L.dinvf; }
+    __host__ __device__ static float ih2(const LevelDesc& L) { return L.ih2f; }
+    __host__ __device__ static float sigma(const InstDesc& I) { return I.sigf; }
+};
+template <> struct LevC<double> {
+    __host__ __device__ static double h(const LevelDesc& L) { return L.h; }
+    __host__ __device__ static double h2(const LevelDesc& L) { return L.h2; }
+    __host__ __device__ static double dinv(const LevelDesc& L) { return L.dinv; }
+    __host__ __device__ static double ih2(const LevelDesc& L) { return 1.0 / L.h2; }
+    __host__ __device__ static double sigma(const InstDesc& I) { return I.sigma; }
 };
 
 template <typename R> struct C2;

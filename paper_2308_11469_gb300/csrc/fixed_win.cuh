@@ -99,7 +99,7 @@ struct FxH2 {
     double h2;
     int add;
     bool pow2;
-    __device__ explicit FxH2(double h) : h2(h * h)
+    __device__ explicit FxH2(double h2_) : h2(h2_)
     {
         const unsigned long long b = fx_bits(h2);
         pow2 = (b & 0x000fffffffffffffull) == 0ull;

@@ -17,7 +17,16 @@ constexpr int TAIL_N_3D = 15;
 inline void set_shift(InstDesc& d, double sigma)
 {
     d.sigma = sigma;
-    for (int l = 0; l < d.nlev; ++l) d.lev[l].dinv = 1.0 / (2.0 * d.D + sigma * d.lev[l].h * d.lev[l].h);
+    d.sigf = (float)sigma;
+    for (int l = 0; l < d.nlev; ++l) {
+        LevelDesc& L = d.lev[l];
+        L.dinv = 1.0 / (2.0 * d.D + sigma * L.h * L.h);
+        L.h2 = L.h * L.h;
+        L.hf = (float)L.h;
+        L.h2f = (float)L.h2;
+        L.dinvf = (float)L.dinv;
+        L.ih2f = (float)(1.0 / L.h2);
+    }
 }
 
 inline int tail_top(int D, int prec_is_fp64)

@@ -372,8 +372,8 @@ k_upres2d(const InstDesc* __restrict__ insts, InstState* __restrict__ st,
             E1w[q] = v;
         }
         __syncthreads();
-        const R h21 = (R)(C.h * C.h);
-        const R dinv1 = (R)C.dinv;
+        const R h21 = LevC<R>::h2(C);
+        const R dinv1 = LevC<R>::dinv(C);
 #pragma unroll 1
         for (int sw = 1; sw <= 2 * NU; ++sw) {
             const int color = (sw - 1) & 1, ring1 = 2 * NU - sw;
@@ -424,8 +424,8 @@ k_upres2d(const InstDesc* __restrict__ insts, InstState* __restrict__ st,
         *Ep = v;
     }
     __syncthreads();
-    const R h2 = (R)(L.h * L.h);
-    const R dinv = (R)L.dinv;
+    const R h2 = LevC<R>::h2(L);
+    const R dinv = LevC<R>::dinv(L);
     sweeps_flat<R, W, TX, TY, NTU, 2 * NU, 2 * NU>(E0, E1, R0, R1, gx0, gy0, x0, y0, n, h2, dinv);
     if (UPRES_LATE_U) {                          // the rhs planes and Cs are dead: u_N there
         stage_u();
@@ -864,7 +864,7 @@ k_residual3d(const InstDesc* __restrict__ insts, InstState* __restrict__ st,
             // the whole instance on the scale of its last iterate, where that is known
             const InstDesc& I = insts[item.inst];
             const InstState s = st[item.inst];
-            const FxH2 hh(I.h);
+            const FxH2 hh(I.lev[0].h2);
             if (s.status == HELM_ST_ACTIVE && hh.pow2 && s.uex > 0 && s.it > 0 && hh.usable(s.uex + 2) && I.n <= 1023) {
                 R r2, em;
                 int ex;

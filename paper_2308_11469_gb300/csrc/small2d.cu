@@ -72,7 +72,7 @@ k_small2d(const InstDesc* __restrict__ insts, InstState* __restrict__ st, const 
     const MgItem item = items[blockIdx.x / CS];
     const InstDesc& I = insts[item.inst];
     const LevelDesc L0 = I.lev[0];
-    const float sigma = (float)I.sigma;
+    const float sigma = I.sigf;
     // host-written tables before the wait
     if constexpr (tail_exact<2, float, N0>())
         for (int i = tid; i < XTAB_FLOATS; i += TNT) xscr[i] = xtab[i];
@@ -128,7 +128,7 @@ k_small2d(const InstDesc* __restrict__ insts, InstState* __restrict__ st, const 
                 // is solved exactly is overwritten)
                 if (c == 0) t_clear<2, float, N0>(base);
                 __syncthreads();
-                t_vcycle<2, float, N0, TNT / 32>(base, (float)L0.h, sigma, &I.lev[0], nu1, nu2, xscr, c == 0);
+                t_vcycle<2, float, N0, TNT / 32>(base, L0.hf, sigma, &I.lev[0], nu1, nu2, xscr, c == 0);
             }
             // u_{N+1} = u_N + e_N on the band's window, and its largest exponents per tile
             if (tid < NT) {

@@ -57,7 +57,7 @@ __device__ __noinline__ bool tail_fx31(const LevelDesc& L0, const double2* __res
     const bool own = t < N * N;
     const int y = t / N + 1, x = t % N + 1, o = y * S + x;
     double2* __restrict__ ge = (double2*)L0.e;
-    const FxH2 hh(L0.h);
+    const FxH2 hh(L0.h2);
     double2 r = make_double2(0.0, 0.0), e = r;
     if (own) {
         r = gr[(size_t)y * L0.pitch + x];
@@ -227,7 +227,7 @@ k_tail(const InstDesc* __restrict__ insts, const InstState* __restrict__ st,
         }
     }
     __syncthreads();
-    t_vcycle<D, R, N0, TNT / 32>(base, (R)L0.h, (R)sigma, &insts[item.inst].lev[item.level], nu1, nu2,
+    t_vcycle<D, R, N0, TNT / 32>(base, LevC<R>::h(L0), LevC<R>::sigma(insts[item.inst]), &insts[item.inst].lev[item.level], nu1, nu2,
                                  xscr, !le);
     c2* __restrict__ go = (c2*)L0.e;
     for (int r = warp; r < ROWS; r += TNT / 32) {
@@ -494,10 +494,10 @@ k_ctail(const InstDesc* __restrict__ insts, const InstState* __restrict__ st,
     // tables, and the coarse iterate windows cleared (their rings and outer rows stay zero)
     const MgItem item = items[blockIdx.x / CT_CS];
     const LevelDesc LA = insts[item.inst].lev[item.level];
-    const float dinvA = (float)LA.dinv;
-    const float dinvB = (float)insts[item.inst].lev[item.level + 1].dinv;
-    const float dinvC = (float)insts[item.inst].lev[item.level + 2].dinv;
-    const float sig = (float)insts[item.inst].sigma;
+    const float dinvA = LA.dinvf;
+    const float dinvB = insts[item.inst].lev[item.level + 1].dinvf;
+    const float dinvC = insts[item.inst].lev[item.level + 2].dinvf;
+    const float sig = insts[item.inst].sigf;
     {
         constexpr int NT4 = XTAB_FLOATS / 4;
         const float4* tab = reinterpret_cast<const float4*>(g_xtab);
@@ -543,7 +543,7 @@ k_ctail(const InstDesc* __restrict__ insts, const InstState* __restrict__ st,
     }
     __syncthreads();
     ct_arrive_relaxed();
-    const float hA = (float)LA.h;
+    const float hA = LA.hf;
     x_solve(EX, RX, xscr, 8.f * hA, sig);
     // ascent: level 63 on its window
     ct_prolong<CT_NC>(EC, loEC, EX, 0, loEC, loEC + W::EC_ROWS - 1);

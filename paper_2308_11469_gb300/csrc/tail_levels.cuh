@@ -528,7 +528,7 @@ __device__ void t_vcycle(typename C2<R>::T* base, R h, R sig, const LevelDesc* l
             constexpr int S = 3;
             constexpr int o = ((D == 3) ? (S + 1) : 1) * S + Lv<D, 1>::HE;  // the single node
             const c2 rr = Rr[o];
-            const R c = -(h * h) * (R)lv->dinv;      // -h^2 / (2D + sigma h^2)
+            const R c = -(h * h) * LevC<R>::dinv(*lv);      // -h^2 / (2D + sigma h^2)
             c2 v;
             v.x = c * rr.x;
             v.y = c * rr.y;
@@ -540,7 +540,7 @@ __device__ void t_vcycle(typename C2<R>::T* base, R h, R sig, const LevelDesc* l
         c2* Ec = base + 2 * Lv<D, N>::SZ;
         c2* Rc = Ec + Lv<D, NC>::SZ;
         const R h2 = h * h;
-        const R dinv = (R)lv->dinv;                     // 1 / (2D + sigma h^2)
+        const R dinv = LevC<R>::dinv(*lv);                     // 1 / (2D + sigma h^2)
         for (int s = 0; s < nu1; ++s) {
             t_sweep<D, R, N, NWARPS>(E, Rr, h2, dinv, 0);
             tsync<NWARPS>();

@@ -50,8 +50,8 @@ k_rbgs(const InstDesc* __restrict__ insts, const InstState* __restrict__ st,
     const c2* __restrict__ r = (const c2*)lev_rhs(L, item.level, sv.it);
     const long P = L.pitch;
     const long PL = (long)L.pitch * L.rows;
-    const R h2 = (R)(L.h * L.h);
-    const R inv = (R)L.dinv;                       // 1 / (2D + sigma h^2)
+    const R h2 = LevC<R>::h2(L);
+    const R inv = LevC<R>::dinv(L);                       // 1 / (2D + sigma h^2)
     // mode 2: the iterate of every level is zero; mode 1: only levels > 0 are (their
     // iterate was cleared by the restriction); mode 0: plain half-sweep.
     const bool zi = (mode == 2) || (mode == 1 && item.level > 0);
@@ -186,8 +186,8 @@ k_rbgs3p(const InstDesc* __restrict__ insts, const InstState* __restrict__ st,
         }
         commit();
     }
-    const R h2 = (R)(Lv.h * Lv.h);
-    const R inv = (R)Lv.dinv;
+    const R h2 = LevC<R>::h2(Lv);
+    const R inv = LevC<R>::dinv(Lv);
     const int y = y0 + w;
     const int jmax = (n - 1) >> 1;
     for (int p = z0; p < z1; ++p) {
@@ -253,8 +253,8 @@ k_restrict(const InstDesc* __restrict__ insts, const InstState* __restrict__ st,
     c2* __restrict__ ce = (c2*)C.e;
     const long P = F.pitch;
     const long PL = (long)F.pitch * F.rows;
-    const R ih2 = (R)(1.0 / (F.h * F.h));
-    const R sig = (R)insts[item.inst].sigma;
+    const R ih2 = LevC<R>::ih2(F);
+    const R sig = LevC<R>::sigma(insts[item.inst]);
     const R scale = (D == 3) ? (R)(1.0 / 64.0) : (R)(1.0 / 16.0);
     const bool ez = (mode == 2) || (mode == 1 && item.level > 0);
     // a warp per coarse row (Y, Z), its lanes over X

@@ -127,9 +127,10 @@ k_down2d(const InstDesc* __restrict__ insts, const InstState* __restrict__ st,
         // scale, four times the largest value's (the residual of an iterate grown by nu1 sweeps
         // is below 25 times it, a row of the full weighting four times that)
         __shared__ int sx[NW];
-        const FxH2 hh(L.h);
+        const FxH2 hh(L.h2);
         int ex = 0;
-        if (sigma == 0.0)
+        const bool plain = fx_bits(sigma) << 1 == 0;   // no shift
+        if (plain)
             for (int q = threadIdx.x; q < W * HH; q += NT) {
                 const int ly = q / W, lx = q - ly * W, o = PL::at(lx, ly);
                 const bool c = (lx + ly + cpar) & 1;
@@ -138,7 +139,7 @@ k_down2d(const InstDesc* __restrict__ insts, const InstState* __restrict__ st,
                 if (!zero) ex = max(ex, fx_exp2((c ? E1 : E0)[o]));
             }
         const int em = block_max_exp<NW * 32>(ex, sx) + 2;
-        if (sigma == 0.0 && hh.usable(em)) {
+        if (plain && hh.usable(em)) {
             longlong2* const F0 = reinterpret_cast<longlong2*>(E0);
             longlong2* const F1 = reinterpret_cast<longlong2*>(E1);
             longlong2* const G0 = reinterpret_cast<longlong2*>(R0);
@@ -202,9 +203,9 @@ k_down2d(const InstDesc* __restrict__ insts, const InstState* __restrict__ st,
         }
     }
     __syncthreads();
-    const R h2 = (R)(L.h * L.h);
-    const R dinv = (R)L.dinv;                      // 1 / (4 + sigma h^2)
-    const R sig = (R)sigma;
+    const R h2 = LevC<R>::h2(L);
+    const R dinv = LevC<R>::dinv(L);                      // 1 / (4 + sigma h^2)
+    const R sig = LevC<R>::sigma(insts[item.inst]);
     sweeps_flat<R, W, TX, TY, NT, 2 * NU + 1, 2 * NU>(E0, E1, R0, R1, gx0, gy0, x0, y0, n, h2, dinv);
     // no pre-smoothing from a zero iterate: e2 stays zero (the ascent kernel knows it and
     // does not read it) and the residual is rhs itself
@@ -356,9 +357,9 @@ k_up2d(const InstDesc* __restrict__ insts, const InstState* __restrict__ st,
         // fixed point (fixed_win.cuh): after the correction the iterate is at most twice the
         // window's largest value, after nu2 sweeps at most 2 + nu2 / 2 times it
         __shared__ int sx[NW];
-        const FxH2 hh(L.h);
+        const FxH2 hh(L.h2);
         int ex = 0;
-        const bool plain = L.dinv == 0.25;         // no shift
+        const bool plain = fx_bits(L.dinv) == fx_bits(0.25);         // no shift
         if (plain) {
             for (int q = threadIdx.x; q < CW * CH; q += NT) ex = max(ex, fx_exp2(Cs[q]));
             for (int q = threadIdx.x; q < W * HH; q += NT) {
@@ -430,8 +431,8 @@ k_up2d(const InstDesc* __restrict__ insts, const InstState* __restrict__ st,
         *Ep = v;
     }
     __syncthreads();
-    const R h2 = (R)(L.h * L.h);
-    const R dinv = (R)L.dinv;
+    const R h2 = LevC<R>::h2(L);
+    const R dinv = LevC<R>::dinv(L);
     sweeps_flat<R, W, TX, TY, NT, 2 * NU - 1, 2 * NU>(E0, E1, R0, R1, gx0, gy0, x0, y0, n, h2, dinv);
     c2* __restrict__ ge = (c2*)L.e;
     for (int ty = threadIdx.x >> 5; ty < TY; ty += NW) {

@@ -48,7 +48,7 @@ k_rbgs64(const InstDesc* __restrict__ insts, const InstState* __restrict__ st, c
     const int n = G.n, half = (n + 1) >> 1, total = n * n * half;
     double2* __restrict__ e = (double2*)L.e;
     const double2* __restrict__ r = (const double2*)lev_rhs(L, item.level, sv.it);
-    const FxH2 hh(L.h);
+    const FxH2 hh(L.h2);
     const double inv = L.dinv;                     // 1 / (6 + sigma h^2)
     const bool zi = (mode == 2) || (mode == 1 && item.level > 0);
     for (int t = blockIdx.x * K3_NT + threadIdx.x; t < total; t += gridDim.x * K3_NT) {
@@ -111,7 +111,7 @@ k_restrict64(const InstDesc* __restrict__ insts, const InstState* __restrict__ s
     double2* __restrict__ ce = (double2*)Cd.e;
     const bool ez = (mode == 2) || (mode == 1 && item.level > 0);
     const double sig = insts[item.inst].sigma;
-    const double ih2 = ez ? 0.0 : 1.0 / (Fd.h * Fd.h);     // (a division costs a warp 1300 clocks)
+    const double ih2 = ez ? 0.0 : 1.0 / Fd.h2;     // (a division costs a warp 1300 clocks)
     for (int t = blockIdx.x * K3_NT + threadIdx.x; t < total; t += gridDim.x * K3_NT) {
         const int row = t / nc, X = t - row * nc + 1, Y = row % nc + 1, Z = row / nc + 1;
         const long oc = C.row(Y, Z) + C.x(X);
