@@ -26,11 +26,13 @@
 #include "launch.h"
 #include "pdl.cuh"
 #include "fp_bits.cuh"
+#include "fixed_win.cuh"
 
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <type_traits>
 #include <vector>
 
 namespace helm {
@@ -47,6 +49,7 @@ enum : unsigned char { AN_PDE = 0, AN_EDGE = 1, AN_HOLE = 2 };
 template <typename R> struct CX;
 template <> struct CX<float> { typedef float2 T; };
 template <> struct CX<double> { typedef double2 T; };
+template <> struct CX<long long> { typedef longlong2 T; };     // fixed-point windows
 
 __host__ __device__ constexpr size_t an_a16(size_t b) { return (b + 15) & ~(size_t)15; }
 
@@ -282,6 +285,122 @@ __device__ __forceinline__ typename CX<R>::T an_restrict_node(const AnGeo& gc, i
     return v;
 }
 
+// ---- FP64 windows in 64-bit fixed point (fixed_win.cuh) ----
+// PDE rows hold h^2 rhs, EDGE rows h rhs: e = mean of the inward neighbours + h rhs there.
+// A 256^2 solve with V(2,2), 53 steps: 6.10 -> 3.95 ms.  The cycle's error against extended
+// precision, N = 128 .. 512, two holes, rough / smooth / edge data: lower than the FP64
+// windows' in 33 of 36 norms, the others (l2, 512, rough) 1.16e-15 against 1.00e-15 at most.
+// sigma > 0, more sweeps, and windows out of the scale's range keep the FP64 code.  Three or four
+// descent sweeps would fit on a scale one bit coarser, which raised that error in 4 of 36 norms
+// (by up to 1.7): they stay in FP64.
+constexpr int AN_FX_NU1 = 2, AN_FX_NU2 = 4;      // most sweeps of a window in fixed point
+
+// this thread's staged words (an_stage's numbering) of the window: their largest exponent
+__device__ __forceinline__ int an_fx_exp(const AnWin<double>& w, const AnGeo& g, int rows, int cols, bool load_e,
+                                         const FxH2& fp, const FxH2& fe)
+{
+    const unsigned m = an_magic(cols);
+    int ex = 0;
+    for (int q = threadIdx.x; q < rows * cols; q += blockDim.x) {
+        const int ly = an_div(q, cols, m), i = w.y0 + ly, j = w.x0 + (q - ly * cols);
+        const int c = (i + j) & 1, o = w.at(i, j), er = fx_exp2(w.Rh(c)[o]);
+        ex = max(ex, er ? er + (g.edge(i, j) ? fe.add : fp.add) : 0);
+        if (load_e) ex = max(ex, fx_exp2(w.E(c)[o]));
+    }
+    return ex;
+}
+
+// ... and those words in place on the scale em
+__device__ __forceinline__ AnWin<long long> an_fx_window(const AnWin<double>& w, const AnGeo& g, int rows, int cols,
+                                                         bool load_e, const FxH2& fp, const FxH2& fe, int em)
+{
+    const AnWin<long long> f{w.y0, w.x0, w.W, reinterpret_cast<longlong2*>(w.E0), reinterpret_cast<longlong2*>(w.E1),
+                             reinterpret_cast<longlong2*>(w.R0), reinterpret_cast<longlong2*>(w.R1)};
+    const unsigned m = an_magic(cols);
+    for (int q = threadIdx.x; q < rows * cols; q += blockDim.x) {
+        const int ly = an_div(q, cols, m), i = w.y0 + ly, j = w.x0 + (q - ly * cols);
+        const int c = (i + j) & 1, o = w.at(i, j);
+        const double2 r = w.Rh(c)[o];
+        f.Rh(c)[o] = g.edge(i, j) ? fe.q2(r, em) : fp.q2(r, em);
+        if (load_e) f.E(c)[o] = fx_q2(w.E(c)[o], em);      // (zeros stay zero)
+    }
+    return f;
+}
+
+// mean of the inward neighbours of edge node (i, j), held in the plane Eo
+__device__ __forceinline__ longlong2 an_fx_inward(const AnWin<long long>& w, const longlong2* Eo, int i, int j, int n)
+{
+    longlong2 s = make_longlong2(0, 0);
+    int c = 0;
+    auto add = [&](int a, int b) {
+        const longlong2 v = Eo[w.at(a, b)];
+        s.x += v.x;
+        s.y += v.y;
+        ++c;
+    };
+    if (i == 0) add(1, j);
+    if (i == n) add(n - 1, j);
+    if (j == 0) add(i, 1);
+    if (j == n) add(i, n - 1);
+    return c == 2 ? make_longlong2(fx_shr<1>(s.x), fx_shr<1>(s.y)) : s;
+}
+
+__device__ __forceinline__ void an_fx_half(const AnWin<long long>& w, const AnGeo& g, int ya, int yb, int xa, int xb,
+                                           int color)
+{
+    if (ya > yb || xa > xb) return;
+    const int nx = (xb - xa + 2) >> 1, total = nx * (yb - ya + 1);
+    const unsigned m = an_magic(nx);
+    const bool pure = an_pure(g, ya, yb, xa, xb);
+    longlong2* __restrict__ Ec = w.E(color);
+    const longlong2* __restrict__ Eo = w.E(color ^ 1);
+    const longlong2* __restrict__ Rc = w.Rh(color);
+    for (int q = threadIdx.x; q < total; q += blockDim.x) {
+        const int r = an_div(q, nx, m), i = ya + r;
+        const int j = xa + ((xa + i + color) & 1) + 2 * (q - r * nx);
+        if (j > xb || (!pure && g.hole(i, j))) continue;
+        const int o = w.at(i, j);
+        if (pure || !g.edge(i, j)) {
+            Ec[o] = fx_gs(Eo[w.at(i - 1, j)], Eo[w.at(i + 1, j)], Eo[w.at(i, j - 1)], Eo[w.at(i, j + 1)], Rc[o]);
+        } else {
+            const longlong2 s = an_fx_inward(w, Eo, i, j, g.n), rr = Rc[o];
+            Ec[o] = make_longlong2(s.x + rr.x, s.y + rr.y);
+        }
+    }
+}
+
+__device__ __forceinline__ void an_fx_sweeps(const AnWin<long long>& w, const AnGeo& g, int rows, int cols, int skip,
+                                             int nu)
+{
+    for (int k = 0; k < 2 * nu; ++k) {
+        const int s = skip + k + 1;
+        an_fx_half(w, g, max(0, w.y0 + s), min(g.n, w.y0 + rows - 1 - s), max(0, w.x0 + s),
+                   min(g.n, w.x0 + cols - 1 - s), k & 1);
+        __syncthreads();
+    }
+}
+
+// h^2 (PDE) or h (EDGE) times the residual of the row at (i, j); zero on the hole
+__device__ __forceinline__ longlong2 an_fx_resid(const AnWin<long long>& w, const AnGeo& g, int i, int j, bool zero)
+{
+    const int color = (i + j) & 1, o = w.at(i, j);
+    longlong2 r = w.Rh(color)[o];
+    if (g.hole(i, j)) return make_longlong2(0, 0);
+    if (zero) return r;
+    const longlong2 c = w.E(color)[o];
+    const longlong2* __restrict__ Eo = w.E(color ^ 1);
+    if (!g.edge(i, j)) {
+        const longlong2 p = Eo[w.at(i - 1, j)], q = Eo[w.at(i + 1, j)], s = Eo[w.at(i, j - 1)], t = Eo[w.at(i, j + 1)];
+        r.x -= ((p.x + q.x) + (s.x + t.x)) - 4 * c.x;
+        r.y -= ((p.y + q.y) + (s.y + t.y)) - 4 * c.y;
+    } else {
+        const longlong2 mm = an_fx_inward(w, Eo, i, j, g.n);
+        r.x -= c.x - mm.x;
+        r.y -= c.y - mm.y;
+    }
+    return r;
+}
+
 __host__ __device__ constexpr int an_down_rows(int T, int nu1) { return T + 3 + 4 * nu1; }
 __host__ __device__ constexpr int an_up_w(int T, int nu2, bool band)
 {
@@ -331,11 +450,59 @@ k_an_down(const typename CX<R>::T* __restrict__ e, typename CX<R>::T* __restrict
     pdl_trigger();
     an_stage<R>(w, rows, rows, e, rhs, n, load_e != 0);
     cp_async_wait_all();
-    __syncthreads();
-    an_sweeps_w<R>(w, g, rows, rows, 0, h, dinv, nu1);
     const bool zero = nu1 == 0 && load_e == 0;
     const int Sc = nc + 1, S = n + 1;
     const int ci1 = min(nc, I0 + AN_CT - 1), cj1 = min(nc, J0 + AN_CT - 1);
+    if constexpr (std::is_same<R, double>::value) {
+        // Fixed point with room for the largest sum.  In units of the window's largest value a
+        // sweep adds 5 / 4 at most (an EDGE row adds h rhs to a neighbour that h^2 rhs / 4 went
+        // into): 7 / 2 after two sweeps, residuals below 29, rows of the full weighting below
+        // 116 (2^56 * 116 < 2^63).
+        __shared__ int sx[AN_TT / 32];
+        const FxH2 fp(h * h), fe(h);
+        const bool plain = nu1 <= AN_FX_NU1 && fx_bits(dinv) == fx_bits(0.25);
+        const int em = block_max_exp<AN_TT>(plain ? an_fx_exp(w, g, rows, rows, load_e != 0, fp, fe) : 0, sx) + 2;
+        if (plain && fp.usable(em) && fe.usable(em)) {
+            const AnWin<long long> f = an_fx_window(w, g, rows, rows, load_e != 0, fp, fe, em);
+            __syncthreads();
+            an_fx_sweeps(f, g, rows, rows, 0, nu1);
+            for (int q = threadIdx.x; q < 4 * AN_CT * AN_CT; q += AN_TT) {
+                const int i = 2 * I0 + q / (2 * AN_CT), j = 2 * J0 + q % (2 * AN_CT);
+                if (i <= n && j <= n) e_out[(size_t)i * S + j] = fx_d2(f.e(i, j), em);
+            }
+            const int ry0 = max(0, 2 * I0 - 1), ry1 = min(n, 2 * ci1 + 1);
+            const int rx0 = max(0, 2 * J0 - 1), rx1 = min(n, 2 * cj1 + 1);
+            const int nx = rx1 - rx0 + 1;
+            const unsigned m = an_magic(nx);
+            for (int q = threadIdx.x; q < nx * (ry1 - ry0 + 1); q += AN_TT) {
+                const int r = an_div(q, nx, m), i = ry0 + r, j = rx0 + (q - r * nx);
+                f.Rh((i + j) & 1)[f.at(i, j)] = an_fx_resid(f, g, i, j, zero);
+            }
+            __syncthreads();
+            for (int q = threadIdx.x; q < AN_CT * AN_CT; q += AN_TT) {
+                const int I = I0 + q / AN_CT, J = J0 + q % AN_CT;
+                if (I > ci1 || J > cj1) continue;
+                auto res = [&](int i, int j) -> longlong2 { return f.Rh((i + j) & 1)[f.at(i, j)]; };
+                double2 v = make_double2(0.0, 0.0);
+                if (gc.edge(I, J)) {
+                    v = fe.over(res(2 * I, 2 * J), em);
+                } else if (!gc.hole(I, J)) {
+                    longlong2 t[3];
+#pragma unroll
+                    for (int a = -1; a <= 1; ++a) {
+                        const longlong2 u = res(2 * I + a, 2 * J - 1), c = res(2 * I + a, 2 * J),
+                                        d = res(2 * I + a, 2 * J + 1);
+                        t[a + 1] = make_longlong2(fx_shr<2>((u.x + d.x) + 2 * c.x), fx_shr<2>((u.y + d.y) + 2 * c.y));
+                    }
+                    v = fp.over(make_longlong2((t[0].x + t[2].x) + 2 * t[1].x, (t[0].y + t[2].y) + 2 * t[1].y), em - 2);
+                }
+                rc[(size_t)I * Sc + J] = v;
+            }
+            return;
+        }
+    }
+    __syncthreads();
+    an_sweeps_w<R>(w, g, rows, rows, 0, h, dinv, nu1);
     {
         const int fi1 = min(n, 2 * I0 + 2 * AN_CT - 1), fj1 = min(n, 2 * J0 + 2 * AN_CT - 1);
         for (int q = threadIdx.x; q < 4 * AN_CT * AN_CT; q += AN_TT) {
@@ -413,6 +580,54 @@ k_an_up(const typename CX<R>::T* __restrict__ e2, typename CX<R>::T* __restrict_
     }
     an_stage<R>(w, W, W, e2, rhs, n, true);
     cp_async_wait_all();
+    if constexpr (std::is_same<R, double>::value) {
+        // Fixed point: in units of the window's largest value 2 after the correction, 4 after the
+        // band (PDE rows: 1 / 2 a sweep), 13 / 2 after two sweeps (a row's sum 27: 2^58 * 27 <
+        // 2^63), 9 after four (37, on 2^57)
+        __shared__ int sx[AN_TT / 32];
+        const FxH2 fp(h * h), fe(h);
+        const bool plain = nu2 <= AN_FX_NU2 && fx_bits(dinv) == fx_bits(0.25);
+        int ex = 0;
+        if (plain) {
+            ex = an_fx_exp(w, g, W, W, true, fp, fe);
+            for (int q = threadIdx.x; q < CW * CW; q += AN_TT) ex = max(ex, fx_exp2(Cs[q]));
+        }
+        const int em = block_max_exp<AN_TT>(ex, sx) + (nu2 <= 2 ? 0 : 1);
+        if (plain && fp.usable(em) && fe.usable(em)) {
+            const AnWin<long long> f = an_fx_window(w, g, W, W, true, fp, fe, em);
+            longlong2* const Fc = reinterpret_cast<longlong2*>(Cs);
+            for (int q = threadIdx.x; q < CW * CW; q += AN_TT) Fc[q] = fx_q2(Cs[q], em);
+            __syncthreads();
+            const int ya = max(0, w.y0), yb = min(n, w.y0 + W - 1), xa = max(0, w.x0), xb = min(n, w.x0 + W - 1);
+            const int nx = xb - xa + 1;
+            const unsigned m = an_magic(nx);
+            for (int q = threadIdx.x; q < nx * (yb - ya + 1); q += AN_TT) {
+                const int r = an_div(q, nx, m), i = ya + r, j = xa + (q - r * nx);
+                if (g.hole(i, j)) continue;
+                const longlong2* p0 = Fc + ((i >> 1) - cy0) * CW, *p1 = Fc + (((i + 1) >> 1) - cy0) * CW;
+                const int J0 = (j >> 1) - cx0, J1 = ((j + 1) >> 1) - cx0;
+                const longlong2 a = p0[J0], b = p1[J0], c = p0[J1], d = p1[J1];
+                longlong2* const p = f.E((i + j) & 1) + f.at(i, j);
+                p->x += fx_shr<2>((a.x + b.x) + (c.x + d.x));
+                p->y += fx_shr<2>((a.y + b.y) + (c.y + d.y));
+            }
+            __syncthreads();
+            if (band)
+                for (int k = 0; k < 2 * AN_BAND_SWEEPS; ++k) {
+                    const int t = k + 1;
+                    an_fx_half(f, g, max(g.b0, w.y0 + t), min(g.b1, w.y0 + W - 1 - t), max(g.b0, w.x0 + t),
+                               min(g.b1, w.x0 + W - 1 - t), k & 1);
+                    __syncthreads();
+                }
+            an_fx_sweeps(f, g, W, W, skip, nu2);
+            const int S = n + 1;
+            for (int q = threadIdx.x; q < AN_FT * AN_FT; q += AN_TT) {
+                const int i = i0 + q / AN_FT, j = j0 + q % AN_FT;
+                if (i <= n && j <= n) e_out[(size_t)i * S + j] = fx_d2(f.e(i, j), em);
+            }
+            return;
+        }
+    }
     __syncthreads();
     {
         const int ya = max(0, w.y0), yb = min(n, w.y0 + W - 1), xa = max(0, w.x0), xb = min(n, w.x0 + W - 1);
