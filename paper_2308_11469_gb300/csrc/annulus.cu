@@ -55,23 +55,6 @@ __host__ __device__ constexpr size_t an_a16(size_t b) { return (b + 15) & ~(size
 
 int grid_for(long work) { return (int)std::min<long>((work + AN_NT - 1) / AN_NT, 152L * 16); }
 
-// mean of the inward neighbours of an edge node (two at a corner)
-template <typename T>
-__device__ __forceinline__ T inward_mean(const T* e, int i, int j, int n)
-{
-    const int S = n + 1;
-    T s;
-    s.x = 0;
-    s.y = 0;
-    int c = 0;
-    if (i == 0) { s.x += e[S + j].x; s.y += e[S + j].y; ++c; }
-    if (i == n) { s.x += e[(n - 1) * S + j].x; s.y += e[(n - 1) * S + j].y; ++c; }
-    if (j == 0) { s.x += e[i * S + 1].x; s.y += e[i * S + 1].y; ++c; }
-    if (j == n) { s.x += e[i * S + n - 1].x; s.y += e[i * S + n - 1].y; ++c; }
-    if (c == 2) { s.x *= 0.5f; s.y *= 0.5f; }
-    return s;
-}
-
 // FP64 <-> inner precision; complex64's format changes run on the integer pipes
 __device__ __forceinline__ double an_widen(float x) { return f2d_bits(x); }
 __device__ __forceinline__ double an_widen(double x) { return x; }
@@ -848,77 +831,10 @@ k_an_init(double2* __restrict__ U0, double2* __restrict__ U1, const double2* __r
     }
 }
 
-// U_out = U_in + e on the non-hole nodes (hole nodes keep the data in both buffers);
-// per-block maxima of |e|^2 into part[2 b + 1]
+// part[block] = the block's sum (by warps in R, then in FP64)
 template <typename R>
-__global__ void __launch_bounds__(AN_NT)
-k_an_update(const double2* __restrict__ Uin, double2* __restrict__ Uout, const typename CX<R>::T* __restrict__ e,
-            const unsigned char* __restrict__ typ, long total, double* __restrict__ part)
+__device__ __forceinline__ void an_block_sum(R r2, double* sa, double* __restrict__ part)
 {
-    typedef typename CX<R>::T c2;
-    R em = 0;
-    for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < total; t += (long)gridDim.x * blockDim.x) {
-        if (typ[t] == AN_HOLE) continue;
-        const c2 ev = e[t];
-        double2 v = Uin[t];
-        v.x += an_widen(ev.x);
-        v.y += an_widen(ev.y);
-        Uout[t] = v;
-        const R a = ev.x * ev.x + ev.y * ev.y;
-        em = em > a ? em : a;
-    }
-    __shared__ double sm[AN_NT / 32];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const R x = __shfl_xor_sync(0xffffffffu, em, o);
-        em = em > x ? em : x;
-    }
-    if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = (double)em;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double m = 0.0;
-        for (int w = 0; w < AN_NT / 32; ++w) m = fmax(m, sm[w]);
-        part[2 * blockIdx.x + 1] = m;
-    }
-}
-
-// r = b - B U in FP64 (PDE: f - (Delta_h U + k^2 U); EDGE: q - (dU/dn - i k U)), stored,
-// rounded to the inner precision, as the next rhs; per-block sums of |r|^2 (of the stored
-// r) into part[2 b]
-template <typename R>
-__global__ void __launch_bounds__(AN_NT)
-k_an_resid(const double2* __restrict__ U, const double2* __restrict__ data, const unsigned char* __restrict__ typ,
-           typename CX<R>::T* __restrict__ rhs, int n, double h, double k2, double k, double* __restrict__ part)
-{
-    typedef typename CX<R>::T c2;
-    const int S = n + 1;
-    const long total = (long)S * S;
-    const double ih2 = 1.0 / (h * h), ih = 1.0 / h;
-    R r2 = 0;
-    for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < total; t += (long)gridDim.x * blockDim.x) {
-        const unsigned char ty = typ[t];
-        if (ty == AN_HOLE) continue;
-        const int q = (int)t, i = q / S, j = q % S;
-        const double2 c = U[q];
-        const double2 dv = data[q];
-        double2 r;
-        if (ty == AN_PDE) {
-            const double2 a = U[q - S], b = U[q + S], cc = U[q - 1], d = U[q + 1];
-            r.x = dv.x - (((a.x + b.x) + (cc.x + d.x) - 4.0 * c.x) * ih2 + k2 * c.x);
-            r.y = dv.y - (((a.y + b.y) + (cc.y + d.y) - 4.0 * c.y) * ih2 + k2 * c.y);
-        } else {
-            const double2 m = inward_mean(U, i, j, n);
-            // dU/dn - i k U = (U - mean) / h + (k U.y, -k U.x)
-            r.x = dv.x - ((c.x - m.x) * ih + k * c.y);
-            r.y = dv.y - ((c.y - m.y) * ih - k * c.x);
-        }
-        c2 ri;
-        ri.x = an_narrow(r.x, R());
-        ri.y = an_narrow(r.y, R());
-        rhs[q] = ri;
-        r2 += ri.x * ri.x + ri.y * ri.y;
-    }
-    __shared__ double sa[AN_NT / 32];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) r2 += __shfl_xor_sync(0xffffffffu, r2, o);
     if ((threadIdx.x & 31) == 0) sa[threadIdx.x >> 5] = (double)r2;
@@ -926,8 +842,154 @@ k_an_resid(const double2* __restrict__ U, const double2* __restrict__ data, cons
     if (threadIdx.x == 0) {
         double a = 0.0;
         for (int w = 0; w < AN_NT / 32; ++w) a += sa[w];
-        part[2 * blockIdx.x] = a;
+        part[blockIdx.x] = a;
     }
+}
+
+// An outer step's update and residual in one pass: U_out = U_in + e on the non-hole nodes (hole
+// nodes keep the data in both buffers; e == nullptr: U_in as it is), r = b - B U_out in FP64
+// (PDE: f - (Delta_h U + k^2 U); EDGE: q - (dU/dn - i k U)) into rhs, rounded to the inner
+// precision; in FP64 also per-block sums of |r|^2 into part[b] (k_an_norm in complex64).
+//
+// A tile's T x T updated nodes and their ring go to shared memory, so that U is read once and
+// e at all only here.  complex128: on the tile's fixed-point scale, the numerators being exact
+// integer sums (6 FP64 operations a node instead of 16; an SM serves about 2 a clock); tiles
+// outside the scale's range in FP64.  complex64 keeps the FP64 numerators, which bound it: an
+// inner cycle in FP32 passes a residual that rounds otherwise in one node of a thousand on as
+// 1e-10 .. 1e-9 of the next steps' residuals.  T as in an_tile; the grid strides over the tiles.
+// 1024^2 complex64: 58 us in two launches -> 43 (36 at the start, without e), and 7 for the norm;
+// its 16 FP64 operations a node take 29 us, its 64 bytes 9.  With the numerators in fixed point
+// 28 us, for histories 3e-10 off.  1 / h^2 comes from the host: an FP64 division in every thread
+// took 4 us.  256^2 complex128: a step 75 -> 73 us.
+template <typename R, int T>
+__global__ void __launch_bounds__(AN_NT)
+k_an_step(const double2* __restrict__ Uin, double2* __restrict__ Uout, const typename CX<R>::T* __restrict__ e,
+          const double2* __restrict__ data, typename CX<R>::T* __restrict__ rhs, AnGeo g, int nt,
+          double ih2, double ih, double k2, double k, double* __restrict__ part)
+{
+    typedef typename CX<R>::T c2;
+    constexpr int W = T + 2, PER = T * T / AN_NT;
+    constexpr bool WIDE = std::is_same<R, double>::value;
+    __shared__ longlong2 F[W * W];
+    __shared__ int sx[AN_NT / 32];
+    __shared__ double sa[AN_NT / 32];
+    double2* const D = reinterpret_cast<double2*>(F);
+    const int n = g.n, S = n + 1, tid = threadIdx.x;
+    R r2 = 0;
+    pdl_wait();
+    pdl_trigger();
+    for (int tile = blockIdx.x; tile < nt * nt; tile += gridDim.x) {
+        const int ty = tile / nt, i0 = ty * T, j0 = (tile - ty * nt) * T;
+        double2 c[PER], dv[PER], rv = make_double2(0.0, 0.0);
+        int ex = 0, ro = -1;
+        auto updated = [&](int i, int j, size_t q) {
+            double2 v = Uin[q];
+            if (e && !g.hole(i, j)) {
+                const c2 ev = e[q];
+                v.x += an_widen(ev.x);
+                v.y += an_widen(ev.y);
+            }
+            if (WIDE) ex = max(ex, fx_exp2(v));
+            return v;
+        };
+#pragma unroll
+        for (int p = 0; p < PER; ++p) {
+            const int q = tid + p * AN_NT, i = i0 + q / T, j = j0 + q % T;
+            c[p] = dv[p] = make_double2(0.0, 0.0);
+            if (i > n || j > n) continue;
+            const size_t gq = (size_t)i * S + j;
+            c[p] = updated(i, j, gq);
+            if (g.hole(i, j)) continue;
+            dv[p] = data[gq];
+            if (e) Uout[gq] = c[p];
+        }
+        if (tid < 4 * T + 4) {                    // the ring: two rows of W, two columns of T
+            const int u = tid < 2 * W ? tid % W : (tid - 2 * W) % T + 1, b = tid < 2 * W ? tid / W : (tid - 2 * W) / T;
+            const int ly = tid < 2 * W ? b * (W - 1) : u, lx = tid < 2 * W ? u : b * (W - 1);
+            const int i = i0 - 1 + ly, j = j0 - 1 + lx;
+            ro = ly * W + lx;
+            if (i >= 0 && i <= n && j >= 0 && j <= n) rv = updated(i, j, (size_t)i * S + j);
+        }
+        int em = -1;                              // -1: FP64
+        if constexpr (WIDE) {
+            em = block_max_exp<AN_NT>(ex, sx);
+            if (em == 0) em = FX_EMIN + 8;
+            if (!fx_usable(em)) em = -1;
+        } else {
+            __syncthreads();                      // the last tile's readers are done
+        }
+        auto put = [&](int o, double2 v) {
+            if (WIDE && em >= 0) F[o] = fx_q2(v, em);
+            else D[o] = v;
+        };
+#pragma unroll
+        for (int p = 0; p < PER; ++p) {
+            const int q = tid + p * AN_NT;
+            put((q / T + 1) * W + q % T + 1, c[p]);
+        }
+        if (ro >= 0) put(ro, rv);
+        __syncthreads();
+#pragma unroll
+        for (int p = 0; p < PER; ++p) {
+            const int q = tid + p * AN_NT, i = i0 + q / T, j = j0 + q % T, o = (q / T + 1) * W + q % T + 1;
+            if (i > n || j > n || g.hole(i, j)) continue;
+            const bool pde = !g.edge(i, j);
+            const double2 cc = c[p];
+            // an EDGE node's inward neighbours (o1; o2 = o1 but at a corner)
+            const int o1 = i == 0 ? o + W : i == n ? o - W : j == 0 ? o + 1 : o - 1;
+            const int o2 = (i == 0 || i == n) && (j == 0 || j == n) ? (j == 0 ? o + 1 : o - 1) : o1;
+            double2 r;
+            if (WIDE && em >= 0) {
+                const longlong2 m = F[o];
+                if (pde) {
+                    const longlong2 a = F[o - W], b = F[o + W], l = F[o - 1], t = F[o + 1];
+                    const long long sx2 = ((a.x + b.x) + (l.x + t.x)) - 4 * m.x, sy2 = ((a.y + b.y) + (l.y + t.y)) - 4 * m.y;
+                    r.x = fma(fx_to_double(sx2, em), -ih2, fma(cc.x, -k2, dv[p].x));
+                    r.y = fma(fx_to_double(sy2, em), -ih2, fma(cc.y, -k2, dv[p].y));
+                } else {
+                    const longlong2 a = F[o1], b = F[o2];
+                    r.x = fma(fx_to_double(2 * m.x - (a.x + b.x), em), -0.5 * ih, fma(cc.y, -k, dv[p].x));
+                    r.y = fma(fx_to_double(2 * m.y - (a.y + b.y), em), -0.5 * ih, fma(cc.x, k, dv[p].y));
+                }
+            } else if (pde) {
+                const double2 a = D[o - W], b = D[o + W], l = D[o - 1], t = D[o + 1];
+                r.x = dv[p].x - (((a.x + b.x) + (l.x + t.x) - 4.0 * cc.x) * ih2 + k2 * cc.x);
+                r.y = dv[p].y - (((a.y + b.y) + (l.y + t.y) - 4.0 * cc.y) * ih2 + k2 * cc.y);
+            } else {
+                // dU/dn - i k U = (U - mean) / h + (k U.y, -k U.x)
+                double2 m = D[o1];
+                if (o2 != o1) m = make_double2((m.x + D[o2].x) * 0.5, (m.y + D[o2].y) * 0.5);
+                r.x = dv[p].x - ((cc.x - m.x) * ih + k * cc.y);
+                r.y = dv[p].y - ((cc.y - m.y) * ih - k * cc.x);
+            }
+            c2 ri;
+            ri.x = an_narrow(r.x, R());
+            ri.y = an_narrow(r.y, R());
+            rhs[(size_t)i * S + j] = ri;
+            if constexpr (WIDE) r2 += ri.x * ri.x + ri.y * ri.y;
+        }
+    }
+    if constexpr (WIDE) an_block_sum(r2, sa, part);
+}
+
+// per-block sums of |rhs|^2 of a complex64 step.  Its FP32 sums follow the rows, whatever the
+// tiles: a start residual lives on a few nodes around the hole, and another order would move
+// the history by their roundings (1e-9 of it).
+__global__ void __launch_bounds__(AN_NT)
+k_an_norm(const float2* __restrict__ rhs, AnGeo g, double* __restrict__ part)
+{
+    __shared__ double sa[AN_NT / 32];
+    const int S = g.n + 1, total = S * S;
+    float r2 = 0;
+    pdl_wait();
+    pdl_trigger();
+    for (int t = blockIdx.x * AN_NT + threadIdx.x; t < total; t += gridDim.x * AN_NT) {
+        const int i = t / S, j = t - i * S;
+        if (g.hole(i, j)) continue;
+        const float2 ri = rhs[t];
+        r2 += ri.x * ri.x + ri.y * ri.y;
+    }
+    an_block_sum(r2, sa, part);
 }
 
 // real part of U -> out (double), and min over PDE nodes of (-L + sqrt(L^2 + 4 E)) / (2 E)
@@ -1496,9 +1558,11 @@ helm_status an_solve(helm_annulus* a, const double2* data, double2* u, double to
     const auto& L0 = a->lev[0];
     const long total = (long)(a->N + 1) * (a->N + 1);
     double2* U[2] = {u, a->U1};
+    const int T = an_tile(a->N), nt = (a->N + T) / T, sblk = std::min(nt * nt, a->nblk);
+    const int npart = std::is_same<R, float>::value ? a->nblk : sblk;
     k_an_init<<<grid_for(total), AN_NT, 0, s>>>(U[0], U[1], data, L0.typ, total);
     add_launches(1);
-    // mode 0: the start residual; mode 1: an outer step's update and residual; both end
+    // mode 0: the start residual; mode 1: an outer step's cycles, update and residual; both end
     // with the norm partials copied to the host (the caller synchronises)
     auto enqueue = [&](int mode, int it) -> helm_status {
         cudaStream_t q = a->ls;
@@ -1507,15 +1571,21 @@ helm_status an_solve(helm_annulus* a, const double2* data, double2* u, double to
                 const helm_status st = an_vcycle<R>(a, 0, c == 0);
                 if (st != HELM_OK) return st;
             }
-            k_an_update<R><<<a->nblk, AN_NT, 0, q>>>(U[(it - 1) & 1], U[it & 1], (const c2*)L0.e, L0.typ, total,
-                                                     a->part);
+        }
+        const double2* const Uin = U[mode == 1 ? (it - 1) & 1 : 0];
+        double2* const Uout = U[it & 1];
+        const c2* const e = mode == 1 ? (const c2*)L0.e : nullptr;
+        auto launch = [&](auto* kern, int nt) {
+            return launch_k(kern, dim3(sblk), dim3(AN_NT), (size_t)0, q, Uin, Uout, e, data, (c2*)L0.rhs, an_geo(L0),
+                            nt, 1.0 / (L0.h * L0.h), 1.0 / L0.h, a->k * a->k, a->k, a->part);
+        };
+        AN_CK(T == 32 ? launch(k_an_step<R, 32>, nt) : launch(k_an_step<R, 16>, nt));
+        an_count(a, 1);
+        if constexpr (std::is_same<R, float>::value) {
+            AN_CK(launch_k(k_an_norm, dim3(npart), dim3(AN_NT), (size_t)0, q, (const c2*)L0.rhs, an_geo(L0), a->part));
             an_count(a, 1);
         }
-        k_an_resid<R><<<a->nblk, AN_NT, 0, q>>>(U[mode == 1 ? (it & 1) : 0], data, L0.typ, (c2*)L0.rhs, a->N,
-                                                L0.h, a->k * a->k, a->k, a->part);
-        an_count(a, 1);
-        AN_CK(cudaGetLastError());
-        AN_CK(cudaMemcpyAsync(a->h_part, a->part, 2 * sizeof(double) * a->nblk, cudaMemcpyDeviceToHost, q));
+        AN_CK(cudaMemcpyAsync(a->h_part, a->part, sizeof(double) * npart, cudaMemcpyDeviceToHost, q));
         return HELM_OK;
     };
     // an outer step of either parity as one graph (its pointers and parameters are fixed for
@@ -1567,7 +1637,7 @@ helm_status an_solve(helm_annulus* a, const double2* data, double2* u, double to
     helm_status st = step(0, 1);
     if (st != HELM_OK) { drop_graphs(); return st; }
     double r2 = 0.0;
-    for (int b = 0; b < a->nblk; ++b) r2 += a->h_part[2 * b];
+    for (int b = 0; b < npart; ++b) r2 += a->h_part[b];
     const double norm0 = std::sqrt(r2);
     int it = 0, status = HELM_MAXITER, run = 0;
     double prev = 1.0, rmin = 1.0;
@@ -1578,7 +1648,7 @@ helm_status an_solve(helm_annulus* a, const double2* data, double2* u, double to
             st = step(1, it);
             if (st != HELM_OK) { drop_graphs(); return st; }
             r2 = 0.0;
-            for (int b = 0; b < a->nblk; ++b) r2 += a->h_part[2 * b];
+            for (int b = 0; b < npart; ++b) r2 += a->h_part[b];
             const double rel = std::sqrt(r2) / norm0;
             if (hist) hist[it] = rel;
             // the cavity's status rule
@@ -1889,13 +1959,13 @@ helm_status helm_annulus_create(helm_annulus** out, int n, double side, double h
     const long total = (long)(n + 1) * (n + 1);
     a->nblk = grid_for(total);
     void* p = nullptr;
-    if (cudaMalloc(&p, total * sizeof(double2) + 2 * sizeof(double) * a->nblk + 256) != cudaSuccess)
+    if (cudaMalloc(&p, total * sizeof(double2) + sizeof(double) * a->nblk + 256) != cudaSuccess)
         return fail(HELM_ENOMEM);
     a->allocs.push_back(p);
     a->U1 = (double2*)p;
     a->part = (double*)((char*)p + total * sizeof(double2));
-    a->kmin = (unsigned long long*)((char*)a->part + 2 * sizeof(double) * a->nblk);
-    if (cudaMallocHost(&a->h_part, 2 * sizeof(double) * a->nblk) != cudaSuccess) return fail(HELM_ENOMEM);
+    a->kmin = (unsigned long long*)((char*)a->part + sizeof(double) * a->nblk);
+    if (cudaMallocHost(&a->h_part, sizeof(double) * a->nblk) != cudaSuccess) return fail(HELM_ENOMEM);
     helm_status st = helm_annulus_set_shift(a, a->alpha);
     if (st != HELM_OK) return fail(st);
     *out = a;

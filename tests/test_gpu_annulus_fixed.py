@@ -60,3 +60,26 @@ def test_iterates_match_the_numpy_cycle(N, side, data, cycle):
     assert it == steps
     err = np.linalg.norm(u.cpu().numpy() - U) / np.linalg.norm(U)
     assert err <= steps * 2.0 ** -53 * 0.4 * N * N, err
+
+
+def test_iterates_beyond_the_scale():
+    """Hole data of 2^1000 (mesh widths that keep the residuals finite): windows and the
+    residual's tiles hold values that have no fixed-point scale and are evaluated in FP64."""
+    from paper_2308_11469_gb300 import binding as B
+    N, side = 128, 2.0 ** 497
+    levels = _levels(N, side)
+    L = levels[0]
+    x = np.arange(N + 1) / N
+    d = np.where(L.hole, 2.0 ** 1000 * (1.0 + 0.5 * x[:, None] + 0.25j * x[None, :]), 0)
+    r = np.where(L.pde, -((L.nbrs(d) - 4.0 * d) / L.h ** 2), 0)
+    e = np.zeros_like(d)
+    _cycle(levels, 0, e, r, 2, 2)
+    plan = B.helm_annulus_create(N, side, 0.15 * side, 0.0, B.HELM_PREC_FP64)
+    dd = torch.from_numpy(d).cuda()
+    u = torch.empty_like(dd)
+    _, it, hist = B.helm_annulus_solve(plan, dd, u, 0.0, 1)
+    B.helm_annulus_destroy(plan)
+    assert it == 1 and np.isfinite(hist).all()
+    U = (d + e) * 2.0 ** -1000
+    err = np.linalg.norm(u.cpu().numpy() * 2.0 ** -1000 - U) / np.linalg.norm(U)
+    assert err <= 2.0 ** -53 * 0.4 * N * N, err
