@@ -42,7 +42,7 @@ constexpr int AN_NT = 256;
 constexpr int AN_NC = 8;            // coarsest level (solved exactly)
 constexpr int AN_BAND = 4;          // band half-width around the hole, in nodes of the level
 constexpr int AN_BAND_SWEEPS = 4;
-constexpr bool AN_GRAPHS = true;     // an outer step replayed as one graph launch
+constexpr bool AN_GRAPHS = true;     // the outer steps as one graph launch
 constexpr size_t AN_SMEM_MAX = 227 * 1024;
 enum : unsigned char { AN_PDE = 0, AN_EDGE = 1, AN_HOLE = 2 };
 
@@ -819,21 +819,99 @@ k_an_tail(typename CX<R>::T* __restrict__ eg, const typename CX<R>::T* __restric
     }
 }
 
-// U := the hole data on hole nodes, 0 elsewhere (both iterate buffers)
+// Control of a solve, in device memory: its buffers (the step's graph is kept with the plan, the
+// caller's pointers are not in it), the outer iteration's state, and the history's ring in
+// page-locked memory.
+struct AnCtl {
+    double2* U[2];
+    const double2* data;
+    double* hist;                     // AN_HIST entries: step N at N % AN_HIST
+    double tol, norm0, prev, rmin;
+    int it, max_outer, run, status;   // status: AN_ACTIVE or the outcome
+    int budget;                       // steps left of this launch
+    unsigned ticket;
+};
+constexpr int AN_ACTIVE = 1000, AN_HIST = 4096;
+
+// U := the hole data on hole nodes, 0 elsewhere (both iterate buffers); starts the control
 __global__ void __launch_bounds__(AN_NT)
-k_an_init(double2* __restrict__ U0, double2* __restrict__ U1, const double2* __restrict__ data,
-          const unsigned char* __restrict__ typ, long total)
+k_an_init(AnCtl* __restrict__ ctl, AnCtl c, const unsigned char* __restrict__ typ, long total)
 {
+    if (blockIdx.x == 0 && threadIdx.x == 0) *ctl = c;
     for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < total; t += (long)gridDim.x * blockDim.x) {
-        const double2 v = (typ[t] == AN_HOLE) ? data[t] : make_double2(0.0, 0.0);
-        U0[t] = v;
-        U1[t] = v;
+        const double2 v = (typ[t] == AN_HOLE) ? c.data[t] : make_double2(0.0, 0.0);
+        c.U[0][t] = v;
+        c.U[1][t] = v;
     }
+}
+
+// a further run of steps
+__global__ void k_an_more(AnCtl* ctl, int budget) { ctl->budget = budget; }
+
+// the result to the caller's buffer (U[0]), the outcome to the host
+__global__ void __launch_bounds__(AN_NT)
+k_an_fin(const AnCtl* __restrict__ ctl, int* __restrict__ out, long total)
+{
+    const int it = ctl->it;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        out[0] = it;
+        out[1] = ctl->status;
+    }
+    if (!(it & 1) || ctl->status == AN_ACTIVE) return;
+    double2* const u = ctl->U[0];
+    const double2* const v = ctl->U[1];
+    for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < total; t += (long)gridDim.x * blockDim.x) u[t] = v[t];
+}
+
+// The last of a launch's blocks sums the np partials, applies the cavity's status rule and sets
+// the loop's condition (gh != 0).  start: the start residual.
+__device__ void an_finish(AnCtl* ctl, const double* part, int np, bool start, unsigned long long gh, double* sa)
+{
+    __shared__ bool last;
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicAdd(&ctl->ticket, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    double r2 = 0.0;
+    for (int b = threadIdx.x; b < np; b += blockDim.x) r2 += __ldcg(part + b);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) r2 += __shfl_xor_sync(0xffffffffu, r2, o);
+    if ((threadIdx.x & 31) == 0) sa[threadIdx.x >> 5] = r2;
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    r2 = 0.0;
+    for (int w = 0; w < (int)blockDim.x / 32; ++w) r2 += sa[w];
+    AnCtl c = *ctl;
+    c.ticket = 0u;
+    const double norm = sqrt(r2);
+    if (start) {
+        c.norm0 = norm;
+        c.hist[0] = norm == 0.0 ? 0.0 : 1.0;
+        c.status = norm == 0.0 ? HELM_CONVERGED : !isfinite(norm) ? HELM_ENONFINITE : c.max_outer < 1 ? HELM_MAXITER
+                                                                                                      : AN_ACTIVE;
+    } else if (c.status == AN_ACTIVE) {            // (a solve that ended at its start: nothing)
+        const double rel = norm / c.norm0;
+        const int it = ++c.it;
+        c.hist[it % AN_HIST] = rel;
+        c.run = (rel >= c.prev) ? c.run + 1 : 0;
+        c.prev = rel;
+        c.rmin = fmin(c.rmin, rel);
+        if (!isfinite(rel)) c.status = HELM_ENONFINITE;
+        else if (rel <= c.tol) c.status = HELM_CONVERGED;
+        else if (rel > 1e4 || (it >= 20 && c.run >= 10 && rel >= 2.0 * c.rmin)) c.status = HELM_DIVERGED;
+        else if (it >= c.max_outer) c.status = HELM_MAXITER;
+        --c.budget;
+    }
+    *ctl = c;
+    if (gh) cudaGraphSetConditional((cudaGraphConditionalHandle)gh, c.status == AN_ACTIVE && c.budget > 0 ? 1u : 0u);
 }
 
 // part[block] = the block's sum (by warps in R, then in FP64)
 template <typename R>
-__device__ __forceinline__ void an_block_sum(R r2, double* sa, double* __restrict__ part)
+__device__ __forceinline__ void an_block_sum(R r2, double* sa, double* part)
 {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) r2 += __shfl_xor_sync(0xffffffffu, r2, o);
@@ -863,9 +941,8 @@ __device__ __forceinline__ void an_block_sum(R r2, double* sa, double* __restric
 // took 4 us.  256^2 complex128: a step 75 -> 73 us.
 template <typename R, int T>
 __global__ void __launch_bounds__(AN_NT)
-k_an_step(const double2* __restrict__ Uin, double2* __restrict__ Uout, const typename CX<R>::T* __restrict__ e,
-          const double2* __restrict__ data, typename CX<R>::T* __restrict__ rhs, AnGeo g, int nt,
-          double ih2, double ih, double k2, double k, double* __restrict__ part)
+k_an_step(AnCtl* ctl, const typename CX<R>::T* __restrict__ e, typename CX<R>::T* __restrict__ rhs, AnGeo g, int nt,
+          double ih2, double ih, double k2, double k, double* part, unsigned long long gh)
 {
     typedef typename CX<R>::T c2;
     constexpr int W = T + 2, PER = T * T / AN_NT;
@@ -878,6 +955,10 @@ k_an_step(const double2* __restrict__ Uin, double2* __restrict__ Uout, const typ
     R r2 = 0;
     pdl_wait();
     pdl_trigger();
+    const int par = ctl->it & 1;
+    const double2* __restrict__ const Uin = ctl->U[par];
+    double2* __restrict__ const Uout = ctl->U[par ^ 1];
+    const double2* __restrict__ const data = ctl->data;
     for (int tile = blockIdx.x; tile < nt * nt; tile += gridDim.x) {
         const int ty = tile / nt, i0 = ty * T, j0 = (tile - ty * nt) * T;
         double2 c[PER], dv[PER], rv = make_double2(0.0, 0.0);
@@ -969,14 +1050,17 @@ k_an_step(const double2* __restrict__ Uin, double2* __restrict__ Uout, const typ
             if constexpr (WIDE) r2 += ri.x * ri.x + ri.y * ri.y;
         }
     }
-    if constexpr (WIDE) an_block_sum(r2, sa, part);
+    if constexpr (WIDE) {
+        an_block_sum(r2, sa, part);
+        an_finish(ctl, part, gridDim.x, e == nullptr, gh, sa);
+    }
 }
 
 // per-block sums of |rhs|^2 of a complex64 step.  Its FP32 sums follow the rows, whatever the
 // tiles: a start residual lives on a few nodes around the hole, and another order would move
 // the history by their roundings (1e-9 of it).
 __global__ void __launch_bounds__(AN_NT)
-k_an_norm(const float2* __restrict__ rhs, AnGeo g, double* __restrict__ part)
+k_an_norm(const float2* __restrict__ rhs, AnGeo g, double* part, AnCtl* ctl, int start, unsigned long long gh)
 {
     __shared__ double sa[AN_NT / 32];
     const int S = g.n + 1, total = S * S;
@@ -990,6 +1074,7 @@ k_an_norm(const float2* __restrict__ rhs, AnGeo g, double* __restrict__ part)
         r2 += ri.x * ri.x + ri.y * ri.y;
     }
     an_block_sum(r2, sa, part);
+    an_finish(ctl, part, gridDim.x, start != 0, gh, sa);
 }
 
 // real part of U -> out (double), and min over PDE nodes of (-L + sqrt(L^2 + 4 E)) / (2 E)
@@ -1339,13 +1424,16 @@ struct helm_annulus {
     int m = 0;
     double2* U1 = nullptr;
     double* part = nullptr;
-    double* h_part = nullptr;
+    AnCtl* ctl = nullptr;
+    double* h_hist = nullptr;             // page-locked: the history's ring, the outcome behind it
+    cudaGraphExec_t loop = nullptr;       // outer steps until the control says otherwise
+    uint64_t loop_step = 0;               // kernels of one of them
     int nblk = 0;
     unsigned long long* kmin = nullptr;
     cudaStream_t stream = nullptr;
     std::vector<void*> allocs;
     cudaStream_t ls = nullptr;            // where an_vcycle and the step launch (stream, or cap)
-    cudaStream_t cap = nullptr;           // non-blocking stream for capturing a step's graph
+    cudaStream_t cap = nullptr;           // non-blocking stream for capturing the loop's body
     bool capturing = false;
     uint64_t captured = 0;                // kernels recorded by the capture in progress
     int t0 = -1;                          // first level of the one-CTA coarse tail
@@ -1548,127 +1636,127 @@ helm_status an_vcycle(helm_annulus* a, int l, bool zero)
     return an_tile(L.n) == 32 ? an_up<R, 32>(a, L, C) : an_up<R, 16>(a, L, C);
 }
 
+// The update and residual of a step on a->ls (start: the start residual); cond: the handle of the
+// loop that it ends (0: none).
+template <typename R>
+helm_status an_step(helm_annulus* a, bool start, unsigned long long cond)
+{
+    typedef typename CX<R>::T c2;
+    const auto& L0 = a->lev[0];
+    const int T = an_tile(a->N), nt = (a->N + T) / T;
+    auto launch = [&](auto* kern) {
+        return launch_k(kern, dim3(std::min(nt * nt, a->nblk)), dim3(AN_NT), (size_t)0, a->ls, a->ctl,
+                        start ? (const c2*)nullptr : (const c2*)L0.e, (c2*)L0.rhs, an_geo(L0), nt,
+                        1.0 / (L0.h * L0.h), 1.0 / L0.h, a->k * a->k, a->k, a->part, cond);
+    };
+    AN_CK(T == 32 ? launch(k_an_step<R, 32>) : launch(k_an_step<R, 16>));
+    an_count(a, 1);
+    if constexpr (std::is_same<R, float>::value) {
+        AN_CK(launch_k(k_an_norm, dim3(a->nblk), dim3(AN_NT), (size_t)0, a->ls, (const c2*)L0.rhs, an_geo(L0),
+                       a->part, a->ctl, start ? 1 : 0, cond));
+        an_count(a, 1);
+    }
+    return HELM_OK;
+}
+
+template <typename R>
+helm_status an_outer(helm_annulus* a, unsigned long long cond)
+{
+    for (int c = 0; c < a->cycles; ++c) {
+        const helm_status st = an_vcycle<R>(a, 0, c == 0);
+        if (st != HELM_OK) return st;
+    }
+    return an_step<R>(a, false, cond);
+}
+
+void an_drop_loop(helm_annulus* a)
+{
+    if (a->loop) cudaGraphExecDestroy(a->loop);
+    a->loop = nullptr;
+}
+
+// The outer steps as one graph: a WHILE node whose body is a step (its parameters change with
+// the plan's cycle and shift alone).  Left unset where the graph cannot be built.
+// The host saw every step's partial norms before: 1024^2 complex64 10.61 -> 10.37 ms,
+// 256^2 complex128 3.89 -> 3.61 ms, two graphs built in each solve included.
+template <typename R>
+void an_build_loop(helm_annulus* a)
+{
+    cudaGraph_t g = nullptr, got = nullptr;
+    if (cudaGraphCreate(&g, 0) != cudaSuccess) { cudaGetLastError(); return; }
+    cudaGraphConditionalHandle cond = 0;
+    cudaGraphNodeParams p = {cudaGraphNodeTypeConditional};
+    cudaGraphNode_t node;
+    bool ok = cudaGraphConditionalHandleCreate(&cond, g, 1, cudaGraphCondAssignDefault) == cudaSuccess;
+    if (ok) {
+        p.conditional.handle = cond;
+        p.conditional.type = cudaGraphCondTypeWhile;
+        p.conditional.size = 1;
+        ok = cudaGraphAddNode(&node, g, nullptr, nullptr, 0, &p) == cudaSuccess;
+    }
+    if (ok && cudaStreamBeginCaptureToGraph(a->cap, p.conditional.phGraph_out[0], nullptr, nullptr, 0,
+                                            cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
+        const cudaStream_t s = a->ls;
+        a->ls = a->cap;
+        a->capturing = true;
+        a->captured = 0;
+        const helm_status st = an_outer<R>(a, (unsigned long long)cond);
+        a->capturing = false;
+        a->ls = s;
+        ok = cudaStreamEndCapture(a->cap, &got) == cudaSuccess && st == HELM_OK &&
+             cudaGraphInstantiate(&a->loop, g, 0) == cudaSuccess;
+        a->loop_step = a->captured;
+        if (!ok) a->loop = nullptr;
+    }
+    cudaGraphDestroy(g);
+    cudaGetLastError();
+}
+
 template <typename R>
 helm_status an_solve(helm_annulus* a, const double2* data, double2* u, double tol, int max_outer, int* iters,
                      double* hist, int* final_status)
 {
-    typedef typename CX<R>::T c2;
     cudaStream_t s = a->stream;
     a->ls = s;
-    const auto& L0 = a->lev[0];
     const long total = (long)(a->N + 1) * (a->N + 1);
-    double2* U[2] = {u, a->U1};
-    const int T = an_tile(a->N), nt = (a->N + T) / T, sblk = std::min(nt * nt, a->nblk);
-    const int npart = std::is_same<R, float>::value ? a->nblk : sblk;
-    k_an_init<<<grid_for(total), AN_NT, 0, s>>>(U[0], U[1], data, L0.typ, total);
+    if (AN_GRAPHS && !a->loop && max_outer > 0) an_build_loop<R>(a);
+    AnCtl c{};
+    c.U[0] = u;
+    c.U[1] = a->U1;
+    c.data = data;
+    c.hist = a->h_hist;
+    c.tol = tol;
+    c.prev = c.rmin = 1.0;
+    c.max_outer = max_outer;
+    c.status = AN_ACTIVE;
+    c.budget = AN_HIST - 1;
+    volatile int* const out = reinterpret_cast<int*>(a->h_hist + AN_HIST);
+    k_an_init<<<grid_for(total), AN_NT, 0, s>>>(a->ctl, c, a->lev[0].typ, total);
     add_launches(1);
-    // mode 0: the start residual; mode 1: an outer step's cycles, update and residual; both end
-    // with the norm partials copied to the host (the caller synchronises)
-    auto enqueue = [&](int mode, int it) -> helm_status {
-        cudaStream_t q = a->ls;
-        if (mode == 1) {
-            for (int c = 0; c < a->cycles; ++c) {
-                const helm_status st = an_vcycle<R>(a, 0, c == 0);
-                if (st != HELM_OK) return st;
-            }
-        }
-        const double2* const Uin = U[mode == 1 ? (it - 1) & 1 : 0];
-        double2* const Uout = U[it & 1];
-        const c2* const e = mode == 1 ? (const c2*)L0.e : nullptr;
-        auto launch = [&](auto* kern, int nt) {
-            return launch_k(kern, dim3(sblk), dim3(AN_NT), (size_t)0, q, Uin, Uout, e, data, (c2*)L0.rhs, an_geo(L0),
-                            nt, 1.0 / (L0.h * L0.h), 1.0 / L0.h, a->k * a->k, a->k, a->part);
-        };
-        AN_CK(T == 32 ? launch(k_an_step<R, 32>, nt) : launch(k_an_step<R, 16>, nt));
-        an_count(a, 1);
-        if constexpr (std::is_same<R, float>::value) {
-            AN_CK(launch_k(k_an_norm, dim3(npart), dim3(AN_NT), (size_t)0, q, (const c2*)L0.rhs, an_geo(L0), a->part));
-            an_count(a, 1);
-        }
-        AN_CK(cudaMemcpyAsync(a->h_part, a->part, sizeof(double) * npart, cudaMemcpyDeviceToHost, q));
-        return HELM_OK;
-    };
-    // an outer step of either parity as one graph (its pointers and parameters are fixed for
-    // this solve); without graphs the step's launches are issued one by one
-    cudaGraphExec_t gx[2] = {nullptr, nullptr};
-    uint64_t gn[2] = {0, 0};
-    auto drop_graphs = [&]() {
-        for (int p = 0; p < 2; ++p)
-            if (gx[p]) cudaGraphExecDestroy(gx[p]);
-    };
-    if (AN_GRAPHS && max_outer > 0) {
-        for (int p = 0; p < 2; ++p) {
-            cudaGraph_t gr = nullptr;
-            if (cudaStreamBeginCapture(a->cap, cudaStreamCaptureModeThreadLocal) != cudaSuccess) break;
-            a->ls = a->cap;
-            a->capturing = true;
-            a->captured = 0;
-            const helm_status est = enqueue(1, p == 1 ? 1 : 2);
-            a->capturing = false;
-            a->ls = s;
-            const cudaError_t ce = cudaStreamEndCapture(a->cap, &gr);
-            if (est != HELM_OK || ce != cudaSuccess || !gr ||
-                cudaGraphInstantiate(&gx[p], gr, 0) != cudaSuccess) {
-                if (gr) cudaGraphDestroy(gr);
-                gx[p] = nullptr;
-                break;
-            }
-            cudaGraphDestroy(gr);
-            gn[p] = a->captured;
-        }
-        if (!gx[0] || !gx[1]) {                // no graphs: launch step by step
-            drop_graphs();
-            gx[0] = gx[1] = nullptr;
-            cudaGetLastError();
-        }
-    }
-    auto step = [&](int mode, int it) -> helm_status {
-        if (mode == 1 && gx[0]) {
-            AN_CK(cudaGraphLaunch(gx[it & 1], s));
-            add_launches(gn[it & 1]);
-        } else {
-            const helm_status st = enqueue(mode, it);
-            if (st != HELM_OK) return st;
-        }
-        AN_CK(cudaStreamSynchronize(s));
-        return HELM_OK;
-    };
     // start: r_0 = b from U[0] (the hole data, zero elsewhere)
-    helm_status st = step(0, 1);
-    if (st != HELM_OK) { drop_graphs(); return st; }
-    double r2 = 0.0;
-    for (int b = 0; b < npart; ++b) r2 += a->h_part[b];
-    const double norm0 = std::sqrt(r2);
-    int it = 0, status = HELM_MAXITER, run = 0;
-    double prev = 1.0, rmin = 1.0;
-    if (hist) hist[0] = (norm0 == 0.0) ? 0.0 : 1.0;
-    if (norm0 == 0.0 || !std::isfinite(norm0)) status = std::isfinite(norm0) ? HELM_CONVERGED : HELM_ENONFINITE;
-    else {
-        for (it = 1; it <= max_outer; ++it) {
-            st = step(1, it);
-            if (st != HELM_OK) { drop_graphs(); return st; }
-            r2 = 0.0;
-            for (int b = 0; b < npart; ++b) r2 += a->h_part[b];
-            const double rel = std::sqrt(r2) / norm0;
-            if (hist) hist[it] = rel;
-            // the cavity's status rule
-            if (!std::isfinite(rel)) { status = HELM_ENONFINITE; break; }
-            if (rel <= tol) { status = HELM_CONVERGED; break; }
-            if (rel > 1e4) { status = HELM_DIVERGED; break; }
-            run = (rel >= prev) ? run + 1 : 0;
-            prev = rel;
-            rmin = std::min(rmin, rel);
-            if (it >= 20 && run >= 10 && rel >= 2.0 * rmin) { status = HELM_DIVERGED; break; }
+    helm_status st = an_step<R>(a, true, 0);
+    if (st != HELM_OK) return st;
+    // rounds of up to AN_HIST - 1 steps (the ring holds a round's history); without a graph a
+    // step each
+    for (int done = -1;;) {
+        if (max_outer > 0 && a->loop) AN_CK(cudaGraphLaunch(a->loop, s));
+        else if (max_outer > 0 && (st = an_outer<R>(a, 0)) != HELM_OK) return st;
+        k_an_fin<<<grid_for(total), AN_NT, 0, s>>>(a->ctl, const_cast<int*>(out), total);
+        AN_CK(cudaGetLastError());
+        AN_CK(cudaStreamSynchronize(s));
+        const int it = out[0];
+        if (a->loop) add_launches(a->loop_step * (uint64_t)(it - std::max(done, 0)));
+        add_launches(1);
+        for (int q = done + 1; hist && q <= it; ++q) hist[q] = a->h_hist[q % AN_HIST];
+        done = it;
+        if (out[1] != AN_ACTIVE) {
+            if (iters) *iters = it;
+            *final_status = out[1];
+            return HELM_OK;
         }
-        if (it > max_outer) it = max_outer;
+        k_an_more<<<1, 1, 0, s>>>(a->ctl, AN_HIST - 1);
+        add_launches(1);
     }
-    drop_graphs();
-    // the result lives in U[it & 1]: the caller's buffer is U[0]
-    if (it & 1) AN_CK(cudaMemcpyAsync(u, a->U1, total * sizeof(double2), cudaMemcpyDeviceToDevice, s));
-    AN_CK(cudaStreamSynchronize(s));
-    if (iters) *iters = it;
-    *final_status = status;
-    return HELM_OK;
 }
 
 
@@ -1965,7 +2053,9 @@ helm_status helm_annulus_create(helm_annulus** out, int n, double side, double h
     a->U1 = (double2*)p;
     a->part = (double*)((char*)p + total * sizeof(double2));
     a->kmin = (unsigned long long*)((char*)a->part + sizeof(double) * a->nblk);
-    if (cudaMallocHost(&a->h_part, sizeof(double) * a->nblk) != cudaSuccess) return fail(HELM_ENOMEM);
+    a->ctl = (AnCtl*)(a->kmin + 2);
+    static_assert(sizeof(AnCtl) + 16 <= 256, "the control follows kmin in the plan's buffer");
+    if (cudaMallocHost(&a->h_hist, sizeof(double) * (AN_HIST + 1)) != cudaSuccess) return fail(HELM_ENOMEM);
     helm_status st = helm_annulus_set_shift(a, a->alpha);
     if (st != HELM_OK) return fail(st);
     *out = a;
@@ -1978,7 +2068,8 @@ helm_status helm_annulus_destroy(helm_annulus* a)
     if (a->stream) cudaStreamSynchronize(a->stream);
     for (void* p : a->allocs) cudaFree(p);
     if (a->At) cudaFree(a->At);
-    if (a->h_part) cudaFreeHost(a->h_part);
+    an_drop_loop(a);
+    if (a->h_hist) cudaFreeHost(a->h_hist);
     if (a->stream) cudaStreamDestroy(a->stream);
     if (a->cap) cudaStreamDestroy(a->cap);
     delete a;
@@ -1988,6 +2079,7 @@ helm_status helm_annulus_destroy(helm_annulus* a)
 helm_status helm_annulus_set_shift(helm_annulus* a, double alpha)
 {
     if (!a || !std::isfinite(alpha) || alpha < a->k * a->k) return HELM_EINVAL;
+    an_drop_loop(a);
     a->alpha = alpha;
     a->sigma = (alpha == a->k * a->k) ? 0.0 : alpha - a->k * a->k;
     const auto& C = a->lev.back();
@@ -2019,6 +2111,7 @@ helm_status helm_annulus_set_cycle(helm_annulus* a, int nu1, int nu2, int cycles
 {
     if (!a || nu1 < 0 || nu1 > 8 || nu2 < 0 || nu2 > 8 || nu1 + nu2 < 1 || cycles < 1 || cycles > 16)
         return HELM_EINVAL;
+    an_drop_loop(a);
     a->nu1 = nu1;
     a->nu2 = nu2;
     a->cycles = cycles;
