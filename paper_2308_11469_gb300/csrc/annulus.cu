@@ -2017,9 +2017,7 @@ helm_status helm_annulus_create(helm_annulus** out, int n, double side, double h
         L.rhs = (char*)L.e + pb;
         L.e2 = (char*)L.rhs + pb;
         if (cudaMemcpy(L.typ, t.data(), pts, cudaMemcpyHostToDevice) != cudaSuccess) return fail(HELM_ECUDA);
-        if (cudaMemset(L.e, 0, pts * eb) != cudaSuccess || cudaMemset(L.rhs, 0, pts * eb) != cudaSuccess ||
-            cudaMemset(L.e2, 0, pts * eb) != cudaSuccess)
-            return fail(HELM_ECUDA);
+        if (cudaMemset(L.e, 0, 3 * pb) != cudaSuccess) return fail(HELM_ECUDA);
         // band: the hole's index box [lo, hi]^2 (centred square) widened by AN_BAND nodes
         int lo = m, hi = 0;
         for (int i = 0; i <= m; ++i)
