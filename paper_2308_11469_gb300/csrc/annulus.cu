@@ -674,11 +674,12 @@ __device__ __forceinline__ void an_dense_solve(const double* At, const int* __re
 // ---------------------------------------------------------------------------
 // The same V-cycle as the tile kernels (sweeps, restriction, prolongation, band sweeps,
 // exact coarsest level), with block-wide barriers between its phases instead of kernel
-// boundaries.  Levels 64, 32, 16, 8 hold about 5.7 K nodes.  In FP64 one SM's arithmetic
-// rate (a small fraction of its FP32 rate) makes the larger of them slower in one CTA than
-// spread over several, so the FP64 tail starts lower.  complex64 from 64: 75 -> 47 us against
-// rows by warps over type bytes and a butterfly per row of the dense solve.
-constexpr int AN_TAIL_TOP_F = 64;
+// boundaries.  complex64 from 32 (1.6 K nodes with 16 and 8): a step of N = 64 takes 49 us, of
+// N = 1024 192; from 64 (5.7 K nodes, whose 2 us half-sweeps one SM makes alone) 60 and 202, from
+// 16 51 and 193.  FP64 from 16: one SM's FP64 rate makes the larger levels slower in one CTA
+// than in tiles.  (From 64, 75 -> 47 us against rows by warps over type bytes and a butterfly
+// per row of the dense solve.)
+constexpr int AN_TAIL_TOP_F = 32;
 constexpr int AN_TAIL_TOP_D = 16;
 constexpr int AN_TAIL_MAX = 4;
 
