@@ -21,7 +21,7 @@
 // bilinear prolongation.  A coarse level represents the hole only to its own spacing, and
 // the coarse-grid correction is poor in the layer between the fine and the coarse hole
 // edges: after each correction a band of a few nodes around the hole is relaxed several
-// times (one CTA), which restores the cycle's contraction (about 0.3 per V(2,2) cycle).
+// times, which restores the cycle's contraction (about 0.3 per V(2,2) cycle).
 #include "../../include/helm.h"
 #include "launch.h"
 #include "pdl.cuh"
@@ -526,11 +526,11 @@ __device__ __forceinline__ typename CX<R>::T an_corrected(typename CX<R>::T v, i
 }
 
 // Ascent of one level: the correction e2 + interpolation of the coarse iterate ec, the band
-// sweeps around the hole, nu2 sweeps; T x T fine nodes go to e_out.  Only the tiles whose window meets the ring make the band sweeps, on a window
-// 2 AN_BAND_SWEEPS nodes wider on every side (their values there are recomputed, the same, by
-// the tiles that share them).  One launch for what were a prolongation (5 us), the band in one
-// CTA (15) and a sweep launch (15-22): complex64 11 us at levels 128 and 256, 13.6 at 512, 28
-// at 1024, cold.
+// sweeps around the hole, nu2 sweeps; T x T fine nodes go to e_out.  Only the tiles whose window
+// meets the ring make the band sweeps, on a window 2 AN_BAND_SWEEPS nodes wider on every side
+// (their values there are recomputed, the same, by the tiles that share them).  One launch for
+// what were a prolongation (5 us), the band in one CTA (15) and a sweep launch (15-22):
+// complex64 9 us at level 64, 10 at 128 and 256, 14 at 512, 28 at 1024, cold.
 template <typename R, int T>
 __global__ void __launch_bounds__(AN_TT, 2)
 k_an_up(const typename CX<R>::T* __restrict__ e2, typename CX<R>::T* __restrict__ e_out,
@@ -2002,23 +2002,33 @@ helm_status helm_annulus_create(helm_annulus** out, int n, double side, double h
     if (cudaStreamCreateWithFlags(&a->cap, cudaStreamNonBlocking) != cudaSuccess) return fail(HELM_ECUDA);
     a->ls = a->stream;
     const size_t eb = prec == HELM_PREC_FP64 ? 16 : 8;
+    // all levels in one allocation: types, iterate, right-hand side, swept iterate of each
+    auto a256 = [](size_t b) { return (b + 255) / 256 * 256; };
+    std::vector<std::vector<unsigned char>> types;
+    size_t bytes = 0;
     for (int m = n; m >= AN_NC; m /= 2) {
-        std::vector<unsigned char> t = an_types(m, side, hole);
-        if (!an_geometry_ok(t, m)) return fail(HELM_EINVAL);
+        types.push_back(an_types(m, side, hole));
+        if (!an_geometry_ok(types.back(), m)) return fail(HELM_EINVAL);
+        const size_t pts = (size_t)(m + 1) * (m + 1);
+        bytes += a256(pts) + 3 * a256(pts * eb);
+    }
+    char* lp = nullptr;
+    if (cudaMalloc((void**)&lp, bytes) != cudaSuccess) return fail(HELM_ENOMEM);
+    a->allocs.push_back(lp);
+    if (cudaMemset(lp, 0, bytes) != cudaSuccess) return fail(HELM_ECUDA);
+    for (int m = n; m >= AN_NC; m /= 2) {
+        const std::vector<unsigned char>& t = types[a->lev.size()];
         helm_annulus::Level L{};
         L.n = m;
         L.h = side / m;
         const size_t pts = (size_t)(m + 1) * (m + 1);
-        void* p = nullptr;
-        const size_t pb = ((pts * eb + 255) / 256) * 256;
-        if (cudaMalloc(&p, ((pts + 255) / 256) * 256 + 3 * pb) != cudaSuccess) return fail(HELM_ENOMEM);
-        a->allocs.push_back(p);
-        L.typ = (unsigned char*)p;
-        L.e = (char*)p + ((pts + 255) / 256) * 256;
+        const size_t pb = a256(pts * eb);
+        L.typ = (unsigned char*)lp;
+        L.e = lp + a256(pts);
         L.rhs = (char*)L.e + pb;
         L.e2 = (char*)L.rhs + pb;
+        lp += a256(pts) + 3 * pb;
         if (cudaMemcpy(L.typ, t.data(), pts, cudaMemcpyHostToDevice) != cudaSuccess) return fail(HELM_ECUDA);
-        if (cudaMemset(L.e, 0, 3 * pb) != cudaSuccess) return fail(HELM_ECUDA);
         // band: the hole's index box [lo, hi]^2 (centred square) widened by AN_BAND nodes
         int lo = m, hi = 0;
         for (int i = 0; i <= m; ++i)
