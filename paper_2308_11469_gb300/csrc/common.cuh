@@ -64,8 +64,9 @@ struct InstDesc {
     const double2* f;
     const double2* g;
     double* part;               // [2 * nres_blocks]: sum |r|^2 partials, then max |e|^2
-    unsigned int* count;        // [0] residual tiles finished in the current launch, [1] (3D)
-                                // the largest biased exponent of the iterate they formed
+    unsigned int* count;        // residual tiles finished in the current launch
+    int* tex;                   // 3D: per residual tile the scale of its next step's residual: the
+                                // largest biased exponent that its window of the iterate held, or 0
     double* hist;               // relres_0..relres_max_outer
     double* einf;               // ||e_N||_inf, N = 0..max_outer-1
     LevelDesc lev[HELM_MAXLEV];
@@ -75,7 +76,7 @@ struct InstState {
     int status;      // HELM_ST_ACTIVE while iterating, else the outcome
     int it;          // outer steps performed (u_it lives in u[it & 1])
     int run;         // consecutive non-decreasing relres steps
-    int uex;         // 3D: largest biased exponent among u_it's components (0: not known)
+    int pad_;
     double norm0;    // ||r_0||_2
     double prev;     // relres of the previous step
     double rmin;     // smallest relres so far

@@ -123,6 +123,10 @@ size_t layout(InstDesc& d, int D, int n, double h, double k, int prec, char* bas
     off += align256((size_t)2 * d.nres_blocks * sizeof(double));
     if (base) d.count = (unsigned int*)(base + off);
     off += 256;
+    if (D == 3) {
+        if (base) d.tex = (int*)(base + off);
+        off += align256((size_t)d.nres_blocks * sizeof(int));
+    }
     set_shift(d, 0.0);
     return off;
 }

@@ -542,31 +542,36 @@ k_upres2d(const InstDesc* __restrict__ insts, InstState* __restrict__ st,
 // three-plane ring of shared memory (1-node halo in x and y)
 // ---------------------------------------------------------------------------
 constexpr int T3X = 32, T3Y = 8, T3Z = 16;
-// Resident CTAs per SM of the 3D residual: 64 registers at 4, which hold a column's planes and
-// the next plane's words in flight (255^3 complex64 solve 15.2 ms on per-plane scales, 6 CTAs;
-// on the instance's scale with 3, 4, 5 CTAs 14.0, 14.0, 16.5; three warps of their own for the
-// ring 15.6, the ring's next words in registers 14.0 at 3 and 15.4 at 4).
+// Resident CTAs per SM of the 3D residual.  On the tile's scale 64 registers at 4, which hold a
+// column's planes and the next plane's words in flight (255^3 complex64 solve 14.0 ms with 3 or 4
+// CTAs, 16.5 with 5; three warps of their own for the ring 15.6).
 constexpr int RES3D_CTAS = 4;
 constexpr int P3 = (T3X + 2) * (T3Y + 2);
 constexpr int RING3 = 2 * (T3X + 2) + 2 * T3Y;
 
-// Per-step form (u_{N+1} = u_N + e_N and r_{N+1}), with h^2 a power of two and the whole
-// instance on one fixed-point scale: four times the largest value of u_N (InstState::uex).  A
-// thread keeps its column's values of planes z - 1, z, z + 1 in registers; a plane's window goes
-// through two slots of shared memory, one barrier a plane, and no exponent has to be reduced or
-// shifted to.  f - k^2 u (+ i p u) is formed in FP64 and joins the numerator in fixed point, so
-// h^2 r is one exact sum, rounded once to the inner precision:
+// Per-step form (u_{N+1} = u_N + e_N and r_{N+1}) where h^2 is a power of two: the tile's window on
+// one fixed-point scale, that of its largest value in u_N (InstDesc::tex), with room for values
+// up to twice it.  A thread keeps its column's values of planes z - 1, z, z + 1 in registers; a
+// plane's window goes through two slots of shared memory, one barrier a plane, and no exponent
+// has to be reduced before it or shifted to.  f - k^2 u (+ i p u) is formed in FP64 and joins the
+// numerator in fixed point, so h^2 r is one integer sum, rounded once to the inner precision:
 //   h^2 r = h^2 (f - k^2 u + i p u) - (sum of neighbours - 6 u).
-// One unit is 2^-56 of the instance's largest value (FP64 rounds its terms at 2^-53 of their
-// own).  Values beyond the scale (an iterate growing more than fourfold in a step, a source or a
-// wall far above it, an infinity or a NaN) are seen in the largest exponent the tile meets:
-// false, and the tile is redone on per-plane scales.
+// em: the scale, eg: em less the exponents that h^2 adds.  One unit is 2^-57 .. 2^-58 of the
+// tile's largest value.  The node values are truncated to it, as in the per-plane form below: what
+// that leaves out has the same mean at a node and at its neighbours, and cancels in the numerator.
+// h^2 (f - k^2 u) is rounded to nearest: truncated, it would be half a unit short at every node,
+// of one sign over whole regions, which the inverse amplifies by N^2 / 30.  No plane of the tile
+// may lie, with the planes beside it, below 2^-4 of the scale: no term is off by more than 2^-53
+// of the largest value on the three planes it joins, the size of FP64's own roundings.
+// A tile that leaves the scale at either end (an iterate that more than doubles in a step or
+// decays across the tile, a source or a wall far above it, an infinity or a NaN) is found out by
+// the exponents that it meets: false, and the tile is redone on per-plane scales.
 // About 330 integer instructions and 4.7 FP64 operations a point (577 and 6.7 on per-plane
-// scales); bound by its load and barrier latency: 255^3 complex64 382 -> 330 us a launch, 3.2 TB/s
-// of its 64 bytes a point.
+// scales); bound by its load and barrier latency.  255^3 complex64 plane wave, 19 steps: 15.11 ms
+// with the per-plane form in every step, 14.44 with this one (random data, a step: 757 us, 740).
 template <typename R, bool DAMP>
 __device__ __forceinline__ bool residual3d_tile_scaled(const InstDesc& I, const InstState& s, const ResItem item,
-                                                       longlong2 (*U)[P3], int* sx, int add, R& r2_out, R& em_out,
+                                                       longlong2 (*U)[P3], int em, int eg, R& r2_out, R& em_out,
                                                        int& ex_out)
 {
     typedef typename C2<R>::T c2;
@@ -584,7 +589,13 @@ __device__ __forceinline__ bool residual3d_tile_scaled(const InstDesc& I, const 
     c2* __restrict__ rhs = (c2*)L0.rhs;            // (a 3D level has one right-hand side)
     const unsigned P = L0.pitch, PL = P * L0.rows;
     const double mk2 = -I.k2, damp = I.damp;
-    const int em = s.uex + 2;
+    // planes (bit z - z0 + 1) with a value of exponent em - 4 or more, largest exponent of the tile
+    __shared__ unsigned seen;
+    __shared__ int exm;
+    if (threadIdx.x == 0) {
+        seen = 0u;
+        exm = 0;
+    }
     const int x0 = 1 + item.tx * T3X, y0 = 1 + item.ty * T3Y, z0 = 1 + item.tz * T3Z;
     const int z1 = min(z0 + T3Z - 1, n);
     const int lx = (threadIdx.x & 31) + 1, ly = (threadIdx.x >> 5) + 1;
@@ -611,7 +622,8 @@ __device__ __forceinline__ bool residual3d_tile_scaled(const InstDesc& I, const 
         if (rin) ur = ry * S + rx;
         if (rint) er = ry * P + xslot<3>(rx, (int)P);
     }
-    unsigned top = 0, gtop = 0;                    // largest high words met (sign off)
+    unsigned got = 0;                              // the warp's share of seen
+    unsigned top = 0, pl = 0;                      // largest high word (sign off): of all, of the plane in hand
     R r2 = 0, emax2 = 0;
     auto hi = [](double v) { return (unsigned)__double2hiint(v) & 0x7fffffffu; };
     // the node's raw words (own: registers), fetched one plane ahead
@@ -631,7 +643,7 @@ __device__ __forceinline__ bool residual3d_tile_scaled(const InstDesc& I, const 
     auto sum = [&](double2 v, c2 ev) -> double2 {
         v.x += Inner<R>::widen(ev.x);
         v.y += Inner<R>::widen(ev.y);
-        top = max(top, max(hi(v.x), hi(v.y)));
+        pl = max(pl, max(hi(v.x), hi(v.y)));
         return v;
     };
     auto fix = [&](double2 v) { return make_longlong2(fx_qt(v.x, em), fx_qt(v.y, em)); };
@@ -641,9 +653,15 @@ __device__ __forceinline__ bool residual3d_tile_scaled(const InstDesc& I, const 
             U[z & 1][ro] = fix(sum(Ru[threadIdx.x], Re[threadIdx.x]));
         }
     };
+    auto met = [&](int z) {                        // all of plane z's values are formed
+        if (__any_sync(0xffffffffu, (int)(pl >> 20) >= em - 4)) got |= 1u << (z - z0 + 1);
+        top = max(top, pl);
+        pl = 0;
+    };
     fetch_ring(z0);
     fetch(z0 - 1);
     longlong2 dn = fix(sum(nu, ne));
+    met(z0 - 1);
     fetch(z0);
     if (live) nf = f[(z0 - 1) * NP + fo];
     double2 cur = sum(nu, ne);
@@ -651,6 +669,7 @@ __device__ __forceinline__ bool residual3d_tile_scaled(const InstDesc& I, const 
     longlong2 fc = fix(cur);
     U[z0 & 1][o] = fc;
     stage_ring(z0);
+    met(z0);
     if (z0 < z1) fetch_ring(z0 + 1);
     fetch(z0 + 1);
     __syncthreads();
@@ -663,6 +682,7 @@ __device__ __forceinline__ bool residual3d_tile_scaled(const InstDesc& I, const 
             U[(z + 1) & 1][o] = up;
             stage_ring(z + 1);
         }
+        met(z + 1);
         double2 g = make_double2(fma(cur.x, mk2, nf.x), fma(cur.y, mk2, nf.y));
         if (more) {
             fetch(z + 2);                          // (z + 2 <= n + 1)
@@ -676,14 +696,14 @@ __device__ __forceinline__ bool residual3d_tile_scaled(const InstDesc& I, const 
                 g.x = fma(cur.y, damp, g.x);
                 g.y = fma(cur.x, -damp, g.y);
             }
-            gtop = max(gtop, max(hi(g.x), hi(g.y)));
-            const long long Gx = fx_qt(g.x, em - add), Gy = fx_qt(g.y, em - add);
+            if ((int)(max(hi(g.x), hi(g.y)) >> 20) > eg + 1) pl = 0x7ff00000u;     // off the scale: as an infinity
+            const long long Gx = fx_q(g.x, eg), Gy = fx_q(g.y, eg);
             const long long tx = (Gx - ((W.x + E.x) + (So.x + No.x))) - ((dn.x + up.x) - 6 * fc.x);
             const long long ty = (Gy - ((W.y + E.y) + (So.y + No.y))) - ((dn.y + up.y) - 6 * fc.y);
             uout[z * SP + uo] = cur;
             c2 ri;
-            ri.x = fx_inner(tx, em - add, R());
-            ri.y = fx_inner(ty, em - add, R());
+            ri.x = fx_inner(tx, eg, R());
+            ri.y = fx_inner(ty, eg, R());
             rhs[z * PL + eo] = ri;
             r2 += abs2(ri);
         }
@@ -692,14 +712,17 @@ __device__ __forceinline__ bool residual3d_tile_scaled(const InstDesc& I, const 
         cur = nxt;
         __syncthreads();
     }
-    const int ex = block_max_exp<NTH>((int)(top >> 20), sx);
-    __syncthreads();
-    const int eg = block_max_exp<NTH>((int)(gtop >> 20), sx);
-    __syncthreads();
+    top = __reduce_max_sync(0xffffffffu, top) >> 20;
+    if ((threadIdx.x & 31) == 0) {
+        atomicOr(&seen, got);
+        atomicMax(&exm, (int)top);
+    }
+    const bool off = __syncthreads_or(pl != 0u);
     r2_out = r2;
     em_out = emax2;
-    ex_out = ex;
-    return ex <= em && (eg == 0 || eg + add <= em);
+    const unsigned want = (2u << (z1 - z0)) - 1u, near = seen | seen >> 1 | seen >> 2;
+    ex_out = exm;
+    return !off && exm <= em + 1 && (near & want) == want;
 }
 
 // The column's planes go through the ring in fixed point
@@ -707,10 +730,11 @@ __device__ __forceinline__ bool residual3d_tile_scaled(const InstDesc& I, const 
 // plane z is summed on the largest scale of planes z - 1, z, z + 1 (the other planes'
 // values shifted down to it), so every node's numerator is exact up to the truncations.
 // Thread t stages the interior node (t mod 32, t / 32) of each plane and keeps it in FP64
-// for its own residual; threads below the ring size stage one ring node each.
-// (not inlined beside the form above, whose registers it would share)
+// for its own residual; threads below the ring size stage one ring node each.  Leaves the
+// tile's scale for the form above in InstDesc::tex, or 0 where a plane and its neighbours lie
+// below 2^-3 of the tile's largest value.
 template <typename R, int MODE, bool DAMP>
-__device__ __noinline__ void residual3d_tile_fx(const InstDesc* __restrict__ insts,
+__device__ __forceinline__ void residual3d_tile_fx(const InstDesc* __restrict__ insts,
                                                    InstState* __restrict__ st, const ResItem item,
                                                    longlong2 (*U)[P3], int* sx, const StepCtl& c)
 {
@@ -729,7 +753,11 @@ __device__ __noinline__ void residual3d_tile_fx(const InstDesc* __restrict__ ins
         return;
     }
     const int tile = (item.tz * I.res_ty + item.ty) * I.res_tx + item.tx;
-    int exm = 0;                                   // largest exponent of the tile's iterate
+    __shared__ int exm, exl;                       // largest exponent of the tile, least of a plane and its neighbours
+    if (threadIdx.x == 0) {                        // (thread 0's)
+        exm = 0;
+        exl = 2047;
+    }
     const double2* __restrict__ uin = (s.it & 1) ? I.u[1] : I.u[0];
     double2* __restrict__ uout = (double2*)((s.it & 1) ? I.u[0] : I.u[1]);
     const double2* __restrict__ f = I.f;
@@ -774,7 +802,7 @@ __device__ __noinline__ void residual3d_tile_fx(const InstDesc* __restrict__ ins
         double2 rv = make_double2(0.0, 0.0);
         if (threadIdx.x < RING) rv = node(rlx, rly, gz, false);
         const int raw = block_max_exp<NTH>(max(fx_exp2(mine), fx_exp2(rv)), sx);
-        exm = max(exm, raw);
+        if (threadIdx.x == 0) exm = max(exm, raw);
         const int ep = fx_scale(raw);
         U[slot][o] = fx_fix2(mine, ep);
         if (threadIdx.x < RING) U[slot][ro] = fx_fix2(rv, ep);
@@ -836,13 +864,23 @@ __device__ __noinline__ void residual3d_tile_fx(const InstDesc* __restrict__ ins
             if (MODE == 1) r2 += abs2(ri);
         }
         cur = nxt;
+        if (threadIdx.x == 0) exl = min(exl, max(max(ep[sp], ep[sc]), ep[sn]));
         const int t = sp;
         sp = sc;
         sc = sn;
         sn = t;
     }
-    if constexpr (MODE == 0) tile_done<double>(I, stp, tile, r2d, b2, MODE, st, c, exm);
-    else tile_done<R>(I, stp, tile, r2, emax2, MODE, st, c, exm);
+    if (threadIdx.x == 0) I.tex[tile] = exm <= FX_EMAX && exl >= exm - 3 ? exm : 0;
+    if constexpr (MODE == 0) tile_done<double>(I, stp, tile, r2d, b2, MODE, st, c);
+    else tile_done<R>(I, stp, tile, r2, emax2, MODE, st, c);
+}
+
+// (not inlined beside the scaled form, whose registers it would share)
+template <typename R, bool DAMP>
+__device__ __noinline__ void residual3d_tile_redo(const InstDesc* __restrict__ insts, InstState* __restrict__ st,
+                                                  const ResItem item, longlong2 (*U)[P3], int* sx, const StepCtl& c)
+{
+    residual3d_tile_fx<R, 1, DAMP>(insts, st, item, U, sx, c);
 }
 
 // (the start residual, once per solve, also forms ||b||: it runs at 4 CTAs per SM, whose 64
@@ -859,23 +897,31 @@ k_residual3d(const InstDesc* __restrict__ insts, InstState* __restrict__ st,
     for (int t = blockIdx.x; t < nitems; t += gridDim.x) {
         const ResItem item = items[t];
         longlong2(*const F)[P3] = reinterpret_cast<longlong2(*)[P3]>(U);
-        bool done = false;
         if constexpr (MODE == 1) {
-            // the whole instance on the scale of its last iterate, where that is known
+            // on the tile's scale, which the start (zero in general) does not tell
             const InstDesc& I = insts[item.inst];
             const InstState s = st[item.inst];
-            const FxH2 hh(I.lev[0].h2);
-            if (s.status == HELM_ST_ACTIVE && hh.pow2 && s.uex > 0 && s.it > 0 && hh.usable(s.uex + 2) && I.n <= 1023) {
-                R r2, em;
-                int ex;
-                done = residual3d_tile_scaled<R, DAMP>(I, s, item, F, sx, hh.add, r2, em, ex);
-                if (done)
-                    tile_done<R>(I, st + item.inst, (item.tz * I.res_ty + item.ty) * I.res_tx + item.tx, r2, em, MODE,
-                                 st, c, ex);
-                __syncthreads();
+            bool done = false;
+            if (s.status == HELM_ST_ACTIVE && s.it > 0 && I.n <= 1023) {
+                const int tile = (item.tz * I.res_ty + item.ty) * I.res_tx + item.tx;
+                // (a load that stays here: moved into the form below it costs it 70 bytes of spills)
+                const int scale = __ldcg(I.tex + tile);
+                const FxH2 hh(I.lev[0].h2);
+                if (hh.pow2 && hh.usable(scale)) {
+                    R r2, em2;
+                    int ex;
+                    done = residual3d_tile_scaled<R, DAMP>(I, s, item, F, scale, scale - hh.add, r2, em2, ex);
+                    if (done) {
+                        if (threadIdx.x == 0) I.tex[tile] = ex;
+                        tile_done<R>(I, st + item.inst, tile, r2, em2, MODE, st, c);
+                    }
+                    __syncthreads();
+                }
             }
+            if (!done) residual3d_tile_redo<R, DAMP>(insts, st, item, F, sx, c);
+        } else {
+            residual3d_tile_fx<R, MODE, DAMP>(insts, st, item, F, sx, c);
         }
-        if (!done) residual3d_tile_fx<R, MODE, DAMP>(insts, st, item, F, sx, c);
         __syncthreads();
     }
 }

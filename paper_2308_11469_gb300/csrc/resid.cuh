@@ -238,18 +238,15 @@ __device__ void instance_last(const InstDesc& I, InstState* stp, int mode, const
     if (mode != 0 && threadIdx.x == 32) I.einf[it] = sqrt(sm[0]);
     if (threadIdx.x == 0) {
         finalize(I, stp, fa, fm, mode);
-        I.count[0] = 0u;
-        stp->uex = (int)__ldcg(I.count + 1);
-        I.count[1] = 0u;
+        *I.count = 0u;
     }
     if (c.ctrl) step_arrive(st_all, c);
 }
 
-// Write this tile's partials; the last tile of the instance reduces them all.  ex: the largest
-// biased exponent of the iterate on the tile (3D).
+// Write this tile's partials; the last tile of the instance reduces them all.
 template <typename T>
 __device__ void tile_done(const InstDesc& I, InstState* stp, int tile, T ta0, T tm0, int mode,
-                          const InstState* st_all, const StepCtl& c, int ex = 0)
+                          const InstState* st_all, const StepCtl& c)
 {
     __shared__ double sa[NTH / 32], sm[NTH / 32];
     __shared__ int last;
@@ -258,7 +255,6 @@ __device__ void tile_done(const InstDesc& I, InstState* stp, int tile, T ta0, T 
     if (threadIdx.x == 0) {
         I.part[tile] = a;
         I.part[I.nres_blocks + tile] = m;
-        if (ex) atomicMax(I.count + 1, (unsigned)ex);
         __threadfence();
         const unsigned prev = atomicAdd(I.count, 1u);
         last = (prev == (unsigned)(I.nres_blocks - 1));
