@@ -66,6 +66,13 @@ int res_rows_per_tile(int D) { return residual_tile_rows(D); }
 // residual tiles along z: 3D tiles march over residual_tile_planes(3) planes; 2D has one
 int res_tz(int D, int n) { return D == 3 ? (n + residual_tile_planes(3) - 1) / residual_tile_planes(3) : 1; }
 
+// is h^2 a power of two?
+bool pow2_h2(const InstDesc& d)
+{
+    int e = 0;
+    return std::frexp(d.lev[0].h2, &e) == 0.5;
+}
+
 // Fill the geometry part of a descriptor and return the workspace bytes it needs (the
 // level arrays, the second iterate buffer and the residual partials).  With base != NULL
 // the pointers are carved out of it.
@@ -167,7 +174,7 @@ struct PlanState {
     size_t mg_cap = 0;
     ResItem* d_res = nullptr;
     size_t res_cap = 0;
-    int nres = 0, max_tail = 1, damp_any = 0, small_cs = 0, l0_off = 0, l0_cnt = 0;
+    int nres = 0, max_tail = 1, damp_any = 0, pow2_any = 0, small_cs = 0, l0_off = 0, l0_cnt = 0;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     cudaGraphConditionalHandle cond = 0;
@@ -247,6 +254,7 @@ struct Engine {
     std::vector<LaunchRec> vcyc_plain;         // one V-cycle from the current iterate
     int max_tail = 1;
     int damp_any = 0;                          // some slot's instance has p != 0
+    int pow2_any = 0;                          // ... a spacing whose square is a power of two
     // 2D complex64 solves of one small size run all their steps in one launch of a cluster
     // of small_cs CTAs each (small2d.cu; 0: launch by launch), from their level-0 items
     int small_cs = 0, l0_off = 0, l0_cnt = 0;
@@ -274,6 +282,7 @@ struct Engine {
         std::swap(nres, p.nres);
         std::swap(max_tail, p.max_tail);
         std::swap(damp_any, p.damp_any);
+        std::swap(pow2_any, p.pow2_any);
         std::swap(small_cs, p.small_cs);
         std::swap(l0_off, p.l0_off);
         std::swap(l0_cnt, p.l0_cnt);
@@ -564,7 +573,10 @@ struct Engine {
         damp_any = 0;
         for (int i = 0; i < cap; ++i) {
             nocc += slots[i] ? 1 : 0;
-            if (slots[i] && slots[i]->d.damp != 0.0) damp_any = 1;
+            if (slots[i]) {
+                if (slots[i]->d.damp != 0.0) damp_any = 1;
+                if (pow2_h2(slots[i]->d)) pow2_any = 1;
+            }
         }
         // 2D complex64 instances of one size whose level 0 is a fused level: level 0's final
         // ascent and the residual launch become one kernel (k_upres2d)
@@ -702,10 +714,10 @@ struct Engine {
                 if (L.color)      // folded step control: L.work instances, cap statuses
                     e = launch_residual(D, prec, d_desc, d_state, d_res + L.off, L.cnt, L.mode, s,
                                         d_ctrl, cap, L.work, use_cond ? 1 : 0, (unsigned long long)cond,
-                                        damp_any);
+                                        damp_any, pow2_any);
                 else
                     e = launch_residual(D, prec, d_desc, d_state, d_res + L.off, L.cnt, L.mode, s,
-                                        nullptr, 0, 0, 0, 0, damp_any);
+                                        nullptr, 0, 0, 0, 0, damp_any, pow2_any);
                 break;
             case LaunchRec::UPRES:     // color: level 1 fused
                 e = launch_upres2d(d_desc, d_state, d_mg + L.off, L.cnt, L.nmax, nu2, L.mode, s, d_ctrl, cap,
@@ -764,17 +776,20 @@ struct Engine {
         return HELM_OK;
     }
 
-    // What the launch plan and its graph depend on: the slot geometry, the cycle, and
-    // whether any instance has a damping term (it selects the residual kernels' variant).
+    // What the launch plan and its graph depend on: the slot geometry, the cycle, and whether
+    // any instance has a damping term or a power of two for h^2 (they select the residual
+    // kernels' variants).
     std::vector<long> current_signature() const
     {
         std::vector<long> sig{cap, nu1, nu2, cycles, tiles, coarse, (latency ? 1L : 0L) + (mixed_sizes ? 2L : 0L)};
-        long damp = 0;
+        long damp = 0, pow2 = 0;
         for (int i = 0; i < cap; ++i) {
             sig.push_back(slots[i] ? (long)slots[i]->d.n * 4 + (long)slots[i]->d.D : -1L);
             if (slots[i] && slots[i]->d.damp != 0.0) damp = 1;
+            if (slots[i] && pow2_h2(slots[i]->d)) pow2 = 1;
         }
         sig.push_back(damp);
+        sig.push_back(pow2);
         return sig;
     }
 

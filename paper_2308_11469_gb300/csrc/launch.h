@@ -131,11 +131,12 @@ cudaError_t setup_2d(int prec);
 // ctrl != nullptr folds the step control (k_check) into the launch: the last of the
 // launch's `ninst` instances to finish its residual scans `nscan` statuses, counts the
 // step and sets the WHILE node's condition (use_cond).  damp != 0: some instance has a
-// damping term p (the kernel variant that forms it).
+// damping term p (the kernel variant that forms it); pow2 != 0 (3D, mode 1): some instance's
+// h^2 is a power of two (the variant with a form of its own for it).
 cudaError_t launch_residual(int D, int prec, const InstDesc* insts, InstState* st,
                             const ResItem* items, int nitems, int mode, cudaStream_t s,
                             int* ctrl = nullptr, int nscan = 0, int ninst = 0, int use_cond = 0,
-                            unsigned long long cond_handle = 0, int damp = 0);
+                            unsigned long long cond_handle = 0, int damp = 0, int pow2 = 0);
 // 2D, complex64 inner solves: level 0's ascent (launch_up2d with nu2 sweeps, e2_mode)
 // fused with the mode-1 residual launch and its folded step control (same arguments as
 // launch_residual's).  items: the level-0 items of every instance (all of size n), whose

@@ -544,8 +544,9 @@ k_upres2d(const InstDesc* __restrict__ insts, InstState* __restrict__ st,
 constexpr int T3X = 32, T3Y = 8, T3Z = 16;
 // Resident CTAs per SM of the 3D residual.  On the tile's scale 64 registers at 4, which hold a
 // column's planes and the next plane's words in flight (255^3 complex64 solve 14.0 ms with 3 or 4
-// CTAs, 16.5 with 5; three warps of their own for the ring 15.6).
-constexpr int RES3D_CTAS = 4;
+// CTAs, 16.5 with 5; three warps of their own for the ring 15.6); on per-plane scales 40 at 6
+// (383 us a launch against 450 at 4).
+constexpr int RES3D_CTAS = 4, RES3D_PLANE_CTAS = 6;
 constexpr int P3 = (T3X + 2) * (T3Y + 2);
 constexpr int RING3 = 2 * (T3X + 2) + 2 * T3Y;
 
@@ -883,10 +884,12 @@ __device__ __noinline__ void residual3d_tile_redo(const InstDesc* __restrict__ i
     residual3d_tile_fx<R, 1, DAMP>(insts, st, item, U, sx, c);
 }
 
+// SCALED: some instance of the launch has a power of two for h^2 (mode 1; without one the
+// per-plane form has the kernel to itself).
 // (the start residual, once per solve, also forms ||b||: it runs at 4 CTAs per SM, whose 64
 // registers cut its spills from 260 to 88 bytes)
-template <typename R, int MODE, bool DAMP>
-__global__ void __launch_bounds__(NTH, MODE == 1 ? RES3D_CTAS : 4)
+template <typename R, int MODE, bool DAMP, bool SCALED>
+__global__ void __launch_bounds__(NTH, MODE == 0 ? 4 : SCALED ? RES3D_CTAS : RES3D_PLANE_CTAS)
 k_residual3d(const InstDesc* __restrict__ insts, InstState* __restrict__ st,
              const ResItem* __restrict__ items, int nitems, StepCtl c)
 {
@@ -897,7 +900,7 @@ k_residual3d(const InstDesc* __restrict__ insts, InstState* __restrict__ st,
     for (int t = blockIdx.x; t < nitems; t += gridDim.x) {
         const ResItem item = items[t];
         longlong2(*const F)[P3] = reinterpret_cast<longlong2(*)[P3]>(U);
-        if constexpr (MODE == 1) {
+        if constexpr (SCALED) {
             // on the tile's scale, which the start (zero in general) does not tell
             const InstDesc& I = insts[item.inst];
             const InstState s = st[item.inst];
@@ -1381,7 +1384,7 @@ cudaError_t run_fp64_rate(double* tflops, double* ms_best)
 cudaError_t launch_residual(int D, int prec, const InstDesc* insts, InstState* st,
                             const ResItem* items, int nitems, int mode, cudaStream_t s,
                             int* ctrl, int nscan, int ninst, int use_cond,
-                            unsigned long long cond_handle, int damp)
+                            unsigned long long cond_handle, int damp, int pow2)
 {
     if (nitems <= 0) return cudaSuccess;
     const StepCtl c{ctrl, nscan, ninst, use_cond, cond_handle};
@@ -1390,15 +1393,17 @@ cudaError_t launch_residual(int D, int prec, const InstDesc* insts, InstState* s
     // persistent CTAs double-buffer their next tile with asynchronous copies (1023^2, one
     // instance: 43 us against 48-49 us); 32 x 32 tiles beat 32 x 8/16/40/64 rows
     const int grid = nitems;
-#define HELM_RES(K, RR)                                                                        \
-    (damp ? (mode ? launch_k(K<RR, 1, true>, dim3(grid), dim3(NTH), 0, s, insts, st, items, nitems, c)  \
-                  : launch_k(K<RR, 0, true>, dim3(grid), dim3(NTH), 0, s, insts, st, items, nitems, c)) \
-          : (mode ? launch_k(K<RR, 1, false>, dim3(grid), dim3(NTH), 0, s, insts, st, items, nitems, c) \
-                  : launch_k(K<RR, 0, false>, dim3(grid), dim3(NTH), 0, s, insts, st, items, nitems, c)))
-    if (D == 2 && prec == 0) HELM_RES(k_residual2d, double);
-    else if (D == 2) HELM_RES(k_residual2d, float);
-    else if (prec == 0) HELM_RES(k_residual3d, double);
-    else HELM_RES(k_residual3d, float);
+#define HELM_RES(K, ...) launch_k(K<__VA_ARGS__>, dim3(grid), dim3(NTH), 0, s, insts, st, items, nitems, c)
+#define HELM_RES2(RR, DD) (mode ? HELM_RES(k_residual2d, RR, 1, DD) : HELM_RES(k_residual2d, RR, 0, DD))
+#define HELM_RES3(RR, DD)                                                                      \
+    (!mode ? HELM_RES(k_residual3d, RR, 0, DD, false)                                          \
+           : pow2 ? HELM_RES(k_residual3d, RR, 1, DD, true) : HELM_RES(k_residual3d, RR, 1, DD, false))
+    if (D == 2 && prec == 0) damp ? HELM_RES2(double, true) : HELM_RES2(double, false);
+    else if (D == 2) damp ? HELM_RES2(float, true) : HELM_RES2(float, false);
+    else if (prec == 0) damp ? HELM_RES3(double, true) : HELM_RES3(double, false);
+    else damp ? HELM_RES3(float, true) : HELM_RES3(float, false);
+#undef HELM_RES3
+#undef HELM_RES2
 #undef HELM_RES
     return cudaGetLastError();
 }
@@ -1463,17 +1468,18 @@ cudaError_t setup_upres()
 cudaError_t setup_outer()
 {
     cudaError_t e;
-#define HELM_CO(K)                                                                   \
-    if ((e = max_carveout(K<float, 0, false>)) != cudaSuccess) return e;             \
-    if ((e = max_carveout(K<float, 1, false>)) != cudaSuccess) return e;             \
-    if ((e = max_carveout(K<double, 0, false>)) != cudaSuccess) return e;            \
-    if ((e = max_carveout(K<double, 1, false>)) != cudaSuccess) return e;            \
-    if ((e = max_carveout(K<float, 0, true>)) != cudaSuccess) return e;              \
-    if ((e = max_carveout(K<float, 1, true>)) != cudaSuccess) return e;              \
-    if ((e = max_carveout(K<double, 0, true>)) != cudaSuccess) return e;             \
-    if ((e = max_carveout(K<double, 1, true>)) != cudaSuccess) return e;
-    HELM_CO(k_residual2d)
-    HELM_CO(k_residual3d)
+#define HELM_CO(...) if ((e = max_carveout(__VA_ARGS__)) != cudaSuccess) return e;
+#define HELM_CO4(R, DD)                          \
+    HELM_CO(k_residual2d<R, 0, DD>)              \
+    HELM_CO(k_residual2d<R, 1, DD>)              \
+    HELM_CO(k_residual3d<R, 0, DD, false>)       \
+    HELM_CO(k_residual3d<R, 1, DD, false>)       \
+    HELM_CO(k_residual3d<R, 1, DD, true>)
+    HELM_CO4(float, false)
+    HELM_CO4(float, true)
+    HELM_CO4(double, false)
+    HELM_CO4(double, true)
+#undef HELM_CO4
 #undef HELM_CO
     if ((e = setup_upres<0>()) != cudaSuccess) return e;
     if ((e = setup_upres<1>()) != cudaSuccess) return e;

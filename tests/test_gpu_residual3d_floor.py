@@ -83,3 +83,30 @@ def test_field_that_decays_across_the_box(n, prec, side, data):
         if data == "steep":
             worst = worst[near >= 2.0 ** -16 * near.max()]
         assert worst.max() <= 32 * U53, (int(worst.argmax()) + 1, worst.max() / U53)
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+def test_one_launch_for_both_kinds_of_spacing(prec):
+    # a batch whose solves share a launch, with and without a power of two for h^2: each gets the
+    # bits of its solve alone
+    from paper_2308_11469_gb300 import binding as B
+    n = 63
+    rng = np.random.default_rng(5)
+    f = torch.from_numpy(rng.standard_normal((n,) * 3) + 1j * rng.standard_normal((n,) * 3)).cuda()
+    g = torch.from_numpy(rng.standard_normal((n + 2,) * 3) + 1j * rng.standard_normal((n + 2,) * 3)).cuda()
+    hs = [1.0 / (n + 1), 0.7 / (n + 1), 0.7 / (n + 1)]
+    batch = B.helm_batch_create(0)
+    B.helm_batch_set_cycle(batch, 0, 2, 1)
+    B.helm_batch_set_lanes(batch, 1)
+    us = [torch.zeros_like(g) for _ in hs]
+    ts = B.helm_batch_submit_many(batch, [(3, n, h, 2.0, f, g, u) for h, u in zip(hs, us)], prec, 1e-9, 60)
+    B.helm_batch_step(batch, 0)
+    got = [B.helm_batch_poll(batch, t, 60) for t in ts]
+    B.helm_batch_destroy(batch)
+    for h, u, r in zip(hs, us, got):
+        plan = B.helm_plan_create(3, n, h, 2.0, prec=prec)
+        B.helm_plan_set_cycle(plan, 0, 2, 1)
+        v = torch.zeros_like(g)
+        st, it, hist = B.helm_solve(plan, f, g, v, 1e-9, 60)
+        B.helm_plan_destroy(plan)
+        assert (st, it) == r[:2] and np.array_equal(hist, r[2]) and torch.equal(u, v)
