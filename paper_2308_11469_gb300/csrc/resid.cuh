@@ -4,7 +4,7 @@
 #include <type_traits>
 
 #include "launch.h"
-#include "fp_bits.cuh"
+#include "float_sum.cuh"
 #include "fixed_lap.cuh"
 #include "fixed_win.cuh"
 
@@ -77,32 +77,12 @@ __device__ void finalize(const InstDesc& I, InstState* stp, double norm2, double
     *stp = s;
 }
 
-// float -> double, exact for every value, without the FP64 pipe unless it is subnormal
-__device__ __forceinline__ double widen_any(float f)
-{
-    const unsigned mag = __float_as_uint(f) & 0x7fffffffu;
-    return mag - 1u < 0x007fffffu ? (double)f : f2d_bits(f);
-}
-
-// Sum of n floats in order, kept as an unevaluated pair (error-free two-sums: exact to 2^-48 of
-// the sum) so that only the last addition is FP64: a warp's FP64 instruction holds its pipe for
-// 64 clocks, and a thread adding eight warps' values in FP64 kept the whole CTA waiting.
-__device__ __forceinline__ double sum_floats(const float* p, int n)
-{
-    float s = 0.f, c = 0.f;
-    for (int i = 0; i < n; ++i) {
-        const float v = p[i], t = s + v, bb = t - s;
-        c += (s - (t - bb)) + (v - bb);
-        s = t;
-    }
-    return isfinite(s) ? widen_any(s) + widen_any(c) : widen_any(s);
-}
-
 // Block-wide sums / maxima in a fixed order (xor-shuffle in T, then the warps' values in
 // order, in FP64).  `sum2`: the second channel is summed (mode 0, ||b||^2) instead of
 // maximised (max |e|^2, non-negative: FP64 maxima are taken on the bits).  Mode 1 reduces its
-// complex64-derived values in FP32, keeping the shuffle tree off the FP64 pipe; the result
-// (thread 0) is FP64 either way.  live: only the first `live` warps hold values.
+// complex64-derived values in FP32 within a warp, keeping the shuffle tree off the FP64 pipe, and
+// adds the warps' sums to FP64's accuracy (float_sum.cuh); the result (thread 0) is FP64 either
+// way.  live: only the first `live` warps hold values.
 template <typename T>
 __device__ __forceinline__ void block_reduce(T a, T m, double& ra, double& rm, double* sa, double* sm,
                                              bool sum2, int live = 32)
