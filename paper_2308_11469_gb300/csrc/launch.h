@@ -183,7 +183,8 @@ struct WsInit {
 };
 cudaError_t launch_init_workspaces(const WsInit* recs, int count, cudaStream_t s);
 // start and end of a plan's solve (one instance): descriptor, state, step control ctrl[0..3]
-// and wall rings from the host's d; state and histories (of up to cap steps) to page-locked
+// and wall rings from the host's d (kernels behind it in the stream read them after their
+// programmatic-launch wait); state and histories (of up to cap steps) to page-locked
 // host memory and the last iterate (count values) to the caller's buffer
 cudaError_t launch_begin(const InstDesc& d, InstDesc* dst, InstState* st, int* ctrl, cudaStream_t s);
 cudaError_t launch_finish(const InstDesc& d, const InstState* st, long count, InstState* h_st, double* h_hist, int cap,

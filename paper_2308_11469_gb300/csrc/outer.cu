@@ -233,7 +233,7 @@ k_upres2d(const InstDesc* __restrict__ insts, InstState* __restrict__ st,
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ double sa[NTH / 32], sm[NTH / 32];
     __shared__ int last;
-    // work item and descriptors are host-written: read them before the wait
+    // work item and descriptors before the wait (see pdl.cuh)
     const MgItem item = items[blockIdx.y];
     const InstDesc& I = insts[item.inst];
     const LevelDesc L = I.lev[0];

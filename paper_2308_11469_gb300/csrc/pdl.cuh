@@ -2,6 +2,13 @@
 // next one may be scheduled while it drains (stream capture turns this into programmatic
 // graph edges).  Each kernel waits for its predecessor's completion (and memory) before
 // its first read of data the predecessor produced, then lets its own successor launch.
+//
+// Only the wait makes a predecessor's writes visible.  The kernels of a step that read a work
+// item or a descriptor before it (k_down2d, k_up2d, k_upres2d, k_tail and others) may do so because
+// those are complete before the first of them can start: copies in the stream and graph launches
+// are ordered without overlap, and k_begin, which writes a plan's descriptor on the device, is
+// followed by the start residual and a graph launch.  A kernel launched behind k_begin outside
+// a graph (k_small2d) reads the descriptor after its wait.
 #pragma once
 #include <cuda_runtime.h>
 

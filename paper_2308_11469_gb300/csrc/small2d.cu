@@ -70,15 +70,15 @@ k_small2d(const InstDesc* __restrict__ insts, InstState* __restrict__ st, const 
     cg::cluster_group cl = cg::this_cluster();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int rank = (int)cl.block_rank();
-    const MgItem item = items[blockIdx.x / CS];
-    const InstDesc& I = insts[item.inst];
-    const LevelDesc L0 = I.lev[0];
-    const float sigma = I.sigf;
-    // host-written tables before the wait
+    // host-written tables before the wait; the descriptor of a plan's solve is not: k_begin wrote it
     if constexpr (tail_exact<2, float, N0>())
         for (int i = tid; i < XTAB_FLOATS; i += TNT) xscr[i] = xtab[i];
     pdl_wait();
     pdl_trigger();
+    const MgItem item = items[blockIdx.x / CS];
+    const InstDesc& I = insts[item.inst];
+    const LevelDesc L0 = I.lev[0];
+    const float sigma = I.sigf;
     if (tid == 0) {
         sst = st[item.inst];
         // steps this launch may make (written by the launch's last arrival only, which every

@@ -140,7 +140,7 @@ k_tail(const InstDesc* __restrict__ insts, const InstState* __restrict__ st,
     extern __shared__ __align__(16) unsigned char smem_raw[];
     c2* base = reinterpret_cast<c2*>(smem_raw);
     const MgItem item = items[blockIdx.x];
-    const LevelDesc L0 = insts[item.inst].lev[item.level];   // host-written: read before the wait
+    const LevelDesc L0 = insts[item.inst].lev[item.level];   // before the wait: see pdl.cuh
     const double sigma = insts[item.inst].sigma;
     pdl_wait();
     pdl_trigger();
@@ -490,7 +490,7 @@ k_ctail(const InstDesc* __restrict__ insts, const InstState* __restrict__ st,
     const int loEB = 16 * k + W::EB_OFF, loRB = 16 * k + W::RB_OFF;
     const int loEC = 8 * k + W::EC_OFF, loRC = 8 * k + W::RC_OFF;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    // before the wait (nothing here depends on the predecessor): descriptors, the sine
+    // before the wait (nothing here depends on the predecessor, see pdl.cuh): descriptors, the sine
     // tables, and the coarse iterate windows cleared (their rings and outer rows stay zero)
     const MgItem item = items[blockIdx.x / CT_CS];
     const LevelDesc LA = insts[item.inst].lev[item.level];

@@ -77,8 +77,8 @@ k_down2d(const InstDesc* __restrict__ insts, const InstState* __restrict__ st,
     constexpr int W = TX + 2 * H, HH = TY + 2 * H;
     typedef Planes<W> PL;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    // work item and level descriptors are written by the host before the launch: read them
-    // before waiting for the predecessor kernel (overlaps its drain)
+    // work item and level descriptors are older than the predecessor kernel (see pdl.cuh): read
+    // them before waiting for it (overlaps its drain)
     const MgItem item = items[blockIdx.y];
     const LevelDesc L = insts[item.inst].lev[item.level];
     const LevelDesc C = insts[item.inst].lev[item.level + 1];
@@ -293,8 +293,8 @@ k_up2d(const InstDesc* __restrict__ insts, const InstState* __restrict__ st,
     constexpr int CW = W / 2 + 2, CH = HH / 2 + 2;
     typedef Planes<W> PL;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    // work item and level descriptors are written by the host before the launch: read them
-    // before waiting for the predecessor kernel (overlaps its drain)
+    // work item and level descriptors are older than the predecessor kernel (see pdl.cuh): read
+    // them before waiting for it (overlaps its drain)
     const MgItem item = items[blockIdx.y];
     const LevelDesc L = insts[item.inst].lev[item.level];
     const LevelDesc C = insts[item.inst].lev[item.level + 1];
