@@ -333,7 +333,7 @@ struct Engine {
         if (D == 2) HELM_CK(setup_2d(prec == HELM_PREC_FP64 ? 0 : 1));
         if (D == 2 && prec != HELM_PREC_FP64) {
             ctail_setup();
-            HELM_CK(setup_small2d());
+            setup_small2d();
         }
         HELM_CK(setup_generic(D, prec == HELM_PREC_FP64 ? 0 : 1));
         HELM_CK(setup_outer());

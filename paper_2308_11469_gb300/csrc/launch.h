@@ -88,11 +88,34 @@ cudaError_t launch_ctail(const InstDesc* insts, const InstState* st, const MgIte
 // whole solves of small 2D complex64 grids (small2d.cu): every remaining outer step of the
 // items (level-0 items of instances of size n), up to the budget ctrl[1] - ctrl[0], in one
 // launch of a cluster of cs CTAs per item.  Adds the steps made to ctrl[0]; ctrl holds 5
-// ints, [3] and [4] zero between launches.  small2d_fits: the cluster size for ninst
-// instances of size n (0: no such kernel, or too many for it); mixed: solves of other sizes
-// run beside them.
+// ints, [3] and [4] zero between launches.  setup_small2d asks the device which forms (size and
+// cluster size) it can hold; small2d_fits: the cluster size for ninst instances of size n (0: no
+// such form, or too many instances for it); mixed: solves of other sizes run beside them.
+enum { SMALL_63_8 = 1, SMALL_63_4 = 2, SMALL_63_2 = 4, SMALL_31_4 = 8, SMALL_31_2 = 16 };
+// the choice among the forms `fits`:
+// A cluster of CS CTAs holds CS whole SMs until its solve ends: fewer CTAs a solve as more
+// solves share the GPU's 152 SMs.  One lane of 63^2 solves, V(0,1), launch by launch against
+// this: 1 solve 447 / 263 us, 8 1006 / 551, 24 2160 / 1384 (CS = 4), 64 2702 / 2027 (CS = 2);
+// above that the clusters queue and the gain fades (four lanes of 50: 4840 / 4423 us).
+// Beside solves of other sizes, more than 32 of them would hold SMs that the larger solves
+// need (512 uneven cavities: 0.3 % slower).  A form that does not fit gives way to the next
+// smaller cluster.
+inline int small2d_pick(int n, int ninst, bool mixed, int fits)
+{
+    if (ninst > (mixed ? 32 : 96)) return 0;
+    if (n == 63) {
+        if (ninst <= 12 && (fits & SMALL_63_8)) return 8;
+        if (ninst <= 32 && (fits & SMALL_63_4)) return 4;
+        return (fits & SMALL_63_2) ? 2 : 0;
+    }
+    if (n == 31) {
+        if (ninst <= 32 && (fits & SMALL_31_4)) return 4;
+        return (fits & SMALL_31_2) ? 2 : 0;
+    }
+    return 0;
+}
 int small2d_fits(int n, int ninst, bool mixed);
-cudaError_t setup_small2d();
+void setup_small2d();
 cudaError_t launch_small2d(const InstDesc* insts, InstState* st, const MgItem* items, int nitems, int n, int cs,
                            int nu1, int nu2, int cycles, int damp, int* ctrl, cudaStream_t s);
 // shared-memory carve-out preferences of the generic and outer kernels

@@ -300,16 +300,22 @@ k_small2d(const InstDesc* __restrict__ insts, InstState* __restrict__ st, const 
     }
 }
 
-template <int N0, int CS>
-cudaError_t small_attrs()
+// can a cluster of this form be resident? (its attributes set, and the driver's own answer)
+template <int N0, int CS, bool DAMP>
+bool small_resident()
 {
     const int b = (int)SmallLay<N0, CS>::BYTES;
-    cudaError_t e = cudaFuncSetAttribute(k_small2d<N0, CS, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_small2d<N0, CS, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-    if (e == cudaSuccess) e = max_carveout(k_small2d<N0, CS, false>);
-    return e == cudaSuccess ? max_carveout(k_small2d<N0, CS, true>) : e;
+    if (cudaFuncSetAttribute(k_small2d<N0, CS, DAMP>, cudaFuncAttributeMaxDynamicSharedMemorySize, b) != cudaSuccess ||
+        max_carveout(k_small2d<N0, CS, DAMP>) != cudaSuccess)
+        return false;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(CS);
+    cfg.blockDim = dim3(TNT);
+    cfg.dynamicSmemBytes = b;
+    int clusters = 0;
+    return cudaOccupancyMaxActiveClusters(&clusters, k_small2d<N0, CS, DAMP>, &cfg) == cudaSuccess && clusters > 0;
 }
+template <int N0, int CS> bool small_ok() { return small_resident<N0, CS, false>() && small_resident<N0, CS, true>(); }
 
 template <int N0, int CS>
 cudaError_t small_launch(const InstDesc* insts, InstState* st, const MgItem* items, int nitems, int nu1, int nu2,
@@ -327,37 +333,35 @@ cudaError_t small_launch(const InstDesc* insts, InstState* st, const MgItem* ite
 
 }  // namespace
 
-cudaError_t setup_small2d()
+namespace {
+// per device: the forms that fit it (bits of small2d_pick) with SMALL_KNOWN; 0: not asked yet
+constexpr int SMALL_KNOWN = 1 << 8;
+std::atomic<int> g_small[64];
+}  // namespace
+
+void setup_small2d()
 {
     // once per device (the attributes are the kernels', not a plan's)
-    static std::atomic<unsigned long long> done{0};
     int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    const unsigned long long bit = 1ull << (dev & 63);
-    if (dev < 64 && (done.load() & bit)) return cudaSuccess;
-    if ((e = small_attrs<63, 8>()) != cudaSuccess) return e;
-    if ((e = small_attrs<63, 4>()) != cudaSuccess) return e;
-    if ((e = small_attrs<63, 2>()) != cudaSuccess) return e;
-    if ((e = small_attrs<31, 4>()) != cudaSuccess) return e;
-    if ((e = small_attrs<31, 2>()) != cudaSuccess) return e;
-    if (dev < 64) done |= bit;
-    return cudaSuccess;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev >= 64 || g_small[dev].load()) {
+        cudaGetLastError();
+        return;
+    }
+    const int fits = (small_ok<63, 8>() ? SMALL_63_8 : 0) | (small_ok<63, 4>() ? SMALL_63_4 : 0) |
+                     (small_ok<63, 2>() ? SMALL_63_2 : 0) | (small_ok<31, 4>() ? SMALL_31_4 : 0) |
+                     (small_ok<31, 2>() ? SMALL_31_2 : 0);
+    cudaGetLastError();
+    g_small[dev] = fits | SMALL_KNOWN;
 }
 
 int small2d_fits(int n, int ninst, bool mixed)
 {
-    // A cluster of CS CTAs holds CS whole SMs until its solve ends: fewer CTAs a solve as more
-    // solves share the GPU's 152 SMs.  One lane of 63^2 solves, V(0,1), launch by launch against
-    // this: 1 solve 447 / 263 us, 8 1006 / 551, 24 2160 / 1384 (CS = 4), 64 2702 / 2027 (CS = 2);
-    // above that the clusters queue and the gain fades (four lanes of 50: 4840 / 4423 us).
-    // Beside solves of other sizes, more than 32 of them would hold SMs that the larger solves
-    // need (512 uneven cavities: 0.3 % slower).
-    const int most = mixed ? 32 : 96;
-    if (ninst > most) return 0;
-    if (n == 63) return ninst <= 12 ? 8 : ninst <= 32 ? 4 : 2;
-    if (n == 31) return ninst <= 32 ? 4 : 2;
-    return 0;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev >= 64) {
+        cudaGetLastError();
+        return 0;
+    }
+    return small2d_pick(n, ninst, mixed, g_small[dev].load());
 }
 
 cudaError_t launch_small2d(const InstDesc* insts, InstState* st, const MgItem* items, int nitems, int n, int cs,
