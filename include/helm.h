@@ -399,8 +399,10 @@ HELM_API helm_status helm_batch_poll(helm_batch* batch, uint64_t ticket, int* do
  * with the Helmholtz residual + update + norm (2D complex64 batches of one size), 10 the
  * cluster tail (levels 255 ... 31 of 2D complex64 cycles in one 8-CTA cluster per solve),
  * 11 two descent steps (rhs restrictions) in one launch, 12 kind 9 with level 1's ascent
- * formed inside it too): launches[k], device milliseconds ms[k] and algorithmic bytes
- * bytes[k] (each datum a launch must read or write, counted once).  nkinds >= 13.
+ * formed inside it too, 13 all the steps of solves of n = 31 or 63 in one launch of a cluster
+ * each; with nkinds = 13 their steps are made launch by launch): launches[k], device
+ * milliseconds ms[k] and algorithmic bytes bytes[k] (each datum a launch must read or write,
+ * counted once).  nkinds >= 13.
  */
 HELM_API helm_status helm_batch_profile(helm_batch* batch, int max_steps, uint64_t* launches,
                                         double* ms, double* bytes, int nkinds);

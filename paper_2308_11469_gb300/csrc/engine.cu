@@ -157,8 +157,9 @@ struct Instance {
 
 struct LaunchRec {
     // UPRES1 names, in helm_batch_profile only, an UPRES launch that also forms level 1's
-    // ascent (color 1); steps hold it as UPRES
-    enum Kind { RBGS, RESTRICT, PROLONG, ZERO, TAIL, RESID, CHECK, DOWN, UP, UPRES, CTAIL, DOWN2, UPRES1, NKINDS } kind;
+    // ascent (color 1; steps hold it as UPRES), and SMALL the one launch of an engine of small
+    // solves (its steps hold the launches that it replaces)
+    enum Kind { RBGS, RESTRICT, PROLONG, ZERO, TAIL, RESID, CHECK, DOWN, UP, UPRES, CTAIL, DOWN2, UPRES1, SMALL, NKINDS } kind;
     int off, cnt, work, color, mode;
     double bytes;   // algorithmic bytes of one launch (each datum it must touch, once)
     int nmax = 0;   // DOWN: the largest level of the launch; UPRES: the level-0 size
@@ -747,6 +748,15 @@ struct Engine {
         HELM_CK(launch_small2d(d_desc, d_state, d_mg + l0_off, l0_cnt, n, small_cs, nu1, nu2, cycles, damp_any,
                                d_ctrl, s));
         return HELM_OK;
+    }
+    // algorithmic bytes of such a launch: u_N, f and r_N in, the last iterate and residual out
+    double small_bytes(const InstState* st) const
+    {
+        double b = 0.0;
+        for (int i = 0; i < cap; ++i)
+            if (slots[i] && st[i].status == HELM_ST_ACTIVE)
+                b += (double)slots[i]->d.n * slots[i]->d.n * (3.0 * 16.0 + 2.0 * elem_bytes(prec));
+        return b;
     }
     // kernels launched by a run that made `steps` steps
     uint64_t step_launches(int steps) const { return small_cs ? (steps > 0) : (uint64_t)steps * step.size(); }
@@ -2169,8 +2179,8 @@ helm_status helm_batch_step(helm_batch* b, int max_steps)
 helm_status helm_batch_profile(helm_batch* b, int max_steps, uint64_t* launches, double* ms,
                                double* bytes, int nkinds)
 {
-    if (!b || max_steps < 0 || !launches || !ms || !bytes || nkinds < (int)LaunchRec::NKINDS)
-        return HELM_EINVAL;
+    if (!b || max_steps < 0 || !launches || !ms || !bytes || nkinds < (int)LaunchRec::SMALL) return HELM_EINVAL;
+    const bool small_kind = nkinds > (int)LaunchRec::SMALL;      // (callers of 13 kinds have no place for it)
     for (int k = 0; k < nkinds; ++k) {
         launches[k] = 0;
         ms[k] = 0.0;
@@ -2186,11 +2196,12 @@ helm_status helm_batch_profile(helm_batch* b, int max_steps, uint64_t* launches,
         if (st != HELM_OK) return st;
         st = E->prepare_plan();
         if (st != HELM_OK) return st;
-        const size_t nl = E->step.size();
+        const bool small = E->small_cs && small_kind;             // all its steps in one launch
+        const size_t nl = small ? 1 : E->step.size();
         std::vector<cudaEvent_t> ev(2 * nl);
         for (auto& x : ev) HELM_CK(cudaEventCreate(&x));
         E->h_ctrl[0] = 0;
-        E->h_ctrl[1] = INT_MAX;
+        E->h_ctrl[1] = small && max_steps > 0 ? max_steps : INT_MAX;
         E->h_ctrl[2] = 1;
         E->h_ctrl[3] = 0;
         HELM_CK(cudaMemcpyAsync(E->d_ctrl, E->h_ctrl, 4 * sizeof(int), cudaMemcpyHostToDevice, b->stream));
@@ -2199,11 +2210,15 @@ helm_status helm_batch_profile(helm_batch* b, int max_steps, uint64_t* launches,
         HELM_CK(cudaStreamSynchronize(b->stream));
         for (int s = 0; (max_steps == 0 || s < max_steps) && s < 1000000; ++s) {
             std::vector<double> lb(nl);
-            for (size_t i = 0; i < nl; ++i) lb[i] = E->launch_bytes(E->step[i], E->h_state);
+            for (size_t i = 0; i < nl; ++i) lb[i] = small ? E->small_bytes(E->h_state) : E->launch_bytes(E->step[i], E->h_state);
             for (size_t i = 0; i < nl; ++i) {
                 HELM_CK(cudaEventRecord(ev[2 * i], b->stream));
-                std::vector<LaunchRec> one{E->step[i]};
-                st = E->enqueue(one, b->stream, false);
+                if (small) {
+                    st = E->enqueue_step(b->stream);
+                } else {
+                    std::vector<LaunchRec> one{E->step[i]};
+                    st = E->enqueue(one, b->stream, false);
+                }
                 if (st != HELM_OK) return st;
                 HELM_CK(cudaEventRecord(ev[2 * i + 1], b->stream));
             }
@@ -2214,7 +2229,7 @@ helm_status helm_batch_profile(helm_batch* b, int max_steps, uint64_t* launches,
             for (size_t i = 0; i < nl; ++i) {
                 float t = 0.f;
                 HELM_CK(cudaEventElapsedTime(&t, ev[2 * i], ev[2 * i + 1]));
-                int k = (int)E->step[i].kind;
+                int k = small ? (int)LaunchRec::SMALL : (int)E->step[i].kind;
                 if (k == LaunchRec::UPRES && E->step[i].color) k = LaunchRec::UPRES1;
                 launches[k] += 1;
                 ms[k] += t;
