@@ -84,7 +84,7 @@ __host__ __device__ __forceinline__ long long fx_fix(double v, int emax)
     return ((long long)a ^ sg) - sg;
 }
 
-// L * 2^(emax - 1080) rounded to the nearest binary64, ties to even.  Needs |L| < 2^62
+// L * 2^(emax - 1080) rounded to the nearest binary64, ties to even.  Needs |L| < 2^63
 // and FX_EMIN <= emax <= FX_EMAX (the result is then normal and finite, or zero).
 __host__ __device__ __forceinline__ double fx_to_double(long long L, int emax)
 {
