@@ -42,7 +42,6 @@ constexpr int AN_NT = 256;
 constexpr int AN_NC = 8;            // coarsest level (solved exactly)
 constexpr int AN_BAND = 4;          // band half-width around the hole, in nodes of the level
 constexpr int AN_BAND_SWEEPS = 4;
-constexpr bool AN_GRAPHS = true;     // the outer steps as one graph launch
 constexpr size_t AN_SMEM_MAX = 227 * 1024;
 enum : unsigned char { AN_PDE = 0, AN_EDGE = 1, AN_HOLE = 2 };
 
@@ -1720,7 +1719,7 @@ helm_status an_solve(helm_annulus* a, const double2* data, double2* u, double to
     cudaStream_t s = a->stream;
     a->ls = s;
     const long total = (long)(a->N + 1) * (a->N + 1);
-    if (AN_GRAPHS && !a->loop && max_outer > 0) an_build_loop<R>(a);
+    if (!a->loop && max_outer > 0) an_build_loop<R>(a);
     AnCtl c{};
     c.U[0] = u;
     c.U[1] = a->U1;

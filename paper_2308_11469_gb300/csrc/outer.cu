@@ -178,8 +178,8 @@ k_residual2d(const InstDesc* __restrict__ insts, InstState* __restrict__ st,
 // two-launch path bit for bit.  Level 0 keeps r_N and
 // r_{N+1} in separate buffers (step parity), so tiles still sweeping with r_N never see
 // another tile's r_{N+1}.
-// The tile is one residual tile of k_residual2d; NTU threads (128 or 256) each stand for
-// 256 / NTU threads of that kernel's map, so partials are formed in its order.
+// The tile is one residual tile of k_residual2d and each thread one of that kernel's map, so
+// partials are formed in its order.
 constexpr int UPY = T2Y;
 
 // The coarse window: fine nodes gx0 .. gx0 + W - 1 (gx0 = x0 - H even when H is odd) read
@@ -212,8 +212,8 @@ template <int NU, int UX, bool L1F = false> constexpr size_t upres_bytes()
     return ub + 2 * planes + cs;
 }
 
-template <int NU, bool DAMP, int NTU, bool L1F>
-__global__ void __launch_bounds__(NTU, NTU == 128 ? 7 : (UPRES_LATE_U ? 6 : 5))
+template <int NU, bool DAMP, bool L1F>
+__global__ void __launch_bounds__(NTH, UPRES_LATE_U ? 6 : 5)
 k_upres2d(const InstDesc* __restrict__ insts, InstState* __restrict__ st,
           const MgItem* __restrict__ items, int e2_mode, StepCtl ctl)
 {
@@ -221,15 +221,13 @@ k_upres2d(const InstDesc* __restrict__ insts, InstState* __restrict__ st,
     typedef float2 c2;
     constexpr int UX = T2;
     constexpr int TX = UX, TY = UPY;
-    constexpr int NWU = NTU / 32;
-    constexpr int VT = NTH / NTU;                // threads of the residual kernel's map per thread
     constexpr int H = 2 * NU + 1;
     constexpr int W = TX + 2 * H, HH = TY + 2 * H;
     constexpr int CW = upres_cw<NU, UX>(), CH = upres_ch<NU>();
     constexpr int UW = TX + 2, UH = TY + 2;
     static_assert(H % 2 == 1 && TX % 2 == 0 && TY % 2 == 0, "gx0, gy0 even");
     typedef Planes<W> PL;
-    static_assert(TY == T2Y && NTH == NTU, "one residual tile, a thread of its map per thread");
+    static_assert(TY == T2Y, "one residual tile, a thread of its map per thread");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ double sa[NTH / 32], sm[NTH / 32];
     __shared__ int last;
@@ -279,7 +277,7 @@ k_upres2d(const InstDesc* __restrict__ insts, InstState* __restrict__ st,
     // stage u_N on the tile plus a 1-node ring (now, or after the sweeps), the coarse
     // window, e2 and r_N
     auto stage_u = [&]() {
-        for (int q = threadIdx.x; q < UW * UH; q += NTU) {
+        for (int q = threadIdx.x; q < UW * UH; q += NTH) {
             const int gx = x0 - 1 + q % UW, gy = y0 - 1 + q / UW;
             const bool in = gx <= n + 1 && gy <= n + 1;
             cp_async_elem<16>(U + q, uin + (in ? (size_t)gy * S + gx : 0), in);
@@ -302,12 +300,12 @@ k_upres2d(const InstDesc* __restrict__ insts, InstState* __restrict__ st,
         const c2* __restrict__ g2e = (const c2*)C2l.e;
         const c2* __restrict__ g1r = (const c2*)C.rhs;
         const int n1 = C.n, n2 = C2l.n, P2 = C2l.pitch;
-        for (int q = threadIdx.x; q < W2X * W2Y; q += NTU) {
+        for (int q = threadIdx.x; q < W2X * W2Y; q += NTH) {
             const int X = c2x0 + q % W2X, Y = c2y0 + q / W2X;
             const bool in = X >= 0 && X <= n2 + 1 && Y >= 0 && Y <= n2 + 1;
             cp_async_elem<sizeof(c2)>(C2w + q, g2e + (in ? (size_t)Y * P2 + X : 0), in);
         }
-        for (int q = threadIdx.x; q < W1X * W1Y; q += NTU) {
+        for (int q = threadIdx.x; q < W1X * W1Y; q += NTH) {
             const int X = c1x0 + q % W1X, Y = c1y0 + q / W1X;
             const bool in = X >= 1 && X <= n1 && Y >= 1 && Y <= n1;
             cp_async_elem<sizeof(c2)>(R1w + q, g1r + (in ? (size_t)Y * PC + X : 0), in);
@@ -317,7 +315,7 @@ k_upres2d(const InstDesc* __restrict__ insts, InstState* __restrict__ st,
         // level 0's window is still arriving
         asm volatile("cp.async.commit_group;\n" ::: "memory");
     } else {
-        for (int q = threadIdx.x; q < CW * CH; q += NTU) {
+        for (int q = threadIdx.x; q < CW * CH; q += NTH) {
             const int cy = q / CW, cx = q - cy * CW;
             const int X = cx0 + cx, Y = cy0 + cy;
             const bool in = X <= nc1 && Y <= nc1;
@@ -326,7 +324,7 @@ k_upres2d(const InstDesc* __restrict__ insts, InstState* __restrict__ st,
     }
     // the window's W x HH nodes numbered row by row over the threads (rows of a few dozen
     // nodes: a warp per row would leave lanes idle)
-    for (int q = threadIdx.x; q < W * HH; q += NTU) {
+    for (int q = threadIdx.x; q < W * HH; q += NTH) {
         const int ly = q / W, lx = q - ly * W;
         const int gy = gy0 + ly;
         const bool yin = gy >= 1 && gy <= n;
@@ -357,7 +355,7 @@ k_upres2d(const InstDesc* __restrict__ insts, InstState* __restrict__ st,
         // without reading it), then nu2 sweeps, each half-sweep one node closer to the coarse
         // window, whose values end final
         const int n1 = C.n;
-        for (int q = threadIdx.x; q < W1X * W1Y; q += NTU) {
+        for (int q = threadIdx.x; q < W1X * W1Y; q += NTH) {
             const int i = q % W1X, j = q / W1X;
             const int X = c1x0 + i, Y = c1y0 + j;
             if (X < 1 || X > n1 || Y < 1 || Y > n1) continue;
@@ -379,7 +377,7 @@ k_upres2d(const InstDesc* __restrict__ insts, InstState* __restrict__ st,
             const int color = (sw - 1) & 1, ring1 = 2 * NU - sw;
             const int xa = max(cx0 - ring1, 1), xb = min(cx0 + CW - 1 + ring1, n1);
             const int ya = max(cy0 - ring1, 1), yb = min(cy0 + CH - 1 + ring1, n1);
-            for (int Y = ya + (int)(threadIdx.x >> 5); Y <= yb; Y += NWU) {
+            for (int Y = ya + (int)(threadIdx.x >> 5); Y <= yb; Y += NTH / 32) {
                 const int xs = xa + (((xa + Y) & 1) ^ color);
                 const int j = Y - c1y0;
                 for (int X = xs + 2 * lane; X <= xb; X += 64) {
@@ -406,7 +404,7 @@ k_upres2d(const InstDesc* __restrict__ insts, InstState* __restrict__ st,
     // the outermost ring's colour-0 nodes it leaves are never read)
     // nodes numbered row by row over the threads: all W of a row, or its W / 2 colour-1 nodes
     constexpr int CNX = (NU == 0) ? W : W / 2;
-    for (int q = threadIdx.x; q < CNX * HH; q += NTU) {
+    for (int q = threadIdx.x; q < CNX * HH; q += NTH) {
         const int ly = q / CNX, i = q - ly * CNX;
         const int gy = gy0 + ly;
         if (gy < 1 || gy > n) continue;
@@ -426,7 +424,7 @@ k_upres2d(const InstDesc* __restrict__ insts, InstState* __restrict__ st,
     __syncthreads();
     const R h2 = LevC<R>::h2(L);
     const R dinv = LevC<R>::dinv(L);
-    sweeps_flat<R, W, TX, TY, NTU, 2 * NU, 2 * NU>(E0, E1, R0, R1, gx0, gy0, x0, y0, n, h2, dinv);
+    sweeps_flat<R, W, TX, TY, NTH, 2 * NU, 2 * NU>(E0, E1, R0, R1, gx0, gy0, x0, y0, n, h2, dinv);
     if (UPRES_LATE_U) {                          // the rhs planes and Cs are dead: u_N there
         stage_u();
         cp_async_wait_all();
@@ -435,9 +433,9 @@ k_upres2d(const InstDesc* __restrict__ insts, InstState* __restrict__ st,
     // u_{N+1} = u_N + e_N on the window (as k_residual2d forms it): the residual nodes of
     // each map thread in registers, the ring by the first threads; the window's largest
     // exponent sets the scale of the exact fixed-point Laplacian numerators
-    constexpr int KY = TY / 8, RING = 2 * (TX + 2) + 2 * TY, RJ = (RING + NTU - 1) / NTU;
-    __shared__ int sx[NWU];
-    double2 cv[VT][KY];
+    constexpr int KY = TY / 8, RING = 2 * (TX + 2) + 2 * TY, RJ = (RING + NTH - 1) / NTH;
+    __shared__ int sx[NTH / 32];
+    double2 cv[KY];
     int exq = 0;
     // window node (lxw, lyw): u_N (+ e_N inside the grid; |e_N|^2 into *em for own nodes)
     auto upd = [&](int lxw, int lyw, R* em) -> double2 {
@@ -452,78 +450,65 @@ k_upres2d(const InstDesc* __restrict__ insts, InstState* __restrict__ st,
         }
         return v;
     };
-    R r2[VT], em[VT];
+    R r2 = 0, em = 0;
+    const int t = threadIdx.x;
 #pragma unroll
-    for (int v = 0; v < VT; ++v) {
-        const int t = threadIdx.x + NTU * v;
-        em[v] = 0;
-#pragma unroll
-        for (int k = 0; k < KY; ++k) {
-            cv[v][k] = upd((t & 31) + 1, (t >> 5) + 8 * k + 1, &em[v]);
-            exq = max(exq, fx_exp2(cv[v][k]));
-        }
+    for (int k = 0; k < KY; ++k) {
+        cv[k] = upd((t & 31) + 1, (t >> 5) + 8 * k + 1, &em);
+        exq = max(exq, fx_exp2(cv[k]));
     }
     double2 rv[RJ];
     int rq[RJ];
 #pragma unroll
     for (int j = 0; j < RJ; ++j) {
-        const int t = threadIdx.x + NTU * j;
+        const int q = t + NTH * j;
         rq[j] = -1;
         rv[j] = make_double2(0.0, 0.0);
-        if (t < RING) {
+        if (q < RING) {
             int rlx, rly;
-            ring_node<TX, TY>(t, rlx, rly);
+            ring_node<TX, TY>(q, rlx, rly);
             rv[j] = upd(rlx, rly, nullptr);
             rq[j] = rly * UW + rlx;
             exq = max(exq, fx_exp2(rv[j]));
         }
     }
     // its barrier also ends the reads of U; uniform over the CTA
-    const int emx = fx_scale(block_max_exp<NTU>(exq, sx));
+    const int emx = fx_scale(block_max_exp<NTH>(exq, sx));
     longlong2* UF = reinterpret_cast<longlong2*>(U);
 #pragma unroll
-    for (int v = 0; v < VT; ++v) {
-        const int t = threadIdx.x + NTU * v;
-#pragma unroll
-        for (int k = 0; k < KY; ++k) UF[((t >> 5) + 8 * k + 1) * UW + (t & 31) + 1] = fx_fix2(cv[v][k], emx);
-    }
+    for (int k = 0; k < KY; ++k) UF[((t >> 5) + 8 * k + 1) * UW + (t & 31) + 1] = fx_fix2(cv[k], emx);
 #pragma unroll
     for (int j = 0; j < RJ; ++j)
         if (rq[j] >= 0) UF[rq[j]] = fx_fix2(rv[j], emx);
     __syncthreads();
     // r_{N+1}: thread t of the residual kernel's map takes the nodes (t mod 32, t / 32 + 8 k)
-    // of the tile; real thread j stands for the map's threads j + NTU v, v < VT
+    // of the tile
     double2* __restrict__ uout = I.u[(sv.it + 1) & 1];
     c2* __restrict__ rhs = (c2*)lev_rhs(L, 0, sv.it + 1);
     const double2* __restrict__ f = I.f;
     const double mih2 = -I.ih2, mk2 = -I.k2;
     const double damp = I.damp;
+    const int lx = (t & 31) + 1;
 #pragma unroll
-    for (int v = 0; v < VT; ++v) {
-        const int t = threadIdx.x + NTU * v;
-        const int lx = (t & 31) + 1;
-        r2[v] = 0;
-#pragma unroll
-        for (int k = 0; k < TY / 8; ++k) {
-            const int ly = (t >> 5) + 8 * k + 1;
-            const int gx = x0 + lx - 1, gy = y0 + ly - 1;
-            if (gx > n || gy > n) continue;
-            const int o = ly * UW + lx;
-            const double2 c = cv[v][k];
-            uout[(size_t)gy * S + gx] = c;
-            const double2 fv = f[(size_t)(gy - 1) * n + (gx - 1)];
-            const double2 r = (emx >= 0)
-                ? helm_resid2d_fx<DAMP>(c, UF[o], UF[o - 1], UF[o + 1], UF[o - UW], UF[o + UW], fv, mih2, mk2,
-                                        damp, emx)
-                : make_double2(fx_nan(), fx_nan());
-            const c2 ri = Inner<R>::from(r);
-            rhs[(size_t)gy * P + gx] = ri;
-            r2[v] += abs2(ri);
-        }
+    for (int k = 0; k < TY / 8; ++k) {
+        const int ly = (t >> 5) + 8 * k + 1;
+        const int gx = x0 + lx - 1, gy = y0 + ly - 1;
+        if (gx > n || gy > n) continue;
+        const int o = ly * UW + lx;
+        const double2 c = cv[k];
+        uout[(size_t)gy * S + gx] = c;
+        const double2 fv = f[(size_t)(gy - 1) * n + (gx - 1)];
+        const double2 r = (emx >= 0)
+            ? helm_resid2d_fx<DAMP>(c, UF[o], UF[o - 1], UF[o + 1], UF[o - UW], UF[o + UW], fv, mih2, mk2,
+                                    damp, emx)
+            : make_double2(fx_nan(), fx_nan());
+        const c2 ri = Inner<R>::from(r);
+        rhs[(size_t)gy * P + gx] = ri;
+        r2 += abs2(ri);
     }
     // the tile's partials in k_residual2d's order, then the instance's ticket
     double ra = 0.0, rm = 0.0;
-    block_reduce<R>(r2[0], em[0], ra, rm, sa, sm, false);
+    block_reduce<R>(r2, em, ra, rm, sa, sm, false);
     const int nb = I.nres_blocks;
     if (threadIdx.x == 0) {
         const int tile = by * I.res_tx + bx;
@@ -1411,10 +1396,6 @@ cudaError_t launch_residual(int D, int prec, const InstDesc* insts, InstState* s
 // tile width of the fused kernel: 32 (256-thread CTAs, four resident per SM, so CTAs in
 // their smoothing phase and CTAs in their FP64 residual phase share each SM)
 constexpr int UPX = 32;
-// threads of the fused kernel (128 or 256; same results).  128 lets 7 CTAs share an SM, so
-// a 1023^2 instance's 1024 tiles run in one wave, but measured slower (83.8 against
-// 80.1 us per outer step): the CTAs' latency-bound phases want the 8 warps.
-constexpr int UPRES_NT = 256;
 
 int upres2d_tiles(int n) { return ((n + UPX - 1) / UPX) * ((n + UPY - 1) / UPY); }
 
@@ -1425,17 +1406,17 @@ cudaError_t launch_upres2d(const InstDesc* insts, InstState* st, const MgItem* i
     if (nitems <= 0) return cudaSuccess;
     const StepCtl c{ctrl, nscan, ninst, use_cond, cond_handle};
     const dim3 g(upres2d_tiles(n), nitems);
-    const dim3 b(UPRES_NT);
+    const dim3 b(NTH);
 #define HELM_UR(NU)                                                                                 \
     case NU:                                                                                        \
         if (l1f) {                                                                                  \
-            if (damp) launch_k(k_upres2d<NU, true, UPRES_NT, true>, g, b, upres_bytes<NU, UPX, true>(), s, \
+            if (damp) launch_k(k_upres2d<NU, true, true>, g, b, upres_bytes<NU, UPX, true>(), s, \
                                insts, st, items, e2_mode, c);                                       \
-            else launch_k(k_upres2d<NU, false, UPRES_NT, true>, g, b, upres_bytes<NU, UPX, true>(), s,    \
+            else launch_k(k_upres2d<NU, false, true>, g, b, upres_bytes<NU, UPX, true>(), s,    \
                           insts, st, items, e2_mode, c);                                            \
-        } else if (damp) launch_k(k_upres2d<NU, true, UPRES_NT, false>, g, b, upres_bytes<NU, UPX>(), s, \
+        } else if (damp) launch_k(k_upres2d<NU, true, false>, g, b, upres_bytes<NU, UPX>(), s, \
                                   insts, st, items, e2_mode, c);                                    \
-        else launch_k(k_upres2d<NU, false, UPRES_NT, false>, g, b, upres_bytes<NU, UPX>(), s, insts, st, \
+        else launch_k(k_upres2d<NU, false, false>, g, b, upres_bytes<NU, UPX>(), s, insts, st, \
                       items, e2_mode, c);                                                           \
         break;
     switch (nu2) {
@@ -1450,12 +1431,12 @@ template <int NU, bool L1F>
 cudaError_t setup_upres_v()
 {
     cudaError_t e;
-    if ((e = cudaFuncSetAttribute(k_upres2d<NU, false, UPRES_NT, L1F>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    if ((e = cudaFuncSetAttribute(k_upres2d<NU, false, L1F>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)upres_bytes<NU, UPX, L1F>())) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_upres2d<NU, true, UPRES_NT, L1F>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    if ((e = cudaFuncSetAttribute(k_upres2d<NU, true, L1F>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)upres_bytes<NU, UPX, L1F>())) != cudaSuccess) return e;
-    if ((e = max_carveout(k_upres2d<NU, false, UPRES_NT, L1F>)) != cudaSuccess) return e;
-    return max_carveout(k_upres2d<NU, true, UPRES_NT, L1F>);
+    if ((e = max_carveout(k_upres2d<NU, false, L1F>)) != cudaSuccess) return e;
+    return max_carveout(k_upres2d<NU, true, L1F>);
 }
 
 template <int NU>

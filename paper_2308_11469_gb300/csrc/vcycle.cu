@@ -106,23 +106,23 @@ k_rbgs(const InstDesc* __restrict__ insts, const InstState* __restrict__ st,
 // updated colour finds its y- and z-neighbours at the same index j (x = 2j + p... / 2j) and its
 // x-neighbours at j, j+1 (odd x) or j-1, j (even x).  No shared-memory word is written by the
 // sweep; results go straight to global memory.
-template <typename R> struct Rb3p {
+struct Rb3p {
     static constexpr int TY = 8;                           // rows per CTA (a warp per row)
     static constexpr int L = 1;                            // planes in flight
     static constexpr int OS = L + 3, RS = L + 1;           // ring slots
     static constexpr int MAX_HP = 264;                     // pitch / 2 of n = 511
     static size_t bytes(int hp) {
-        return (size_t)(OS * (TY + 2) + RS * TY) * hp * sizeof(typename C2<R>::T);
+        return (size_t)(OS * (TY + 2) + RS * TY) * hp * sizeof(float2);
     }
 };
 
-template <typename R>
-__global__ void __launch_bounds__(32 * Rb3p<R>::TY)
+__global__ void __launch_bounds__(32 * Rb3p::TY)
 k_rbgs3p(const InstDesc* __restrict__ insts, const InstState* __restrict__ st,
          const MgItem* __restrict__ items, int color, int zchunk)
 {
-    typedef typename C2<R>::T c2;
-    typedef Rb3p<R> K;
+    typedef float R;
+    typedef float2 c2;
+    typedef Rb3p K;
     constexpr int TY = K::TY, L = K::L;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const MgItem item = items[blockIdx.y];
@@ -324,23 +324,23 @@ k_restrict(const InstDesc* __restrict__ insts, const InstState* __restrict__ st,
 // the fine planes 2 Z - 1 .. 2 Z + 1 are staged whole (16-byte cp.async) in a ring of five
 // fine planes (three in use, the next coarse plane's two in flight); the weights and the
 // order of the 27-term sums are k_restrict's.
-template <typename R> struct Rs3p {
+struct Rs3p {
     static constexpr int TYC = 4;                          // coarse rows per CTA
     static constexpr int NT = 256;                         // two warps per coarse row
     static constexpr int NS = 5;                           // fine-plane slots
     static constexpr int MAX_P = 528;                      // pitch of n = 511
     static size_t bytes(int pitch) {
-        return (size_t)NS * (2 * TYC + 1) * pitch * sizeof(typename C2<R>::T);
+        return (size_t)NS * (2 * TYC + 1) * pitch * sizeof(float2);
     }
 };
 
-template <typename R>
-__global__ void __launch_bounds__(Rs3p<R>::NT)
+__global__ void __launch_bounds__(Rs3p::NT)
 k_restrict3p(const InstDesc* __restrict__ insts, const InstState* __restrict__ st,
              const MgItem* __restrict__ items, int zchunk)
 {
-    typedef typename C2<R>::T c2;
-    typedef Rs3p<R> K;
+    typedef float R;
+    typedef float2 c2;
+    typedef Rs3p K;
     constexpr int TYC = K::TYC, FR = 2 * TYC + 1;         // fine rows per plane slot
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const MgItem item = items[blockIdx.y];
@@ -543,13 +543,13 @@ static cudaError_t carve()
 {
     cudaError_t e;
     if constexpr (D == 3 && sizeof(R) == 4) {              // the z-marching forms are complex64 only
-        if ((e = max_carveout(k_restrict3p<R>)) != cudaSuccess) return e;
-        if ((e = cudaFuncSetAttribute(k_restrict3p<R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)Rs3p<R>::bytes(Rs3p<float>::MAX_P))) != cudaSuccess)
+        if ((e = max_carveout(k_restrict3p)) != cudaSuccess) return e;
+        if ((e = cudaFuncSetAttribute(k_restrict3p, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)Rs3p::bytes(Rs3p::MAX_P))) != cudaSuccess)
             return e;
-        if ((e = max_carveout(k_rbgs3p<R>)) != cudaSuccess) return e;
-        if ((e = cudaFuncSetAttribute(k_rbgs3p<R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)Rb3p<R>::bytes(Rb3p<float>::MAX_HP))) != cudaSuccess)
+        if ((e = max_carveout(k_rbgs3p)) != cudaSuccess) return e;
+        if ((e = cudaFuncSetAttribute(k_rbgs3p, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)Rb3p::bytes(Rb3p::MAX_HP))) != cudaSuccess)
             return e;
     }
     if constexpr (D == 3 && sizeof(R) == 8) {              // FP64 has its own level kernels
@@ -575,9 +575,9 @@ cudaError_t launch_rbgs(int D, int prec, const InstDesc* insts, const InstState*
     if (D == 3 && prec == 0) return launch_rbgs64(insts, st, items, nitems, work, color, mode, s);
     // 3D plain half-sweeps of levels 127 .. 511: the plane-marching form
     const int hp = (nmax + 2 + 15) / 16 * 8;
-    if (D == 3 && mode == 0 && nmax >= 127 && hp <= Rb3p<float>::MAX_HP) {
-        const int ty = Rb3p<float>::TY;
-        const size_t sm = Rb3p<float>::bytes(hp);
+    if (D == 3 && mode == 0 && nmax >= 127 && hp <= Rb3p::MAX_HP) {
+        const int ty = Rb3p::TY;
+        const size_t sm = Rb3p::bytes(hp);
         const int per_sm = (int)(227 * 1024 / (sm + 1024));
         const int nyb = (nmax + ty - 1) / ty;
         // z chunks so that the launch is about one wave of resident CTAs
@@ -586,7 +586,7 @@ cudaError_t launch_rbgs(int D, int prec, const InstDesc* insts, const InstState*
         const int zchunk = (nmax + nzc - 1) / nzc;
         nzc = (nmax + zchunk - 1) / zchunk;
         dim3 g(nyb * nzc, nitems);
-        launch_k(k_rbgs3p<float>, g, dim3(32 * ty), sm, s, insts, st, items, color, zchunk);
+        launch_k(k_rbgs3p, g, dim3(32 * ty), sm, s, insts, st, items, color, zchunk);
         return cudaGetLastError();
     }
     dim3 g = mg_grid(work, nitems);
@@ -603,16 +603,16 @@ cudaError_t launch_restrict(int D, int prec, const InstDesc* insts, const InstSt
     // 3D complex64 restriction of the rhs alone (every iterate of the launch zero) from fine
     // levels 127 .. 511: the z-marching form
     const int pitch = (nmax + 2 + 15) / 16 * 16;
-    if (D == 3 && mode == 2 && nmax >= 127 && pitch <= Rs3p<float>::MAX_P) {
+    if (D == 3 && mode == 2 && nmax >= 127 && pitch <= Rs3p::MAX_P) {
         const int nc = (nmax - 1) / 2;
-        const size_t sm = Rs3p<float>::bytes(pitch);
+        const size_t sm = Rs3p::bytes(pitch);
         const int per_sm = (int)(227 * 1024 / (sm + 1024));
-        const int nyb = (nc + Rs3p<float>::TYC - 1) / Rs3p<float>::TYC;
+        const int nyb = (nc + Rs3p::TYC - 1) / Rs3p::TYC;
         int nzc = (152 * (per_sm < 1 ? 1 : per_sm)) / (nyb * nitems);
         nzc = nzc < 1 ? 1 : (nzc > nc / 4 ? nc / 4 : nzc);      // at least 4 coarse planes a CTA
         const int zchunk = (nc + nzc - 1) / nzc;
         nzc = (nc + zchunk - 1) / zchunk;
-        launch_k(k_restrict3p<float>, dim3(nyb * nzc, nitems), dim3(Rs3p<float>::NT), sm, s, insts, st, items,
+        launch_k(k_restrict3p, dim3(nyb * nzc, nitems), dim3(Rs3p::NT), sm, s, insts, st, items,
                  zchunk);
         return cudaGetLastError();
     }
