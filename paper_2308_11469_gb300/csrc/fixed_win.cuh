@@ -10,8 +10,9 @@
 // average to every node: a constant that the coarse levels amplify by N^2 / 14, 1.4e-14 of a
 // 1023^2 cycle's result for a rough right-hand side).  One unit is 2^-58 (2^-56 in the descent, whose residuals need headroom)
 // of the window's largest value, where FP64 rounds every partial sum at 2^-53 of its own size:
-// the cycle's error is no larger (measured against 64-bit cycles in
-// tests/test_gpu_fixed_win.py).  Values return to FP64 rounded to nearest, ties to even.
+// the cycle's error is no larger, as a part of the window's largest value (measured against
+// 64-bit cycles in tests/test_gpu_fixed_win.py; values below 2^-5 of it, 2^-3 in the descent, keep
+// fewer than FP64's 53 bits).  Values return to FP64 rounded to nearest, ties to even.
 //
 // 1023^2 FP64 solve, V(0,1), 17 steps: 3.77 -> 2.78 ms; 63^2, V(2,2): 1294 -> 1137 us.
 //

@@ -24,7 +24,7 @@
 //
 // Iterates, residuals and histories are those of the launch-by-launch path bit for bit.
 // 63^2 plane-wave cavity, V(2,2), 12 steps: 317 us a solve against 501 us (a step 18 us, its
-// V-cycle 11.5); 270 with one round trip to the host a solve.
+// V-cycle 11.5); 275 with one round trip to the host a solve.
 #include <atomic>
 
 #include <cooperative_groups.h>
