@@ -337,7 +337,7 @@ struct Engine {
             setup_small2d();
         }
         HELM_CK(setup_generic(D, prec == HELM_PREC_FP64 ? 0 : 1));
-        HELM_CK(setup_outer());
+        HELM_CK(setup_outer(D, prec == HELM_PREC_FP64 ? 0 : 1));
         return grow(4);
     }
 

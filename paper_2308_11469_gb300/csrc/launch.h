@@ -120,7 +120,7 @@ cudaError_t launch_small2d(const InstDesc* insts, InstState* st, const MgItem* i
                            int nu1, int nu2, int cycles, int damp, int* ctrl, cudaStream_t s);
 // shared-memory carve-out preferences of the generic and outer kernels
 cudaError_t setup_generic(int D, int prec);
-cudaError_t setup_outer();
+cudaError_t setup_outer(int D, int prec);
 
 // ---- fused 2D multigrid (vcycle2d.cu): two launches per level ----
 // descent: nu1 sweeps + residual + restriction; e (or zero) -> e2, coarse rhs.

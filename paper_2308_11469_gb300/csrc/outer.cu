@@ -1446,27 +1446,39 @@ cudaError_t setup_upres()
     return e != cudaSuccess ? e : setup_upres_v<NU, true>();
 }
 
-cudaError_t setup_outer()
+template <typename R>
+static cudaError_t setup_residual(int D)
 {
     cudaError_t e;
 #define HELM_CO(...) if ((e = max_carveout(__VA_ARGS__)) != cudaSuccess) return e;
-#define HELM_CO4(R, DD)                          \
-    HELM_CO(k_residual2d<R, 0, DD>)              \
-    HELM_CO(k_residual2d<R, 1, DD>)              \
-    HELM_CO(k_residual3d<R, 0, DD, false>)       \
-    HELM_CO(k_residual3d<R, 1, DD, false>)       \
-    HELM_CO(k_residual3d<R, 1, DD, true>)
-    HELM_CO4(float, false)
-    HELM_CO4(float, true)
-    HELM_CO4(double, false)
-    HELM_CO4(double, true)
-#undef HELM_CO4
+    if (D == 2) {
+        HELM_CO(k_residual2d<R, 0, false>)
+        HELM_CO(k_residual2d<R, 0, true>)
+        HELM_CO(k_residual2d<R, 1, false>)
+        HELM_CO(k_residual2d<R, 1, true>)
+        return cudaSuccess;
+    }
+    HELM_CO(k_residual3d<R, 0, false, false>)
+    HELM_CO(k_residual3d<R, 0, true, false>)
+    HELM_CO(k_residual3d<R, 1, false, false>)
+    HELM_CO(k_residual3d<R, 1, true, false>)
+    HELM_CO(k_residual3d<R, 1, false, true>)
+    HELM_CO(k_residual3d<R, 1, true, true>)
 #undef HELM_CO
-    if ((e = setup_upres<0>()) != cudaSuccess) return e;
-    if ((e = setup_upres<1>()) != cudaSuccess) return e;
-    if ((e = setup_upres<2>()) != cudaSuccess) return e;
-    if ((e = setup_upres<3>()) != cudaSuccess) return e;
-    if ((e = setup_upres<4>()) != cudaSuccess) return e;
+    return cudaSuccess;
+}
+
+cudaError_t setup_outer(int D, int prec)
+{
+    cudaError_t e = prec == 0 ? setup_residual<double>(D) : setup_residual<float>(D);
+    if (e != cudaSuccess) return e;
+    if (D == 2 && prec != 0) {
+        if ((e = setup_upres<0>()) != cudaSuccess) return e;
+        if ((e = setup_upres<1>()) != cudaSuccess) return e;
+        if ((e = setup_upres<2>()) != cudaSuccess) return e;
+        if ((e = setup_upres<3>()) != cudaSuccess) return e;
+        if ((e = setup_upres<4>()) != cudaSuccess) return e;
+    }
     return max_carveout(k_check);
 }
 
